@@ -309,7 +309,7 @@ static bool oz_wanted(const Level& L) {
 
 static size_t oz_bytes(long long nblk, int nparts, int nseps, int m) {
   const size_t mm = (size_t)m * m, sl = (size_t)oz_slice_blocks_bytes(m), nb = nblk / mm, np = std::max(1, nparts);
-  return (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + np * mm * sizeof(double) +
+  return (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + 2 * np * mm * sizeof(double) +
          np * ((size_t)2 * 9 * m * 32 * 2 + 3 * m * sizeof(int));
 }
 
@@ -450,6 +450,7 @@ int Level::allocate() {
     Z.on = true;
     if (gj_wanted(*this)) {
       const size_t pb = (size_t)9 * m * 32 * 2;
+      DM_ALLOC(Z.W, np * mm * sizeof(double));
       DM_ALLOC(Z.U, np * pb);
       DM_ALLOC(Z.V, np * pb);
       DM_ALLOC(Z.eU, np * ex);
@@ -691,6 +692,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
   out.ZL = static_cast<double*>(L.ZL);
   out.ZR = static_cast<double*>(L.ZR);
   out.Y = Z.Y;
+  out.W = Z.W;
   out.band = Z.band;
   // banded A and C as the previous factorisation found them (profiling costs
   // only: the kernels read the flag this factorisation's slicing sets)
@@ -738,7 +740,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
       Cost cb, cf;
       cb.bytes = np * 16.0 * m * m;           // B_0 read, written to G
       cf.bytes = np * (16.0 + 18.0) * m * m;  // G_t read and written, nine bf16 slices written
-      if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, G, st));
+      if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, Z.W, st));
       for (int k0 = 0; k0 < m; k0 += 32) {
         const double kw = std::min(32, m - k0);
         Cost cp, cu;
@@ -747,12 +749,12 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
         cu.flops = np * 2.0 * m * (m - kw) * kw;
         cu.bytes = np * (16.0 * m * (m - kw) + 18.0 * 32.0 * 2 * m);
         DM_LAUNCH(pf, st, K_INV_PANEL, cp, np,
-                  launch_gj_panel(L.d_parts, np, t, m, k0 / 32, G, Z.piv, Z.U, Z.eU, Z.V, Z.eV, L.status, st));
+                  launch_gj_panel(L.d_parts, np, t, m, k0 / 32, Z.W, Z.piv, Z.U, Z.eU, Z.V, Z.eV, L.status, st));
         if (m > 32)
           DM_LAUNCH(pf, st, K_INV_UPDATE, cu, np,
-                    launch_gj_update(L.d_parts, np, t, m, k0 / 32, G, Z.eU, Z.eV, Z.gj_maps, L.d_err, st));
+                    launch_gj_update(L.d_parts, np, t, m, k0 / 32, Z.W, Z.piv, Z.eU, Z.eV, Z.gj_maps, L.d_err, st));
       }
-      DM_LAUNCH(pf, st, K_INV, cf, np, launch_gj_finish(L.d_parts, np, t, m, G, Z.piv, Z.G, Z.eG, st));
+      DM_LAUNCH(pf, st, K_INV, cf, np, launch_gj_finish(L.d_parts, np, t, m, Z.W, G, Z.piv, Z.G, Z.eG, st));
     } else {
       DM_LAUNCH(pf, st, K_INV, L.c_inv[t], np, launch_inv<double>(L.d_parts, np, t, L.B, G, L.status, L.max_m, st));
       OzSliceJobs jg;
@@ -781,7 +783,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
               launch_oz_step(1, L.d_parts, nbk, t, m, out, lexp[1], r0exp[1], r1exp[1], maps[1], L.d_err, st));
     if (Z.band)  // both products of launch B when A is banded
       DM_LAUNCH(pf, st, K_BANDED, band_cost(nbk, 2), nbk,
-                launch_band_b(L.d_parts, nbk, t, m, L.A, L.B, out.Acal, out.ZL, G, Z.Y, Z.band, st));
+                launch_band_b(L.d_parts, nbk, t, m, L.A, L.B, out.Acal, out.ZL, G, Z.W, Z.Y, Z.band, st));
     OzSliceJobs jy;
     jy.job[0] = job(Z.Y, Z.YT, Z.eYT, 5);
     Cost c2 = cs;

@@ -1,0 +1,605 @@
+// Float64 block inverse G_t = D_t^{-1} of the digit-sliced levels: blocked
+// Gauss-Jordan with partial pivoting (the paper's inversion, Section 4;
+// Gauss-Jordan as in the library's other inverses), panels of 32 columns, the
+// rank-32 trailing updates as digit-sliced tensor-core products (dm_oz.cu,
+// k_oz_step<3>).
+//
+// The pivoting is implicit: rows stay where they are, and the pivot of column
+// k is the row p_k of largest magnitude in column k among the rows that were
+// no pivot before.  For a panel K = [k0, k0 + 32) with pivot rows p_K:
+//   1. k_gj_panel: in-place Gauss-Jordan restricted to the panel's columns
+//      (row p_k scaled by 1/M[p_k][k] with 1/M[p_k][k] in column k, every
+//      other row i minus M[i][k] times row p_k with -M[i][k]/M[p_k][k] in
+//      column k); the panel then holds U = [W in the rows p_K; -M_RK W
+//      elsewhere] (W = M[p_K, K]^{-1}).  It also writes U's row slices and the
+//      column slices of V = M[p_K, J], J the columns outside K.
+//   2. k_oz_step<3>: M[:, J] = (M[:, J], rows p_K zeroed) + U V.
+// After the last panel the working matrix W satisfies D^{-1}[k][p_j] =
+// W[p_k][j]; k_gj_finish moves the entries there and writes the row slices of
+// the inverse.  The working matrix is a buffer per subsystem (rolling), so it
+// stays in L2 from step to step.
+#include <cuda.h>
+#include <cuda_runtime.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cstdint>
+#include <cstring>
+
+#include "dm_internal.cuh"
+#include "dm_slices.cuh"
+
+namespace dm {
+namespace gj {
+
+constexpr int S = kRsSlices;
+constexpr int PW = 32;                 // panel width
+constexpr int SW = 8;                  // subpanel width
+constexpr int PS = PW + 1;             // row stride of the panel in shared memory (float64)
+constexpr int kMaxChain = 8;           // most warps that run the pivot chain
+constexpr int kHelpers = 8;            // more warps for the rank-8 updates, beside the chain's
+
+__global__ void __launch_bounds__(256) k_gj_copy_b0(const PartDesc* __restrict__ parts, int m,
+                                                    const double* __restrict__ B, double* __restrict__ W) {
+  const PartDesc p = parts[blockIdx.x];
+  const long long mm = (long long)m * m;
+  double* w = W + (long long)blockIdx.x * mm;
+  const double* b = B + p.blk;
+  for (long long e = threadIdx.x + (long long)blockIdx.y * blockDim.x; e < mm; e += (long long)blockDim.x * gridDim.y)
+    w[e] = b[e];
+}
+
+// zero, below 2^-1022 (whose reciprocal overflows), at or above 2^1022
+// (whose reciprocal is not a normal number) or not finite
+__device__ __forceinline__ bool gj_unusable(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return b < 0x0010000000000000ull || b >= 0x7fd0000000000000ull;
+}
+
+// 1/x for a usable pivot x (2^-1022 <= |x| < 2^1022) in integer arithmetic,
+// within 0.52 units in the last place.  x = X 2^(E - 52), X its 53-bit
+// significand; Y 2^-24 = y0 ~ 2^52 / X from the float32 reciprocal of X's
+// leading bits, relative error |h| < 2^-21.  The residual h = 1 - X y0 2^-52 =
+// H 2^-76 is exact in the low 64 bits of X Y, and 1/X = y0 2^-52 (1 + h + h^2)
+// up to h^3 (a Householder step of third order).  No float64 instruction: a
+// third of the pivot chain would be the three a float64 refinement takes.
+__device__ __forceinline__ double gj_recip(double x) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(bits >> 52) & 0x7ff;
+  const uint32_t xh = ((uint32_t)(bits >> 32) & 0xfffffu) | 0x100000u, xl = (uint32_t)bits;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f800000u | (xh << 12 >> 9) | (xl >> 29))));
+  const uint32_t rb = __float_as_uint(r);
+  const uint32_t Y = ((rb & 0x7fffffu) | 0x800000u) << ((rb >> 23) - 126u & 1u);  // r in [1/2, 1]
+  const unsigned long long XY = (unsigned long long)xl * Y + ((unsigned long long)(xh * Y) << 32);
+  const long long H = (long long)(0ull - XY);  // 2^76 - X Y, |H| < 2^55
+  const int Hh = (int)(H >> 24);
+  const long long c = H + (((long long)Hh * Hh) >> 28);  // (h + h^2) 2^76
+  const long long ch = c >> 16;                          // |ch| < 2^40
+  const long long cy = (long long)(int)(ch >> 24) * (int)Y * (1ll << 24) + (long long)((uint32_t)ch & 0xffffffu) * Y;
+  const unsigned long long y = ((unsigned long long)Y << 36) + (unsigned long long)(cy >> 24);  // 2^60 / (X 2^-52)
+  const unsigned long long mant = (y + 64) >> 7;  // leading bit at 52, or 2^53
+  return __longlong_as_double((long long)((bits & 0x8000000000000000ull) +
+                                          ((unsigned long long)(2044 - ex) << 52) + mant));
+}
+
+__device__ __forceinline__ uint32_t abs_hi(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
+
+// What the chain's warps exchange per pivot (double-buffered by its parity).
+struct __align__(16) GjCand {  // a warp's best row for the next pivot
+  double v;       // its element of the pivot column
+  uint32_t key;   // 0: no eligible row; else the high word of |v| + 1
+  int idx;        // the row
+};
+struct __align__(16) GjPivot {  // the pivot
+  double inv;  // its reciprocal (0 when unusable)
+  int idx;     // its row
+  int warp;    // the warp that holds it
+};
+struct GjShared {
+  GjCand cand[2][kMaxChain];
+  GjPivot piv[2];
+  double row[2][kMaxChain][SW];  // every candidate row after the pending pivot's update
+};
+
+// The pivot chain of one subpanel (columns c0 .. c0 + w - 1 of the panel), run
+// by warps 0 .. nw - 1: lane `lane` of warp `warp` holds rows 32 warp + lane +
+// 32 CW i, i < RPL, eight columns each, in registers.
+//
+// A float64 instruction holds its warp for 64 cycles on GB300 (measured; one
+// warp per SM sub-partition, dependent or not), and other instructions of the
+// same warp do not overlap it.  So the chain's warps do the multiply-adds (9
+// RPL float64 instructions per pivot) and the search among their own rows, and a control warp
+// picks the pivot among the warps' candidates and takes its reciprocal in
+// integer arithmetic while they run.  Per pivot: every row updates its next
+// pivot column first and the warps publish their best candidates (largest
+// high word of |value|: candidates that agree to 2^-20 count as equal, the
+// first one is taken); then they update the other seven columns and publish
+// the candidate rows; after one barrier with the control warp every row takes
+// its multiplier.  The pivot's own row takes part as zeros plus the
+// reciprocal times itself, so that no result is selected after a
+// multiply-add.
+//
+// The registers rotate by one column per pivot (register c of `a` holds
+// column (j - 1 + c) mod 8 before pivot j, of `b` column (j + c) mod 8 after
+// it), from one set to the other: rotated in place, every multiply-add would
+// wait until the one before has read its operands.
+template <int RPL>
+struct GjRows {
+  double a[RPL][SW], fn[RPL];  // fn: minus the multiplier of the pending pivot
+  bool dead[RPL];              // past the block's end, or a pivot row already
+};
+
+template <int CW, int RPL>
+__device__ __forceinline__ void gj_pivot(const GjRows<RPL>& in, GjRows<RPL>& out, double (&s)[SW], int buf, int nw,
+                                         GjShared& sh, int warp, int lane) {
+  uint32_t key = 0;
+  double bnv = 0.0;
+  int bi = 0;
+#pragma unroll
+  for (int i = 0; i < RPL; ++i) out.a[i][0] = fma(in.fn[i], s[1], in.a[i][1]);
+#pragma unroll
+  for (int i = 0; i < RPL; ++i) {
+    const uint32_t ki = in.dead[i] ? 0u : abs_hi(out.a[i][0]) + 1u;
+    if (i == 0 || ki > key) key = ki, bnv = out.a[i][0], bi = i;
+  }
+  const uint32_t wkey = __reduce_max_sync(0xffffffffu, key);
+  const int src = (int)__reduce_min_sync(0xffffffffu, key == wkey ? (uint32_t)lane : 32u);
+  if (lane == src) {
+    GjCand& cd = sh.cand[buf][warp];
+    cd.v = bnv;
+    cd.key = wkey;
+    cd.idx = 32 * warp + lane + 128 * bi;
+  }
+  asm volatile("bar.arrive 1, %0;" ::"r"(32 * nw + 32) : "memory");
+  // src < 32: adds nothing, but keeps the multiply-adds below after the search
+  const int z = src & 64;
+#pragma unroll
+  for (int i = 0; i < RPL; ++i) {
+    const double f = __hiloint2double(__double2hiint(in.fn[i]) + z, __double2loint(in.fn[i]));
+#pragma unroll
+    for (int c = 2; c < SW; ++c) out.a[i][c - 1] = fma(f, s[c], in.a[i][c]);
+    out.a[i][SW - 1] = fma(f, s[0], in.a[i][0]);
+  }
+  if (lane == src) {
+#pragma unroll
+    for (int i = 0; i < RPL; ++i)
+      if (bi == i) {
+#pragma unroll
+        for (int c = 0; c < SW; c += 2)
+          *reinterpret_cast<double2*>(&sh.row[buf][warp][c]) = make_double2(out.a[i][c], out.a[i][c + 1]);
+      }
+  }
+  asm volatile("bar.sync 2, %0;" ::"r"(32 * nw + 32) : "memory");
+  const GjPivot pv = sh.piv[buf];
+  const double* u = sh.row[buf][pv.warp];
+#pragma unroll
+  for (int c = 0; c < SW; c += 2) {
+    const double2 u2 = *reinterpret_cast<const double2*>(u + c);
+    s[c] = u2.x;
+    s[c + 1] = u2.y;
+  }
+  s[0] = 1.0;
+#pragma unroll
+  for (int i = 0; i < RPL; ++i) {
+    out.fn[i] = -out.a[i][0] * pv.inv;
+    out.a[i][0] = 0.0;
+    out.dead[i] = in.dead[i];
+    if (32 * warp + lane + 32 * CW * i == pv.idx) {
+      out.dead[i] = true;
+      out.fn[i] = pv.inv;
+#pragma unroll
+      for (int c = 1; c < SW; ++c) out.a[i][c] = 0.0;
+    }
+  }
+}
+
+template <int CW, int RPL>
+__device__ __forceinline__ void gj_chain(double* P, int m, int c0, int w, int nw, const uint32_t* used, GjShared& sh,
+                                         int warp, int lane) {
+  GjRows<RPL> x, y;
+#pragma unroll
+  for (int i = 0; i < RPL; ++i) {
+    const int row = 32 * warp + lane + 32 * CW * i;
+    x.dead[i] = row >= m || ((used[row >> 5] >> (row & 31)) & 1u) != 0;
+    x.fn[i] = 0.0;
+#pragma unroll
+    for (int c = 0; c < SW; ++c) x.a[i][c] = row < m ? P[row * PS + c0 + ((c + 7) & 7)] : 0.0;
+  }
+  double s[SW];  // the pending pivot's row (1 in its own column)
+#pragma unroll
+  for (int c = 0; c < SW; ++c) s[c] = 0.0;
+#pragma unroll 1
+  for (int j = 0; j < w; j += 2) {
+    gj_pivot<CW, RPL>(x, y, s, 0, nw, sh, warp, lane);
+    if (j + 1 < w)
+      gj_pivot<CW, RPL>(y, x, s, 1, nw, sh, warp, lane);
+    else
+      x = y;
+  }
+  // the last pivot's update
+#pragma unroll
+  for (int i = 0; i < RPL; ++i) {
+    const int row = 32 * warp + lane + 32 * CW * i;
+#pragma unroll
+    for (int c = 0; c < SW; ++c) y.a[i][c] = fma(x.fn[i], s[c], x.a[i][c]);
+    if (row < m)
+#pragma unroll
+      for (int c = 0; c < SW; ++c) P[row * PS + c0 + ((w - 1 + c) & 7)] = y.a[i][c];
+  }
+}
+
+// The control warp's side of gj_chain.
+__device__ __forceinline__ void gj_control(int c0, int w, int nw, GjShared& sh, int* piv_s, int lane, bool& bad) {
+#pragma unroll 1
+  for (int j = 0; j < w; ++j) {
+    asm volatile("bar.sync 1, %0;" ::"r"(32 * nw + 32) : "memory");
+    const GjCand c = sh.cand[j & 1][min(lane, nw - 1)];
+    const uint32_t kmax = __reduce_max_sync(0xffffffffu, c.key);
+    const int best = (int)__reduce_min_sync(0xffffffffu, c.key == kmax ? (uint32_t)lane : 32u);
+    const double inv = gj_unusable(c.v) ? 0.0 : gj_recip(c.v);
+    if (lane == best) {
+      sh.piv[j & 1] = GjPivot{inv, c.idx, best};
+      piv_s[c0 + j] = c.idx;
+      if (__double_as_longlong(inv) == 0) bad = true;
+    }
+    asm volatile("bar.sync 2, %0;" ::"r"(32 * nw + 32) : "memory");
+  }
+}
+
+__device__ __forceinline__ void mma_k16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(b0));
+}
+
+// T 2^s rounded to float64 (to nearest, halves up), |T| < 2^63, by integer
+// operations; `odd` is set when the result is outside the normal range (then
+// the value is not the result).
+__device__ __forceinline__ double round_scaled(long long T, int s, bool& odd) {
+  const unsigned long long a = (unsigned long long)(T < 0 ? -T : T);
+  const int lz = __clzll(a);
+  const unsigned long long an = a << (lz & 63);                   // leading bit at 63
+  const unsigned long long mant = (an >> 11) + ((an >> 10) & 1);  // leading bit at 52 (or 2^53)
+  const int ex = 1022 + 63 - lz + s;                              // the leading bit adds one to the exponent
+  odd = odd || (a != 0 && (unsigned)ex > 2044u);
+  const unsigned long long r = ((unsigned long long)T & 0x8000000000000000ull) + ((unsigned long long)ex << 52) + mant;
+  return __longlong_as_double(a == 0 ? 0ll : (long long)r);
+}
+
+constexpr int kNotFinite = 1 << 14;  // scale of a row or column with a NaN or an infinity
+
+__device__ __forceinline__ int bal_exponent(uint32_t hmax) {
+  return hmax >= 0x7ff00000u ? kNotFinite : scale_exponent(hmax);
+}
+
+// Rank-8 update of nq of the panel's 8-column groups (from column n0 on, wrapping) after
+// a subpanel's pivots: P[i][c] = (i a pivot row of the subpanel ? 0 : P[i][c])
+// + sum_j U[i][j] V[j][c], U the subpanel's columns, V its pivot rows before
+// the update; warp wi of nwk takes every nwk-th 16 x 8 tile.
+// In float64 instructions it would cost twice the pivot chain itself, so it
+// runs on the tensor cores: seven balanced base-256 digits per operand (row
+// scales for U, column scales for V), the 28 digit products with s + t <= 8
+// in 16 mma.sync per 16 x 8 tile (two digit pairs share a K = 16
+// instruction), sums below 8 * 7 * 2^14 < 2^22, exact; one integer rounding
+// and one float64 add per entry.  (tcgen05 has no use here: K = 8 and the
+// operands are in registers.)
+__device__ __noinline__ void gj_rank8(double* P, const double (*V)[PW], int mt, int c0, int n0, int nq,
+                                      const int* sub_piv, int w, int wi, int nwk) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, tg = lane & 3;
+  uint32_t b[kBalSlices];
+  int fe[2], qb = -1, nc = 0;
+#pragma unroll 1
+  for (int i = wi; i < mt * nq; i += nwk) {
+    const int q = i / mt, rt = i - q * mt;
+    if (q != qb) {  // the group's digits of V
+      qb = q;
+      nc = (n0 + SW * q) & (PW - 1);
+      const double v0 = V[2 * tg][nc + g], v1 = V[2 * tg + 1][nc + g];
+      uint32_t h = max(abs_hi(v0), abs_hi(v1));
+      h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
+      h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
+      const int e = bal_exponent(h);
+      uint32_t d0[kBalSlices], d1[kBalSlices];
+      digits7((unsigned long long)__double_as_longlong(v0), e, d0);
+      digits7((unsigned long long)__double_as_longlong(v1), e, d1);
+#pragma unroll
+      for (int k = 0; k < kBalSlices; ++k) b[k] = pack_hi(d0[k], d1[k]);
+      fe[0] = __shfl_sync(0xffffffffu, e, 8 * tg);
+      fe[1] = __shfl_sync(0xffffffffu, e, 8 * tg + 4);
+    }
+    {
+      uint32_t a[2][kBalSlices];
+      int re[2];
+      bool z[2];
+#pragma unroll
+      for (int h2 = 0; h2 < 2; ++h2) {
+        const int row = 16 * rt + 8 * h2 + g;
+        const double v0 = P[row * PS + c0 + 2 * tg], v1 = P[row * PS + c0 + 2 * tg + 1];
+        uint32_t h = max(abs_hi(v0), abs_hi(v1));
+        h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
+        h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
+        re[h2] = bal_exponent(h);
+        uint32_t d0[kBalSlices], d1[kBalSlices];
+        digits7((unsigned long long)__double_as_longlong(v0), re[h2], d0);
+        digits7((unsigned long long)__double_as_longlong(v1), re[h2], d1);
+#pragma unroll
+        for (int k = 0; k < kBalSlices; ++k) a[h2][k] = pack_hi(d0[k], d1[k]);
+        z[h2] = false;
+#pragma unroll
+        for (int j = 0; j < SW; ++j) z[h2] = z[h2] || (j < w && sub_piv[j] == row);
+      }
+      int A[kBalSlices][4];  // acc_d, d = 2 .. 8
+#pragma unroll
+      for (int d = 2; d <= 8; ++d) {
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        int s = 1;
+#pragma unroll
+        for (; s + 1 <= d - 1; s += 2)
+          mma_k16(c, a[0][s - 1], a[1][s - 1], a[0][s], a[1][s], b[d - s - 1], b[d - s - 2]);
+        if (s <= d - 1) mma_k8(c, a[0][s - 1], a[1][s - 1], b[d - s - 1]);
+#pragma unroll
+        for (int o = 0; o < 4; ++o) A[d - 2][o] = __float_as_int(c[o] + 12582912.0f) - 0x4B400000;
+      }
+      double v[4];
+      bool odd = re[0] == kNotFinite || re[1] == kNotFinite || fe[0] == kNotFinite || fe[1] == kNotFinite;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        // units 2^(e_r + f_c + 2 - 60): the last accumulator's low four bits are dropped
+        const long long T = (long long)(A[0][o] * 256 + A[1][o]) * (1ll << 36) +
+                            (long long)(A[2][o] * 256 + A[3][o]) * (1ll << 20) +
+                            (long long)(A[4][o] * 256 + A[5][o]) * 16 + (A[6][o] >> 4);
+        v[o] = round_scaled(T, re[o >> 1] + fe[o & 1] - 58, odd);
+      }
+      if (odd) {  // results outside the normal range, NaN and infinite operands
+#pragma unroll 1
+        for (int o = 0; o < 4; ++o) {
+          int t[kBalSlices];
+#pragma unroll
+          for (int k = 0; k < kBalSlices; ++k) t[k] = o == 0 ? A[k][0] : o == 1 ? A[k][1] : o == 2 ? A[k][2] : A[k][3];
+          const long long T = (long long)(t[0] * 256 + t[1]) * (1ll << 36) + (long long)(t[2] * 256 + t[3]) * (1ll << 20) +
+                              (long long)(t[4] * 256 + t[5]) * 16 + (t[6] >> 4);
+          const int er = o < 2 ? re[0] : re[1], ec = (o & 1) ? fe[1] : fe[0];
+          const double x = er == kNotFinite || ec == kNotFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                : ldexp((double)T, er + ec - 58);
+          if (o == 0) v[0] = x;
+          if (o == 1) v[1] = x;
+          if (o == 2) v[2] = x;
+          if (o == 3) v[3] = x;
+        }
+      }
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        double* d = P + (16 * rt + 8 * (o >> 1) + g) * PS + nc + 2 * tg + (o & 1);
+        *d = (z[o >> 1] ? 0.0 : *d) + v[o];
+      }
+    }
+  }
+}
+
+// Eight values' digits to a slice array: slice sl at dst + sl * stride.
+__device__ __noinline__ void gj_slice8(double v0, double v1, double v2, double v3, double v4, double v5, double v6, double v7,
+                                       int e, __nv_bfloat16* dst, int stride) {
+  const double v[8] = {v0, v1, v2, v3, v4, v5, v6, v7};
+  uint32_t d[8][S];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) digits9((unsigned long long)__double_as_longlong(v[c]), e, d[c]);
+#pragma unroll
+  for (int sl = 0; sl < S; ++sl)
+    *reinterpret_cast<uint4*>(dst + (long long)sl * stride) =
+        make_uint4(pack_hi(d[0][sl], d[1][sl]), pack_hi(d[2][sl], d[3][sl]), pack_hi(d[4][sl], d[5][sl]),
+                   pack_hi(d[6][sl], d[7][sl]));
+}
+
+// One panel of every active subsystem's working matrix, a CTA per block: up to
+// eight chain warps (a row per lane; two rows above m = 256), the control
+// warp, and eight helpers.  Bound by the chain's float64 instructions and
+// barriers: about 1150 cycles per pivot to m = 128 (one warp per SM
+// sub-partition) and 1700 at m = 256 (two).  A cluster of CTAs with the rows
+// split and a cluster barrier per pivot took 83 / 90 / 98 us per panel at m =
+// 64 / 128 / 256, this one 40 / 47 / 76 us (34, 97, 64 blocks).  The loops
+// stay rolled: the code runs once per launch, and unrolled it waited for its
+// instructions.
+template <int CW, int RPL>
+__global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
+    k_gj_panel(const PartDesc* __restrict__ parts, int t, int m, int panel, double* __restrict__ W,
+               int* __restrict__ piv, __nv_bfloat16* __restrict__ Us, int* __restrict__ Uexp,
+               __nv_bfloat16* __restrict__ Vs, int* __restrict__ Vexp, int* __restrict__ status) {
+  extern __shared__ __align__(16) double P[];  // [16 ceil(m / 16)][PS]
+  __shared__ GjShared sh;
+  constexpr int kWorkers = CW + kHelpers, kWarps = kWorkers + 1, kThreads = 32 * kWarps;  // the last: control
+  __shared__ double V[SW][PW];
+  __shared__ int piv_s[PW];
+  __shared__ uint32_t used[kMaxM / 32];
+  const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const PartDesc p = parts[q];
+  if (t >= p.L) return;
+  double* M = W + (long long)q * m * m;
+  const int k0 = PW * panel, kw = min(PW, m - k0), mt = (m + 15) / 16;
+  const int nw = min(CW, (m + 31) / 32);
+  if (tid < kMaxM / 32) used[tid] = 0;
+  __syncthreads();
+  for (int k = tid; k < k0; k += kThreads) {
+    const int r = piv[(long long)q * m + k];
+    atomicOr(&used[r >> 5], 1u << (r & 31));
+  }
+#pragma unroll 8
+  for (int i = warp; i < 16 * mt; i += kWarps)
+    P[i * PS + lane] = (i < m && lane < kw) ? M[(long long)i * m + k0 + lane] : 0.0;
+  __syncthreads();
+  bool bad = false;
+  // Per subpanel: the pivots on warps 0-3 and the control warp while warps 4-7 finish the rank-8
+  // update of the subpanel before (its 16 columns that are not next); then
+  // all warps update the next subpanel's columns (after the last subpanel all
+  // other columns), which its chain waits for.
+#pragma unroll 1
+  for (int c0 = 0; c0 < kw; c0 += SW) {
+    const int w = min(SW, kw - c0);
+    if (warp < nw)
+      gj_chain<CW, RPL>(P, m, c0, w, nw, used, sh, warp, lane);
+    else if (warp == kWorkers)
+      gj_control(c0, w, nw, sh, piv_s, lane, bad);
+    else if (warp >= CW && c0 > 0)
+      gj_rank8(P, V, mt, c0 - SW, c0 + SW, 2, piv_s + c0 - SW, SW, warp - CW, kHelpers);
+    __syncthreads();
+    // this subpanel's pivot rows of the other columns
+    if (warp < SW) V[warp][lane] = warp < w ? P[piv_s[c0 + min(warp, w - 1)] * PS + lane] : 0.0;
+    if (tid < w) atomicOr(&used[piv_s[c0 + tid] >> 5], 1u << (piv_s[c0 + tid] & 31));
+    __syncthreads();
+    if (kw > SW && warp < kWorkers)
+      gj_rank8(P, V, mt, c0, c0 + SW, c0 + SW < kw ? 1 : 3, piv_s + c0, w, warp, kWorkers);
+    __syncthreads();
+  }
+  if (tid < kw) piv[(long long)q * m + k0 + tid] = piv_s[tid];
+  // the eliminated panel and the row slices of U (scale per row over its 32
+  // values): four threads per row, eight values each
+#pragma unroll 1
+  for (int i0 = 0; i0 < m; i0 += kThreads / 4) {
+    const int i = i0 + (tid >> 2), cb = (tid & 3) * 8;
+    double v[8];
+    uint32_t hmax = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      v[c] = i < m ? P[i * PS + cb + c] : 0.0;
+      hmax = max(hmax, abs_hi(v[c]));
+    }
+    hmax = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, 1));
+    hmax = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, 2));
+    if (i < m) {
+      const int e = scale_exponent(hmax);
+      if ((tid & 3) == 0) Uexp[(long long)q * m + i] = e;
+      gj_slice8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], e, Us + (long long)q * S * m * PW + (long long)i * PW + cb, m * PW);
+    }
+  }
+  for (int i = warp; i < m; i += kWarps)
+    if (lane < kw) M[(long long)i * m + k0 + lane] = P[i * PS + lane];
+  // the column slices of V = the pivot rows outside the panel (transposed: row
+  // j of the copy holds V[0..31][j]; the panel's own columns are never read)
+#pragma unroll 1
+  for (int j0 = 0; j0 < m; j0 += kThreads / 4) {
+    const int j = j0 + (tid >> 2), cb = (tid & 3) * 8;  // four threads per column, eight rows each
+    const bool in = j < m && (j < k0 || j >= k0 + kw);
+    double v[8];
+    uint32_t vmax = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = in && cb + c < kw ? M[(long long)piv_s[cb + c] * m + j] : 0.0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) vmax = max(vmax, abs_hi(v[c]));
+    vmax = max(vmax, __shfl_xor_sync(0xffffffffu, vmax, 1));
+    vmax = max(vmax, __shfl_xor_sync(0xffffffffu, vmax, 2));
+    if (in) {
+      const int e = scale_exponent(vmax);
+      if ((tid & 3) == 0) Vexp[(long long)q * m + j] = e;
+      gj_slice8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], e, Vs + (long long)q * S * m * PW + (long long)j * PW + cb, m * PW);
+    }
+  }
+  if (bad) atomicMin(status + p.sys, p.row0 + t + 1);
+}
+
+// After the last panel: D^{-1}[k][p_j] = W[p_k][j] moved to its place in G
+// and the row slices of the block inverse G_t written (the left operand of
+// the next products), one pass: a CTA takes 32 rows of one block (blockIdx.x
+// = block * groups + group), a warp a row at a time: the row is read once,
+// scattered to its final column order in shared memory (its largest magnitude
+// does not depend on the order), then written as float64 and as digit slices.
+__global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ parts, int t, int m,
+                                                   const double* __restrict__ W, double* __restrict__ G,
+                                                   const int* __restrict__ piv, __nv_bfloat16* __restrict__ Gs,
+                                                   int* __restrict__ eG) {
+  __shared__ int ip[kMaxMTensor];
+  __shared__ __align__(16) double rowb[8][kMaxMTensor];
+  const int groups = (m + 31) / 32;
+  const int q = blockIdx.x / groups, g = blockIdx.x - q * groups;
+  const PartDesc p = parts[q];
+  if (t >= p.L) return;
+  const long long mm = (long long)m * m;
+  const double* M = W + (long long)q * mm;
+  double* Gt = G + p.blk + (long long)t * mm;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int c = threadIdx.x; c < m; c += blockDim.x) ip[c] = piv[(long long)q * m + c];
+  __syncthreads();
+  double* rb = rowb[warp];
+  const int rend = min(m, 32 * g + 32);
+  for (int r = 32 * g + warp; r < rend; r += 8) {
+    uint32_t hmax = 0;
+    const double* src = M + (long long)ip[r] * m;
+    for (int c = lane; c < m; c += 32) {
+      const double v = src[c];
+      rb[ip[c]] = v;
+      hmax = max(hmax, abs_hi(v));
+    }
+    hmax = __reduce_max_sync(0xffffffffu, hmax);
+    const int e = scale_exponent(hmax);
+    if (lane == 0) eG[(long long)q * m + r] = e;
+    __syncwarp();
+    for (int c0 = lane * 8; c0 < m; c0 += 256) {  // m % 8 == 0
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        const double2 d2 = *reinterpret_cast<const double2*>(rb + c0 + u);
+        v[u] = d2.x;
+        v[u + 1] = d2.y;
+        *reinterpret_cast<double2*>(Gt + (long long)r * m + c0 + u) = d2;
+      }
+      uint32_t d[8][S];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) digits9((unsigned long long)__double_as_longlong(v[u]), e, d[u]);
+#pragma unroll
+      for (int sl = 0; sl < S; ++sl)
+        *reinterpret_cast<uint4*>(Gs + ((long long)q * S + sl) * mm + (long long)r * m + c0) =
+            make_uint4(pack_hi(d[0][sl], d[1][sl]), pack_hi(d[2][sl], d[3][sl]), pack_hi(d[4][sl], d[5][sl]),
+                       pack_hi(d[6][sl], d[7][sl]));
+    }
+    __syncwarp();
+  }
+}
+
+}  // namespace gj
+
+// The blocked Gauss-Jordan inversion of block row t of every active subsystem
+// (working matrix W: D_t, written by launch B of the step before), as phases:
+// the copy of B_0, per panel of 32 columns the panel and its trailing update
+// (dm_oz.cu), and the finishing pass.
+void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, cudaStream_t st) {
+  if (nparts > 0 && t == 0)
+    gj::k_gj_copy_b0<<<dim3(nparts, std::max(1, m * m / 8192)), 256, 0, st>>>(parts, m, B, W);
+}
+
+void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, int* piv, void* Us,
+                     int* Uexp, void* Vs, int* Vexp, int* status, cudaStream_t st) {
+  if (nparts <= 0) return;
+  const size_t smem = (size_t)16 * ((m + 15) / 16) * gj::PS * sizeof(double);
+#define DM_GJ(C_, R_)                                                                                                   \
+  do {                                                                                                              \
+    static bool set = false;                                                                                        \
+    if (!set) {                                                                                                     \
+      cudaFuncSetAttribute(gj::k_gj_panel<C_, R_>, cudaFuncAttributeMaxDynamicSharedMemorySize,                         \
+                           32 * C_ * R_ * gj::PS * (int)sizeof(double));                                                \
+      set = true;                                                                                                   \
+    }                                                                                                               \
+    gj::k_gj_panel<C_, R_><<<nparts, 32 * (C_ + gj::kHelpers + 1), smem, st>>>(                                     \
+        parts, t, m, pnl, W, piv, static_cast<__nv_bfloat16*>(Us), Uexp, static_cast<__nv_bfloat16*>(Vs), Vexp,     \
+        status);                                                                                                    \
+  } while (0)
+  if (m <= 128) DM_GJ(4, 1);
+  else if (m <= 256) DM_GJ(8, 1);
+  else DM_GJ(8, 2);
+#undef DM_GJ
+}
+
+void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
+                      void* Gs, int* eG, cudaStream_t st) {
+  if (nparts <= 0) return;
+  gj::k_gj_finish<<<nparts * ((m + 31) / 32), 256, 0, st>>>(parts, t, m, W, G, piv, static_cast<__nv_bfloat16*>(Gs),
+                                                             eG);
+}
+
+}  // namespace dm

@@ -6,6 +6,9 @@
 
 namespace dm {
 
+constexpr int kMaxM = 512;
+constexpr int kMaxR = 64;
+
 // Flags of a subsystem (partition) descriptor.
 enum : int {
   HAS_LEFT = 1,   // subsystem k > 0: spike for h^{k-1} (top block A of its first row)
@@ -145,6 +148,8 @@ bool tc2_eligible(int m);
 struct OzOut {
   const double* B;
   double *G, *Acal, *ZL, *ZR, *Y;  // Y: Y_{t+1} per subsystem (rolling, float64)
+  double* W;       // working matrix of the blocked inversion per subsystem (rolling): D_{t+1} goes there (null: to G)
+  const int* piv;  // the inversion's pivot rows [subsystem][m] (KIND 3)
   // the supplementary blocks (Eq. e2311), one separator per CTA row
   const SepDesc* seps;
   double *HA, *HB, *HC;
@@ -182,7 +187,8 @@ void launch_band_detect(const double* A, const double* C, long long n, int m, in
 void launch_band_gc(const PartDesc* parts, int nparts, int t, int m, const double* G, const double* C, double* Acal,
                     double* ZR, const int* band, cudaStream_t st);
 void launch_band_b(const PartDesc* parts, int nparts, int t, int m, const double* A, const double* B,
-                   const double* Acal, const double* ZL, double* G, double* Y, const int* band, cudaStream_t st);
+                   const double* Acal, const double* ZL, double* G, double* W, double* Y, const int* band,
+                   cudaStream_t st);
 void launch_band_h(const SepDesc* seps, int nseps, int m, const double* A, const double* B, const double* C,
                    const double* ZL, const double* ZR, double* HA, double* HB, double* HC, const int* band,
                    cudaStream_t st);
@@ -201,22 +207,20 @@ void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, co
 void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m, const OzOut& out, const int* lexp,
                     const int* rexp0, const int* rexp1, const void* maps3, int* errflag, cudaStream_t st,
                     int aux = 0);
-// Blocked Gauss-Jordan inversion with the rank-32 updates as digit-sliced
-// tensor-core products; maps2 = the panel-slice maps (U with 128-row boxes,
-// V with 48-row boxes), piv [nparts][m] (the column permutation), Us / Vs
-// [nparts][9][m][32] bf16, Uexp / Vexp [nparts][m]; Gs / eG receive the row
-// slices of the inverses ([nparts][9][m][m] bf16, [nparts][m]).
-void launch_gj_inverse(const PartDesc* parts, int nparts, int t, int m, const double* B, double* G, int* piv,
-                       void* Us, int* Uexp, void* Vs, int* Vexp, const void* maps2, int* status, int* errflag,
-                       void* Gs, int* eG, cudaStream_t st);
-// its phases (launch_gj_inverse runs them in order)
-void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* G, cudaStream_t st);
-void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* G, int* piv, void* Us,
+// Blocked Gauss-Jordan inversion (dm_gj.cu) in the working matrices W
+// [nparts][m][m], with the rank-32 updates as digit-sliced tensor-core
+// products; maps2 = the panel-slice maps (U with 128-row boxes, V with
+// oz_box_rows_gj() rows), piv [nparts][m] (the pivot row of every column), Us /
+// Vs [nparts][9][m][32] bf16, Uexp / Vexp [nparts][m].  Phases: begin (t = 0
+// only: W = B_0), per panel panel and update, finish (the inverse to G_t, its
+// row slices to Gs [nparts][9][m][m] bf16 / eG [nparts][m]).
+void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, cudaStream_t st);
+void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, int* piv, void* Us,
                      int* Uexp, void* Vs, int* Vexp, int* status, cudaStream_t st);
-void launch_gj_update(const PartDesc* parts, int nparts, int t, int m, int pnl, double* G, const int* Uexp,
-                      const int* Vexp, const void* maps2, int* errflag, cudaStream_t st);
-void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, double* G, const int* piv, void* Gs, int* eG,
-                      cudaStream_t st);
+void launch_gj_update(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, const int* piv,
+                      const int* Uexp, const int* Vexp, const void* maps2, int* errflag, cudaStream_t st);
+void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
+                      void* Gs, int* eG, cudaStream_t st);
 int tc2_ntile(int m);
 bool tc2_make_map(int mode, const void* base, long long blocks, int m, int box_rows, void* out);
 int tc2_map_bytes();
@@ -224,8 +228,5 @@ void launch_tc2_convert(int mode, const double* src64, const float* src32, const
                         bool trans, void* dst, long long cap_blocks, cudaStream_t st);
 void launch_tc2_step(int mode, int kind, const PartDesc* parts, int nparts, int step, int m, const int lo[3],
                      const Tc2Out& out, const void* maps3, int* errflag, cudaStream_t st);
-
-constexpr int kMaxM = 512;
-constexpr int kMaxR = 64;
 
 }  // namespace dm

@@ -32,7 +32,6 @@
 // epilogue combines the accumulators in 64-bit integers and scales once in
 // float64 (GB300's float64 pipe is narrow).  Operand slices of results are
 // made by separate slicing launches, which see whole rows and columns.
-#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -116,9 +115,10 @@ namespace oz {
 // `step`, over the subsystems.  Exponent arrays: [block][m] ints, indexed
 // like the slices.
 // KIND 3: the trailing update of panel `step` (columns K = [32 step, 32 step
-// + 32)) of the blocked Gauss-Jordan inversion of block row `aux`:
-// M[:, J] = (M[:, J] with the rows K zeroed) + U V, U the eliminated panel,
-// V = M[K, J] before the update (both as slices, K = 32), J the other columns.
+// + 32), pivot rows p_K = piv[K]) of the blocked Gauss-Jordan inversion of
+// block row `aux` in the working matrix: M[:, J] = (M[:, J] with the rows p_K
+// zeroed) + U V, U the eliminated panel, V = M[p_K, J] before the update
+// (both as slices, K = 32), J the other columns.
 // KIND 4, 5: the supplementary blocks of a separator (Eq. e2311), left A_q /
 // C_q: KIND 4 j = 0: HB = B_q - A_q ZR^j[q-1], j = 1: HA = -A_q ZL^j[q-1];
 // KIND 5 j = 0: HB -= C_q ZL^{j+1}[q+1], j = 1: HC = -C_q ZR^{j+1}[q+1]
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     double* stg = stage_out + ew * STG;
     const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
     const int cl = lane & 7, r0 = lane >> 3;
-    const int k0 = 32 * step;  // KIND 3: the panel's columns and pivot rows
+    const int k0 = 32 * step;  // KIND 3: the panel's columns
     int lt = 0;
     for (int tile = blockIdx.x; tile < ntiles && !*verr; tile += gridDim.x) {
       const OzTile w = oz_tile<KIND>(tile, parts, out, step, aux, m, ntm, ntn);
@@ -363,10 +363,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool rmw = KIND == 2 && j == 0, dnext = KIND == 1 && j == 0, gj = KIND == 3, hb = KIND >= 4 && j == 0;
       const bool upd = rmw || dnext || gj || hb;
       const long long o = p.blk + (long long)t * mm;
+      // the working matrix of the blocked inversion (or D_{t+1}'s place in G)
+      double* const wk = out.W ? out.W + (long long)pidx * mm : out.G + o + mm;
       const double* src = rmw    ? out.ZL + o
-                          : gj   ? out.G + o
+                          : gj   ? wk
                           : hb   ? (KIND == 4 ? out.B + sd.blk_q : out.HB + sd.hblk)
                                  : out.B + o + mm;
+      // KIND 3: which of the warp's 32 rows are pivot rows of the panel
+      uint32_t zrows = 0;
+      if (KIND == 3) {
+        const int pv = k0 + lane < m ? out.piv[(long long)pidx * m + k0 + lane] : -1;
+        zrows = __reduce_or_sync(0xffffffffu, pv >= 0 && (pv >> 5) == (rbase >> 5) ? 1u << (pv & 31) : 0u);
+      }
       // the values chunk ci's stores update, loaded one chunk ahead
       auto load_in = [&](int ci, double (&in)[8]) {
         const int n = w.tn * NTK + half * (NTK / 2) + 8 * ci + cl;
@@ -374,8 +382,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int rr = rbase + r0 + 4 * i;
-          in[i] = (upd && n < m && outside && rr < m && !(gj && rr >= k0 && rr < k0 + 32)) ? src[(long long)rr * m + n]
-                                                                                          : 0.0;
+          in[i] = (upd && n < m && outside && rr < m && !(gj && ((zrows >> (r0 + 4 * i)) & 1u)))
+                      ? src[(long long)rr * m + n]
+                      : 0.0;
         }
       };
       double incur[8], innext[8];
@@ -480,13 +489,13 @@ __global__ void __launch_bounds__(kThreads, 1)
               double* d = (j == 0) ? (t < p.L - 1 ? out.Acal : out.ZR) : out.ZL;
               d[o + e] = v;
             } else if (dnext) {
-              out.G[o + mm + e] = incur[i] - v;                    // D_{t+1} = B_{t+1} - A_{t+1} Acal_t
+              wk[e] = incur[i] - v;                                // D_{t+1} = B_{t+1} - A_{t+1} Acal_t
             } else if (KIND == 1) {
               out.Y[(long long)pidx * mm + e] = -v;                // Y_{t+1} = -A_{t+1} Bcal_t
             } else if (rmw) {
               out.ZL[o + e] = incur[i] - v;                        // ZL_t -= Acal_t ZL_{t+1}
             } else if (gj) {
-              out.G[o + e] = incur[i] + v;                         // Gauss-Jordan trailing update
+              wk[e] = incur[i] + v;                                // Gauss-Jordan trailing update
             } else {
               out.ZR[o + e] = -v;                                  // ZR_t = -Acal_t ZR_{t+1}
             }
@@ -626,485 +635,6 @@ __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__
 //   4 ZR_{L-1} columns (last row, right spike) -> slot;  5 Y_{t+1} columns -> rolling (q);
 //   6 ZL_t columns, backward step;        7 ZR_t columns, backward step;
 //   8 Y_0 = A_first columns -> rolling (q), at the start of a factorisation.
-// ---------------------------------------------------------------- blocked Gauss-Jordan inversion
-// The float64 block inverse G_t = D_t^{-1} with partial pivoting (the
-// paper's inversion, Section 4; Gauss-Jordan as in the library's other
-// inverses), blocked by panels of 32 columns so that 15/16 of its float64
-// multiply-adds (the rank-32 trailing updates) run on the tensor cores as
-// digit-sliced products (KIND 3 above).  For panel K = [k0, k0 + 32):
-//   1. k_gj_panel (float64, a cluster of CTAs per block, a thread per row
-//      holding the panel's 32 values): for each k in K, the pivot row r =
-//      argmax_{i >= k} |M[i][k]| (ties to the lowest row) is exchanged with
-//      row k, then in-place Gauss-Jordan restricted to the panel's columns:
-//      row k scaled by 1/M[k][k] with 1/M[k][k] in column k, every other row
-//      i minus M[i][k] times row k with -M[i][k]/M[k][k] in column k.  The
-//      panel then holds U = [W; -M_RK W] (W = M_KK^{-1}); the kernel applies
-//      the row exchanges to the other columns and writes U's row slices and
-//      the column slices of V = M[K, J] (the pivot rows outside K).
-//   2. k_oz_step<3>: M[:, J] = (M[:, J], rows K zeroed) + U V.
-// After the last panel, k_gj_finish undoes the row exchanges on the columns
-// (column c of the working matrix is column piv[c] of D^{-1}) and writes the
-// row slices of the inverse.
-__global__ void __launch_bounds__(256) k_gj_copy_b0(const PartDesc* __restrict__ parts, int m,
-                                                    const double* __restrict__ B, double* __restrict__ G) {
-  const PartDesc p = parts[blockIdx.x];
-  const long long mm = (long long)m * m;
-  for (long long e = threadIdx.x; e < mm; e += blockDim.x) G[p.blk + e] = B[p.blk + e];
-}
-
-// One panel, one cluster of kGjCS CTAs per block: CTA `rank` holds rows
-// [rank R, rank R + R) (R = ceil(m / kGjCS)); warp w of it rows R rank + 16 w
-// + (0..15), two lanes per row (lane = 16 h + row): lane half h holds panel
-// columns 16 h .. 16 h + 15 in registers, rotated by one column per pivot (at
-// pivot kk the row's register c of half h is panel column (kk + 16 h + c) mod
-// 32, so the pivot column is always register 0 of half 0 and the loop needs
-// no unrolling; after 32 pivots the order is back).
-//
-// GB300's float64 unit takes a warp instruction per about 68 cycles per SM
-// sub-partition and a dependent one 66 cycles later (a division about 460),
-// so the per-pivot chain keeps float64 instructions to the arithmetic: the
-// pivot search orders the float64 bits of |M[i][k]| as integers, the checks
-// read the bits, the reciprocal is taken once per CTA, the rank-1 update (16
-// multiply-adds per lane) is spread over four warps per CTA, and it overlaps
-// the cluster barrier by one pivot of lookahead.  With pivot kk's scaled row
-// known, every row first updates only its next pivot column; the warps and
-// then the CTA choose their best row for pivot kk + 1 on it (a strict order:
-// magnitude, then lowest row), and that row is published as it is BEFORE
-// pivot kk's update, with its multiplier f and the reciprocal of its updated
-// pivot (row k + 1 likewise).  The CTA arrives at the cluster barrier, makes
-// the bulk update of its rows, then waits; each lane then reads the kGjCS
-// candidates and element `lane` (+ 1, the rotation) of each candidate row
-// and of row k + 1 through distributed shared memory (one round of
-// independent loads), picks the winner and applies pivot kk's update to that
-// one element (the multiply-add its owner made).  The exchanges of rows
-// outside the panel are applied after the last pivot as one permutation
-// (pivot rows are always taken from rows >= k, so every row outside K that
-// moves receives a row of K).
-constexpr int kGjCS = 4;
-constexpr int kGjThreads = 128;
-constexpr int kGjWarps = kGjThreads / 32;
-static_assert(kGjWarps * 16 * kGjCS >= kMaxMTensor, "a lane pair per row");
-
-struct __align__(16) GjKey {
-  unsigned long long key;  // 0: not eligible; 1: NaN; else |value| bits + 2
-  int idx;                 // row (unique per thread, so the order is strict)
-  int pad;
-};
-
-struct __align__(16) GjCand {
-  unsigned long long key;
-  int idx, pad;
-  double inv;  // 1 / the candidate's updated pivot (0 when unusable)
-  double f;    // the candidate's multiplier of the previous pivot
-};
-
-__device__ __forceinline__ bool gj_before(unsigned long long ok, int oi, unsigned long long k, int i) {
-  return ok > k || (ok == k && oi < i);
-}
-
-__device__ __forceinline__ unsigned long long gj_key(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-  return b > 0x7ff0000000000000ull ? 1ull : b + 2ull;
-}
-
-// zero, below 2^-1022 (whose reciprocal overflows), at or above 2^1022
-// (whose reciprocal is not a normal number) or not finite
-__device__ __forceinline__ bool gj_unusable(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-  return b < 0x0010000000000000ull || b >= 0x7fd0000000000000ull;
-}
-
-// 1/x for a usable pivot x (2^-1022 <= |x| < 2^1022): the PTX reciprocal
-// approximation rcp.approx.ftz.f64 refined by two Newton-Raphson steps for
-// f(y) = 1/y - x, y <- y + y (1 - x y), each of which squares the relative
-// error (within about one unit in the last place of 1/x).  It has no
-// branch, so the compiler can interleave it with the pivot search.
-__device__ __forceinline__ double gj_recip(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
-}
-
-// The CTA's best of every lane's (key, idx): the warp's largest key (its high
-// word, then its low word among the lanes with that high word) and the lowest
-// row holding it, by three warp reductions; then the best of the warps' bests
-// after a CTA barrier (the same result in every thread).
-__device__ __forceinline__ GjKey gj_cta_best(unsigned long long key, int idx, GjKey* wbest, int warp, int lane) {
-  const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
-  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-  const unsigned mi = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? (unsigned)idx : 0xffffffffu);
-  key = ((unsigned long long)mh << 32) | ml;
-  idx = (int)mi;
-  if (lane == 0) wbest[warp] = GjKey{key, idx, 0};
-  __syncthreads();
-  GjKey best = wbest[0];
-#pragma unroll
-  for (int w = 1; w < kGjWarps; ++w) {
-    const GjKey o = wbest[w];
-    if (gj_before(o.key, o.idx, best.key, best.idx)) best = o;
-  }
-  return best;
-}
-
-__device__ __forceinline__ GjCand gj_read_cand(const GjCand* c) {
-  const uint4* v = reinterpret_cast<const uint4*>(c);
-  const uint4 a = v[0], b = v[1];
-  GjCand r;
-  r.key = ((unsigned long long)a.y << 32) | a.x;
-  r.idx = (int)a.z;
-  r.pad = 0;
-  r.inv = __hiloint2double((int)b.y, (int)b.x);
-  r.f = __hiloint2double((int)b.w, (int)b.z);
-  return r;
-}
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-
-__global__ void __launch_bounds__(kGjThreads) k_gj_panel(const PartDesc* __restrict__ parts, int t, int m, int panel,
-                                                        double* __restrict__ G, int* __restrict__ piv,
-                                                        __nv_bfloat16* __restrict__ Us, int* __restrict__ Uexp,
-                                                        __nv_bfloat16* __restrict__ Vs, int* __restrict__ Vexp,
-                                                        int* __restrict__ status) {
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  // published per pivot (double-buffered: a buffer is rewritten two pivots
-  // later, after a cluster barrier that every reader of it has passed)
-  __shared__ __align__(16) double crow[2][32], krow[2][32];
-  __shared__ GjCand cand[2];
-  __shared__ double kf[2];
-  // this CTA's own
-  __shared__ GjKey wbest[kGjWarps];
-  __shared__ __align__(16) double sprow[kGjWarps][32], xrow[kGjWarps][32];
-  __shared__ int piv_s[32], perm[kMaxMTensor], cperm[kMaxMTensor];
-  const int rank = (int)cl.block_rank();
-  const int q = blockIdx.x / kGjCS;
-  const PartDesc p = parts[q];
-  if (t >= p.L) return;  // the same for every CTA of the cluster
-  const long long mm = (long long)m * m;
-  double* M = G + p.blk + (long long)t * mm;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, h = lane >> 4, rl = warp * 16 + (lane & 15);
-  const int R = (m + kGjCS - 1) / kGjCS, i = rank * R + rl;
-  const bool valid = rl < R && i < m;
-  const int k0 = 32 * panel, kw = min(32, m - k0);  // kw % 8 == 0
-  const int noidx = m + rank * kGjThreads + tid;   // an index no row has
-  double reg[16];
-#pragma unroll
-  for (int c = 0; c < 16; c += 2) {
-    double2 v2 = make_double2(0.0, 0.0);
-    if (valid && 16 * h + c < kw) v2 = *reinterpret_cast<const double2*>(M + (long long)i * m + k0 + 16 * h + c);
-    reg[c] = v2.x;
-    reg[c + 1] = v2.y;
-  }
-  bool bad = false;
-  double* sp = sprow[warp];
-  double* xr = xrow[warp];
-  int r;  // the current pivot row
-  {
-    // pivot k0: candidates from the rows as they are
-    const bool elig = h == 0 && valid && i >= k0;
-    const GjKey best = gj_cta_best(elig ? gj_key(reg[0]) : 0ull, elig ? i : noidx, wbest, warp, lane);
-    if (valid && i == best.idx) {
-#pragma unroll
-      for (int c = 0; c < 16; c += 2)
-        *reinterpret_cast<double2*>(&crow[0][16 * h + c]) = make_double2(reg[c], reg[c + 1]);
-      if (h == 0) {
-        cand[0].inv = gj_unusable(reg[0]) ? 0.0 : gj_recip(reg[0]);
-        cand[0].f = 0.0;
-      }
-    }
-    if (valid && i == k0)
-#pragma unroll
-      for (int c = 0; c < 16; c += 2)
-        *reinterpret_cast<double2*>(&krow[0][16 * h + c]) = make_double2(reg[c], reg[c + 1]);
-    if (tid == 0) cand[0].key = best.key, cand[0].idx = best.idx;
-    cl.sync();
-    GjCand w = gj_read_cand(cl.map_shared_rank(&cand[0], 0));
-    double prow = cl.map_shared_rank(&crow[0][0], 0)[lane];
-#pragma unroll
-    for (int s = 1; s < kGjCS; ++s) {
-      const GjCand o = gj_read_cand(cl.map_shared_rank(&cand[0], s));
-      const double v = cl.map_shared_rank(&crow[0][0], s)[lane];
-      if (gj_before(o.key, o.idx, w.key, w.idx)) w = o, prow = v;
-    }
-    const double xk = cl.map_shared_rank(&krow[0][0], k0 / R)[lane];
-    const double p0 = __shfl_sync(0xffffffffu, prow, 0);
-    double inv = w.inv;
-    if (gj_unusable(p0)) inv = 0.0, bad = true;
-    r = w.idx;
-    if (r < k0 || r >= m) r = k0, inv = 0.0, bad = true;  // never: the winner is an eligible row
-    sp[lane] = lane == 0 ? inv : prow * inv;  // the scaled pivot row
-    xr[lane] = xk;                            // the old row k
-    if (tid == 0) piv_s[0] = r;
-    __syncwarp();
-  }
-  // the cluster's published candidates and rows, mapped once (buffer b at + b)
-  const GjCand* rcand[kGjCS];
-  const double* rcrow[kGjCS];
-#pragma unroll
-  for (int s = 0; s < kGjCS; ++s) {
-    rcand[s] = cl.map_shared_rank(&cand[0], s);
-    rcrow[s] = cl.map_shared_rank(&crow[0][0], s);
-  }
-  // the CTA holding row k + 1 and that row's place in it, advanced per pivot
-  int ko = (k0 + 1) / R, kro = (k0 + 1) - ko * R;
-#pragma unroll 1
-  for (int kk = 0; kk < 32; ++kk) {
-    if (kk >= kw) {  // padding columns of a narrow last panel: rotate only
-      const double nxt = __shfl_xor_sync(0xffffffffu, reg[0], 16);
-#pragma unroll
-      for (int c = 0; c < 15; ++c) reg[c] = reg[c + 1];
-      reg[15] = nxt;
-      continue;
-    }
-    const int k = k0 + kk;
-    const bool la = kk + 1 < kw, swap = i == r && i != k;  // row r takes the old row k
-    if (swap)
-#pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const double2 v2 = *reinterpret_cast<const double2*>(&xr[16 * h + c]);
-        reg[c] = v2.x;
-        reg[c + 1] = v2.y;
-      }
-    const double other = __shfl_xor_sync(0xffffffffu, reg[0], 16);  // the other half's first column
-    const double f = h == 0 ? reg[0] : other;  // the row's multiplier (column kk)
-    if (la) {
-      // the next pivot column of every row first, its candidates, and the
-      // CTA's best row published before the update
-      const int buf = (kk + 1) & 1;
-      const double new1 = i == k ? sp[1] : fma(-f, sp[1], reg[1]);
-      const bool elig = h == 0 && valid && i > k;
-      const double rinv = gj_recip(new1);  // every row's, overlapping the search
-      const GjKey best = gj_cta_best(elig ? gj_key(new1) : 0ull, elig ? i : noidx, wbest, warp, lane);
-      if (valid && i == best.idx) {
-#pragma unroll
-        for (int c = 0; c < 16; c += 2)
-          *reinterpret_cast<double2*>(&crow[buf][16 * h + c]) = make_double2(reg[c], reg[c + 1]);
-        if (h == 0) {
-          cand[buf].inv = gj_unusable(new1) ? 0.0 : rinv;
-          cand[buf].f = f;
-        }
-      }
-      if (valid && i == k + 1) {
-#pragma unroll
-        for (int c = 0; c < 16; c += 2)
-          *reinterpret_cast<double2*>(&krow[buf][16 * h + c]) = make_double2(reg[c], reg[c + 1]);
-        if (h == 0) kf[buf] = f;
-      }
-      if (tid == 0) cand[buf].key = best.key, cand[buf].idx = best.idx;
-      cluster_arrive();
-    }
-    // pivot kk's update of this thread's row, rotated by one column
-    if (valid) {
-      double s16[16];  // this half's 16 values of the scaled pivot row
-#pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const double2 v2 = *reinterpret_cast<const double2*>(&sp[16 * h + c]);
-        s16[c] = v2.x;
-        s16[c + 1] = v2.y;
-      }
-      const double snext = sp[h == 0 ? 16 : 0];  // the next half's first value
-      if (i == k) {
-#pragma unroll
-        for (int c = 0; c < 15; ++c) reg[c] = s16[c + 1];
-        reg[15] = snext;
-      } else {
-#pragma unroll
-        for (int c = 0; c < 15; ++c) reg[c] = fma(-f, s16[c + 1], reg[c + 1]);
-        reg[15] = h == 0 ? fma(-f, snext, other) : -f * snext;
-      }
-    }
-    if (la) {
-      cluster_wait();
-      const int buf = (kk + 1) & 1, src = (lane + 1) & 31;
-      GjCand w = gj_read_cand(rcand[0] + buf);
-      double pre = rcrow[0][32 * buf + src];
-#pragma unroll
-      for (int s = 1; s < kGjCS; ++s) {
-        const GjCand o = gj_read_cand(rcand[s] + buf);
-        const double v = rcrow[s][32 * buf + src];
-        if (gj_before(o.key, o.idx, w.key, w.idx)) w = o, pre = v;
-      }
-      const double kpre = cl.map_shared_rank(&krow[buf][0], ko)[src];
-      const double kfk = *cl.map_shared_rank(&kf[buf], ko);
-      if (++kro == R) kro = 0, ++ko;
-      // pivot kk's update of element `lane` of the winner and of row k + 1
-      const double spc = sp[src];
-      const double u = src == 0 ? -w.f * spc : fma(-w.f, spc, pre);
-      const double x = src == 0 ? -kfk * spc : fma(-kfk, spc, kpre);
-      // u at lane 0 is the winner's updated pivot, the same multiply-add of the
-      // same operands its owner made: the owner's inv is 0 exactly when it is unusable
-      double inv = w.inv;
-      if (inv == 0.0) bad = true;
-      r = w.idx;
-      if (r <= k || r >= m) r = k + 1, inv = 0.0, bad = true;  // never: the winner is an eligible row
-      __syncwarp();
-      sp[lane] = lane == 0 ? inv : u * inv;
-      xr[lane] = x;
-      if (tid == 0) piv_s[kk + 1] = r;
-      __syncwarp();
-    }
-  }
-  // the eliminated panel and the row slices of U (scale per row over its 32 values)
-  uint32_t hmax = 0;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) hmax = max(hmax, (uint32_t)(__double_as_longlong(reg[c]) >> 32) & 0x7fffffffu);
-  hmax = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, 16));
-  if (valid) {
-#pragma unroll
-    for (int c = 0; c < 16; c += 2)
-      if (16 * h + c < kw)
-        *reinterpret_cast<double2*>(M + (long long)i * m + k0 + 16 * h + c) = make_double2(reg[c], reg[c + 1]);
-    const int e = scale_exponent(hmax);
-    if (h == 0) Uexp[(long long)q * m + i] = e;
-    __nv_bfloat16* u = Us + (long long)q * S * m * 32 + (long long)i * 32 + 16 * h;
-#pragma unroll
-    for (int c0 = 0; c0 < 16; c0 += 8) {
-      uint32_t d[8][S];
-#pragma unroll
-      for (int uu = 0; uu < 8; ++uu) digits9((unsigned long long)__double_as_longlong(reg[c0 + uu]), e, d[uu]);
-#pragma unroll
-      for (int sl = 0; sl < S; ++sl) {
-        uint4 w;
-        w.x = (d[0][sl] >> 16) | (d[1][sl] & 0xffff0000u);
-        w.y = (d[2][sl] >> 16) | (d[3][sl] & 0xffff0000u);
-        w.z = (d[4][sl] >> 16) | (d[5][sl] & 0xffff0000u);
-        w.w = (d[6][sl] >> 16) | (d[7][sl] & 0xffff0000u);
-        *reinterpret_cast<uint4*>(u + (long long)sl * m * 32 + c0) = w;
-      }
-    }
-  }
-  // net row permutation of the pivots: position x ends up holding row perm[x];
-  // rank 0 also carries the inversion's column permutation (the exchanges of
-  // every panel so far applied in pivot order, from the identity at panel 0):
-  // column c of the final working matrix is column piv[c] of D^{-1}
-  int* colp = piv + (long long)q * m;
-  for (int c = tid; c < m; c += kGjThreads) {
-    perm[c] = c;
-    if (rank == 0) cperm[c] = panel == 0 ? c : colp[c];
-  }
-  __syncthreads();
-  if (tid == 0)
-    for (int kk = 0; kk < kw; ++kk) {
-      const int a = k0 + kk, b = piv_s[kk];
-      int tmp = perm[a];
-      perm[a] = perm[b];
-      perm[b] = tmp;
-      if (rank == 0) {
-        tmp = cperm[a];
-        cperm[a] = cperm[b];
-        cperm[b] = tmp;
-      }
-    }
-  __syncthreads();
-  if (rank == 0)
-    for (int c = tid; c < m; c += kGjThreads) colp[c] = cperm[c];
-  // a thread per column outside the panel (shared among the cluster's CTAs):
-  // the column slices of V = the pivot rows (transposed: row j of the copy
-  // holds V[0..31][j]; zero inside the panel), then the rows outside K that
-  // took part in an exchange receive their rows of K (read before written:
-  // the V loads come first, from this thread's own column)
-  for (int jcol = tid * kGjCS + rank; jcol < m; jcol += kGjCS * kGjThreads) {
-    const bool inK = jcol >= k0 && jcol < k0 + kw;
-    double vv[32];
-    uint32_t vmax = 0;
-#pragma unroll
-    for (int kk = 0; kk < 32; ++kk) {
-      vv[kk] = (!inK && kk < kw) ? M[(long long)perm[k0 + kk] * m + jcol] : 0.0;
-      vmax = max(vmax, (uint32_t)(__double_as_longlong(vv[kk]) >> 32) & 0x7fffffffu);
-    }
-    if (!inK)
-      for (int kk = 0; kk < kw; ++kk) {
-        const int x = piv_s[kk];
-        if (x >= k0 + kw) M[(long long)x * m + jcol] = M[(long long)perm[x] * m + jcol];
-      }
-    const int e = scale_exponent(vmax);
-    Vexp[(long long)q * m + jcol] = e;
-    __nv_bfloat16* vdst = Vs + (long long)q * S * m * 32 + (long long)jcol * 32;
-#pragma unroll
-    for (int c0 = 0; c0 < 32; c0 += 8) {
-      uint32_t d[8][S];
-#pragma unroll
-      for (int uu = 0; uu < 8; ++uu) digits9((unsigned long long)__double_as_longlong(vv[c0 + uu]), e, d[uu]);
-#pragma unroll
-      for (int sl = 0; sl < S; ++sl) {
-        uint4 w;
-        w.x = (d[0][sl] >> 16) | (d[1][sl] & 0xffff0000u);
-        w.y = (d[2][sl] >> 16) | (d[3][sl] & 0xffff0000u);
-        w.z = (d[4][sl] >> 16) | (d[5][sl] & 0xffff0000u);
-        w.w = (d[6][sl] >> 16) | (d[7][sl] & 0xffff0000u);
-        *reinterpret_cast<uint4*>(vdst + (long long)sl * m * 32 + c0) = w;
-      }
-    }
-  }
-  if (rank == 0 && tid == 0 && bad) atomicMin(status + p.sys, p.row0 + t + 1);
-  cl.sync();  // no CTA leaves while another may still read its shared memory
-}
-
-// After the last panel: the column permutation undone and the row slices of
-// the block inverse G_t written (the left operand of the next products), one
-// pass: a CTA takes 32 rows of one block (blockIdx.x = block * groups +
-// group), a warp a row at a time: the row is read once, scattered to its
-// final column order in shared memory (its largest magnitude does not depend
-// on the order), then written back as float64 and as nine digit slices.
-__global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ parts, int t, int m,
-                                                   double* __restrict__ G, const int* __restrict__ piv,
-                                                   __nv_bfloat16* __restrict__ Gs, int* __restrict__ eG) {
-  __shared__ int ip[kMaxMTensor];
-  __shared__ __align__(16) double rowb[8][kMaxMTensor];
-  const int groups = (m + 31) / 32;
-  const int q = blockIdx.x / groups, g = blockIdx.x - q * groups;
-  const PartDesc p = parts[q];
-  if (t >= p.L) return;
-  const long long mm = (long long)m * m;
-  double* M = G + p.blk + (long long)t * mm;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int c = threadIdx.x; c < m; c += blockDim.x) ip[c] = piv[(long long)q * m + c];
-  __syncthreads();
-  double* rb = rowb[warp];
-  const int rend = min(m, 32 * g + 32);
-  for (int r = 32 * g + warp; r < rend; r += 8) {
-    uint32_t hmax = 0;
-    for (int c = lane; c < m; c += 32) {
-      const double v = M[(long long)r * m + c];
-      rb[ip[c]] = v;
-      hmax = max(hmax, (uint32_t)(__double_as_longlong(v) >> 32) & 0x7fffffffu);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) hmax = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, o));
-    const int e = scale_exponent(hmax);
-    if (lane == 0) eG[(long long)q * m + r] = e;
-    __syncwarp();
-    for (int c0 = lane * 8; c0 < m; c0 += 256) {  // m % 8 == 0
-      double v[8];
-#pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        const double2 d2 = *reinterpret_cast<const double2*>(rb + c0 + u);
-        v[u] = d2.x;
-        v[u + 1] = d2.y;
-        *reinterpret_cast<double2*>(M + (long long)r * m + c0 + u) = d2;
-      }
-      uint32_t d[8][S];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) digits9((unsigned long long)__double_as_longlong(v[u]), e, d[u]);
-#pragma unroll
-      for (int sl = 0; sl < S; ++sl) {
-        uint4 w;
-        w.x = (d[0][sl] >> 16) | (d[1][sl] & 0xffff0000u);
-        w.y = (d[2][sl] >> 16) | (d[3][sl] & 0xffff0000u);
-        w.z = (d[4][sl] >> 16) | (d[5][sl] & 0xffff0000u);
-        w.w = (d[6][sl] >> 16) | (d[7][sl] & 0xffff0000u);
-        *reinterpret_cast<uint4*>(Gs + ((long long)q * S + sl) * mm + (long long)r * m + c0) = w;
-      }
-    }
-    __syncwarp();
-  }
-}
-
 // Several per-subsystem slicing jobs in one launch (blockIdx.y = job).
 __global__ void __launch_bounds__(256) k_oz_slice_jobs(const PartDesc* __restrict__ parts, int step, int m,
                                                        OzSliceJobs jobs) {
@@ -1236,8 +766,8 @@ __device__ __forceinline__ void load_row_band(double (*lb)[2 * kBandMax + 1], co
 __global__ void __launch_bounds__(256) k_band_b(const PartDesc* __restrict__ parts, int t, int m,
                                                 const double* __restrict__ A, const double* __restrict__ B,
                                                 const double* __restrict__ Acal, const double* __restrict__ ZL,
-                                                double* __restrict__ G, double* __restrict__ Y,
-                                                const int* __restrict__ band) {
+                                                double* __restrict__ G, double* __restrict__ W,
+                                                double* __restrict__ Y, const int* __restrict__ band) {
   __shared__ double lb[32][2 * kBandMax + 1];
   const int w = *band;
   if (w > kBandMax) return;
@@ -1249,13 +779,14 @@ __global__ void __launch_bounds__(256) k_band_b(const PartDesc* __restrict__ par
   load_row_band(lb, A + o + mm, g, m, w);
   __syncthreads();
   const double* X = (j == 0 ? Acal : ZL) + o;
+  double* D = W ? W + (long long)q * mm : G + o + mm;  // the inversion's working matrix, if there is one
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int r = 32 * g + warp; r < min(m, 32 * g + 32); r += 8)
     for (int n = lane; n < m; n += 32) {
       const double v = band_row(lb[r - 32 * g], X, r, n, m, w);
       const long long e = (long long)r * m + n;
       if (j == 0)
-        G[o + mm + e] = B[o + mm + e] - v;  // D_{t+1}
+        D[e] = B[o + mm + e] - v;           // D_{t+1}
       else
         Y[(long long)q * mm + e] = -v;      // Y_{t+1}
     }
@@ -1381,60 +912,17 @@ void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, co
   oz::k_oz_slice_jobs<<<dim3(nparts * ((m + 31) / 32), njobs), 256, 0, st>>>(parts, step, m, jobs);
 }
 
-// The blocked Gauss-Jordan inversion of block row t of every active
-// subsystem (in place in G; t = 0 starts from B_0), as four phases: the copy
-// of B_0, per panel of 32 columns the panel and its trailing update, and the
-// finishing pass (the column permutation undone, the row slices written).
-void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* G, cudaStream_t st) {
-  if (nparts > 0 && t == 0) oz::k_gj_copy_b0<<<nparts, 256, 0, st>>>(parts, m, B, G);
-}
-
-void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* G, int* piv, void* Us,
-                     int* Uexp, void* Vs, int* Vexp, int* status, cudaStream_t st) {
+// The trailing update of one panel of the blocked inversion (dm_gj.cu).
+void launch_gj_update(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, const int* piv,
+                      const int* Uexp, const int* Vexp, const void* maps2, int* errflag, cudaStream_t st) {
   if (nparts <= 0) return;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nparts * oz::kGjCS);
-  cfg.blockDim = dim3(oz::kGjThreads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = oz::kGjCS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, oz::k_gj_panel, parts, t, m, pnl, G, piv, static_cast<__nv_bfloat16*>(Us), Uexp,
-                     static_cast<__nv_bfloat16*>(Vs), Vexp, status);
-}
-
-void launch_gj_update(const PartDesc* parts, int nparts, int t, int m, int pnl, double* G, const int* Uexp,
-                      const int* Vexp, const void* maps2, int* errflag, cudaStream_t st) {
-  if (nparts <= 0) return;
-  OzOut out{nullptr, G, nullptr, nullptr, nullptr, nullptr};
+  OzOut out{};
+  out.W = W;
+  out.piv = piv;
   unsigned char maps3[3 * 128];
   std::memcpy(maps3, maps2, 2 * 128);
   std::memcpy(maps3 + 2 * 128, static_cast<const unsigned char*>(maps2) + 128, 128);
   launch_oz_step(3, parts, nparts, pnl, m, out, Uexp, Vexp, Vexp, maps3, errflag, st, t);
-}
-
-void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, double* G, const int* piv, void* Gs, int* eG,
-                      cudaStream_t st) {
-  if (nparts <= 0) return;
-  oz::k_gj_finish<<<nparts * ((m + 31) / 32), 256, 0, st>>>(parts, t, m, G, piv, static_cast<__nv_bfloat16*>(Gs),
-                                                             eG);
-}
-
-void launch_gj_inverse(const PartDesc* parts, int nparts, int t, int m, const double* B, double* G, int* piv,
-                       void* Us, int* Uexp, void* Vs, int* Vexp, const void* maps2, int* status, int* errflag,
-                       void* Gs, int* eG, cudaStream_t st) {
-  if (nparts <= 0) return;
-  launch_gj_begin(parts, nparts, t, m, B, G, st);
-  for (int pnl = 0; pnl < (m + 31) / 32; ++pnl) {
-    launch_gj_panel(parts, nparts, t, m, pnl, G, piv, Us, Uexp, Vs, Vexp, status, st);
-    if (m > 32) launch_gj_update(parts, nparts, t, m, pnl, G, Uexp, Vexp, maps2, errflag, st);
-  }
-  launch_gj_finish(parts, nparts, t, m, G, piv, Gs, eG, st);
 }
 
 void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m, const OzOut& out, const int* lexp,
@@ -1479,7 +967,13 @@ void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, 
   if (nseps <= 0) return;
   oz::k_oz_slice_seps<<<dim3(nseps * ((m + 31) / 32), 5), 256, 0, st>>>(
       seps, m, C, ZL, ZR, static_cast<__nv_bfloat16*>(a.Cq), a.eCq, static_cast<__nv_bfloat16*>(a.S), a.eS, band);
-  OzOut out{B, nullptr, nullptr, nullptr, nullptr, nullptr, seps, HA, HB, HC, band};
+  OzOut out{};
+  out.B = B;
+  out.seps = seps;
+  out.HA = HA;
+  out.HB = HB;
+  out.HC = HC;
+  out.band = band;
   unsigned char maps3[3 * 128];
   std::memcpy(maps3, mapA, 128);
   std::memcpy(maps3 + 128, a.maps[1], 128);
@@ -1496,9 +990,10 @@ void launch_band_gc(const PartDesc* parts, int nparts, int t, int m, const doubl
 }
 
 void launch_band_b(const PartDesc* parts, int nparts, int t, int m, const double* A, const double* B,
-                   const double* Acal, const double* ZL, double* G, double* Y, const int* band, cudaStream_t st) {
+                   const double* Acal, const double* ZL, double* G, double* W, double* Y, const int* band,
+                   cudaStream_t st) {
   if (nparts <= 0 || !band) return;
-  oz::k_band_b<<<dim3(nparts * ((m + 31) / 32), 2), 256, 0, st>>>(parts, t, m, A, B, Acal, ZL, G, Y, band);
+  oz::k_band_b<<<dim3(nparts * ((m + 31) / 32), 2), 256, 0, st>>>(parts, t, m, A, B, Acal, ZL, G, W, Y, band);
 }
 
 void launch_band_h(const SepDesc* seps, int nseps, int m, const double* A, const double* B, const double* C,

@@ -46,6 +46,35 @@ __device__ __forceinline__ void digits9(unsigned long long bits, int e, uint32_t
     q[k] = __float_as_uint(__uint_as_float(0x4b000000u | d[k]) - 8388608.0f) | sign;
 }
 
+constexpr int kBalSlices = 7;
+
+// Seven balanced base-256 digits of v, |v| < 2^e: v = 2^(e+1) sum_{s=1..7}
+// d_s 2^(-8s), rounded to the nearest multiple of 2^(e-55), every d_s an
+// integer in [-128, 128] and so exact in bf16 (bit patterns in the high half
+// of each word, as digits9).  The scaled integer is biased by 128 in every
+// byte, so that each digit is one byte minus 128.  v must be finite.
+__device__ __forceinline__ void digits7(unsigned long long bits, int e, uint32_t (&q)[kBalSlices]) {
+  const int ex = (int)((bits >> 52) & 0x7ff);
+  const unsigned long long mant = (bits & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
+  const int sh = (ex ? ex : 1) - 1075 + 55 - e;  // <= 2 for |v| < 2^e
+  const int dn = min(-sh, 60);
+  const unsigned long long Y = sh >= 0 ? (mant << (sh & 63)) : ((mant + (1ull << (dn - 1))) >> dn);
+  const unsigned long long Z = ((bits >> 63) ? 0ull - Y : Y) + 0x0080808080808080ull;
+  const uint32_t hi = (uint32_t)(Z >> 32), lo = (uint32_t)Z;
+  const uint32_t w[kBalSlices] = {0x4b000000u | (hi >> 16),
+                                  __byte_perm(hi, 0x4b000000u, 0x7541),
+                                  __byte_perm(hi, 0x4b000000u, 0x7540),
+                                  __byte_perm(lo, 0x4b000000u, 0x7543),
+                                  __byte_perm(lo, 0x4b000000u, 0x7542),
+                                  __byte_perm(lo, 0x4b000000u, 0x7541),
+                                  __byte_perm(lo, 0x4b000000u, 0x7540)};
+#pragma unroll
+  for (int k = 0; k < kBalSlices; ++k) q[k] = __float_as_uint(__uint_as_float(w[k]) - 8388736.0f);
+}
+
+// Two bf16 values (high halves of a and b) in one register, a first.
+__device__ __forceinline__ uint32_t pack_hi(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
+
 // Exponent e with |v| < 2^e for every v whose high word (sign cleared) is at
 // most hmax; subnormal or zero maxima share e = -1021.
 __device__ __forceinline__ int scale_exponent(uint32_t hmax) {
