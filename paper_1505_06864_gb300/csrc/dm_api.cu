@@ -310,7 +310,7 @@ static bool oz_wanted(const Level& L) {
 static size_t oz_bytes(long long nblk, int nparts, int nseps, int m) {
   const size_t mm = (size_t)m * m, sl = (size_t)oz_slice_blocks_bytes(m), nb = nblk / mm, np = std::max(1, nparts);
   return (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + 2 * np * mm * sizeof(double) +
-         np * ((size_t)2 * 9 * m * 32 * 2 + 3 * m * sizeof(int));
+         np * ((size_t)2 * 7 * m * 32 * 2 + 3 * m * sizeof(int));
 }
 
 // The supplementary blocks of a sliced level as digit-sliced tensor-core
@@ -445,11 +445,11 @@ int Level::allocate() {
     const long long rblk[5] = {nb, np, np, 2 * np, 2 * np};
     bool ok = true;
     for (int i = 0; ok && i < 3; ++i) ok = oz_make_map(lbase[i], lblk[i], m, oz_box_rows_left(), Z.maps[i]);
-    for (int i = 0; ok && i < 5; ++i) ok = oz_make_map(rbase[i], rblk[i], m, oz_box_rows_right(), Z.maps[3 + i]);
+    for (int i = 0; ok && i < 5; ++i) ok = oz_make_map(rbase[i], rblk[i], m, oz_box_rows_right(m), Z.maps[3 + i]);
     if (!ok) return set_error(DM_ECUDA, "tensor map creation for the float64 slice products failed (m = %d)", m);
     Z.on = true;
     if (gj_wanted(*this)) {
-      const size_t pb = (size_t)9 * m * 32 * 2;
+      const size_t pb = (size_t)7 * m * 32 * 2;
       DM_ALLOC(Z.W, np * mm * sizeof(double));
       DM_ALLOC(Z.U, np * pb);
       DM_ALLOC(Z.V, np * pb);
@@ -478,7 +478,7 @@ int Level::allocate() {
       DM_ALLOC(a.eCq, nseps * ex);
       DM_ALLOC(a.eS, 4LL * nseps * ex);
       ok = oz_make_map(a.Cq, nseps, m, oz_box_rows_left(), a.maps[0]) &&
-           oz_make_map(a.S, 4LL * nseps, m, oz_box_rows_right(), a.maps[1]);
+           oz_make_map(a.S, 4LL * nseps, m, oz_box_rows_right(m), a.maps[1]);
       if (!ok) return set_error(DM_ECUDA, "tensor map creation for the sliced assembly failed (m = %d)", m);
       Z.asm_on = true;
     }
@@ -729,7 +729,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
   Cost cslice = L.c_cvt;
   DM_LAUNCH_K(pf, st, K_TC_CONVERT, cslice, 1, Z.band ? 4 : 3, slice_inputs());
   Cost cs;
-  cs.bytes = 26.0 * m * m;  // one block: float64 read, nine bf16 slices written
+  cs.bytes = (8.0 + 2.0 * oz_slices(m)) * m * m;  // one block: float64 read, its bf16 slices written
   for (int t = 0; t < L.Lmax; ++t) {
     const int np = L.active_fwd[t], nbk = L.active_back[t];
     if (Z.gj) {
@@ -739,15 +739,15 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
       // G_t's row slices
       Cost cb, cf;
       cb.bytes = np * 16.0 * m * m;           // B_0 read, written to G
-      cf.bytes = np * (16.0 + 18.0) * m * m;  // G_t read and written, nine bf16 slices written
+      cf.bytes = np * (16.0 + 2.0 * oz_slices(m)) * m * m;  // G_t read and written, its bf16 slices written
       if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, Z.W, st));
       for (int k0 = 0; k0 < m; k0 += 32) {
         const double kw = std::min(32, m - k0);
         Cost cp, cu;
         cp.flops = np * 2.0 * m * kw * kw;
-        cp.bytes = np * (16.0 * m * kw + 18.0 * 32.0 * 2 * m + 8.0 * kw * m);
+        cp.bytes = np * (16.0 * m * kw + 14.0 * 32.0 * 2 * m + 8.0 * kw * m);
         cu.flops = np * 2.0 * m * (m - kw) * kw;
-        cu.bytes = np * (16.0 * m * (m - kw) + 18.0 * 32.0 * 2 * m);
+        cu.bytes = np * (16.0 * m * (m - kw) + 14.0 * 32.0 * 2 * m);
         DM_LAUNCH(pf, st, K_INV_PANEL, cp, np,
                   launch_gj_panel(L.d_parts, np, t, m, k0 / 32, Z.W, Z.piv, Z.U, Z.eU, Z.V, Z.eV, L.status, st));
         if (m > 32)

@@ -32,7 +32,7 @@
 namespace dm {
 namespace gj {
 
-constexpr int S = kRsSlices;
+constexpr int S = kBalSlices;           // digit slices of U and V (K = 32)
 constexpr int PW = 32;                 // panel width
 constexpr int SW = 8;                  // subpanel width
 constexpr int PS = PW + 1;             // row stride of the panel in shared memory (float64)
@@ -149,7 +149,7 @@ __device__ __forceinline__ void gj_pivot(const GjRows<RPL>& in, GjRows<RPL>& out
     GjCand& cd = sh.cand[buf][warp];
     cd.v = bnv;
     cd.key = wkey;
-    cd.idx = 32 * warp + lane + 128 * bi;
+    cd.idx = 32 * warp + lane + 32 * CW * bi;
   }
   asm volatile("bar.arrive 1, %0;" ::"r"(32 * nw + 32) : "memory");
   // src < 32: adds nothing, but keeps the multiply-adds below after the search
@@ -261,20 +261,6 @@ __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, 
       : "r"(a0), "r"(a1), "r"(b0));
 }
 
-// T 2^s rounded to float64 (to nearest, halves up), |T| < 2^63, by integer
-// operations; `odd` is set when the result is outside the normal range (then
-// the value is not the result).
-__device__ __forceinline__ double round_scaled(long long T, int s, bool& odd) {
-  const unsigned long long a = (unsigned long long)(T < 0 ? -T : T);
-  const int lz = __clzll(a);
-  const unsigned long long an = a << (lz & 63);                   // leading bit at 63
-  const unsigned long long mant = (an >> 11) + ((an >> 10) & 1);  // leading bit at 52 (or 2^53)
-  const int ex = 1022 + 63 - lz + s;                              // the leading bit adds one to the exponent
-  odd = odd || (a != 0 && (unsigned)ex > 2044u);
-  const unsigned long long r = ((unsigned long long)T & 0x8000000000000000ull) + ((unsigned long long)ex << 52) + mant;
-  return __longlong_as_double(a == 0 ? 0ll : (long long)r);
-}
-
 constexpr int kNotFinite = 1 << 14;  // scale of a row or column with a NaN or an infinity
 
 __device__ __forceinline__ int bal_exponent(uint32_t hmax) {
@@ -299,6 +285,7 @@ __device__ __noinline__ void gj_rank8(double* P, const double (*V)[PW], int mt, 
   int fe[2], qb = -1, nc = 0;
 #pragma unroll 1
   for (int i = wi; i < mt * nq; i += nwk) {
+    __syncwarp();  // mma.sync below takes whole warps
     const int q = i / mt, rt = i - q * mt;
     if (q != qb) {  // the group's digits of V
       qb = q;
@@ -309,8 +296,8 @@ __device__ __noinline__ void gj_rank8(double* P, const double (*V)[PW], int mt, 
       h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
       const int e = bal_exponent(h);
       uint32_t d0[kBalSlices], d1[kBalSlices];
-      digits7((unsigned long long)__double_as_longlong(v0), e, d0);
-      digits7((unsigned long long)__double_as_longlong(v1), e, d1);
+      digits<7>((unsigned long long)__double_as_longlong(v0), e, d0);
+      digits<7>((unsigned long long)__double_as_longlong(v1), e, d1);
 #pragma unroll
       for (int k = 0; k < kBalSlices; ++k) b[k] = pack_hi(d0[k], d1[k]);
       fe[0] = __shfl_sync(0xffffffffu, e, 8 * tg);
@@ -329,8 +316,8 @@ __device__ __noinline__ void gj_rank8(double* P, const double (*V)[PW], int mt, 
         h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
         re[h2] = bal_exponent(h);
         uint32_t d0[kBalSlices], d1[kBalSlices];
-        digits7((unsigned long long)__double_as_longlong(v0), re[h2], d0);
-        digits7((unsigned long long)__double_as_longlong(v1), re[h2], d1);
+        digits<7>((unsigned long long)__double_as_longlong(v0), re[h2], d0);
+        digits<7>((unsigned long long)__double_as_longlong(v1), re[h2], d1);
 #pragma unroll
         for (int k = 0; k < kBalSlices; ++k) a[h2][k] = pack_hi(d0[k], d1[k]);
         z[h2] = false;
@@ -391,7 +378,7 @@ __device__ __noinline__ void gj_slice8(double v0, double v1, double v2, double v
   const double v[8] = {v0, v1, v2, v3, v4, v5, v6, v7};
   uint32_t d[8][S];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) digits9((unsigned long long)__double_as_longlong(v[c]), e, d[c]);
+  for (int c = 0; c < 8; ++c) digits<S>((unsigned long long)__double_as_longlong(v[c]), e, d[c]);
 #pragma unroll
   for (int sl = 0; sl < S; ++sl)
     *reinterpret_cast<uint4*>(dst + (long long)sl * stride) =
@@ -510,17 +497,19 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
 // = block * groups + group), a warp a row at a time: the row is read once,
 // scattered to its final column order in shared memory (its largest magnitude
 // does not depend on the order), then written as float64 and as digit slices.
+template <int S>
 __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ parts, int t, int m,
                                                    const double* __restrict__ W, double* __restrict__ G,
                                                    const int* __restrict__ piv, __nv_bfloat16* __restrict__ Gs,
                                                    int* __restrict__ eG) {
-  __shared__ int ip[kMaxMTensor];
-  __shared__ __align__(16) double rowb[8][kMaxMTensor];
+  __shared__ int ip[kMaxM];
+  __shared__ double rowb[8][kMaxM];
   const int groups = (m + 31) / 32;
   const int q = blockIdx.x / groups, g = blockIdx.x - q * groups;
   const PartDesc p = parts[q];
   if (t >= p.L) return;
   const long long mm = (long long)m * m;
+  const int mp = slice_pitch(m);
   const double* M = W + (long long)q * mm;
   double* Gt = G + p.blk + (long long)t * mm;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -540,21 +529,17 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
     const int e = scale_exponent(hmax);
     if (lane == 0) eG[(long long)q * m + r] = e;
     __syncwarp();
-    for (int c0 = lane * 8; c0 < m; c0 += 256) {  // m % 8 == 0
+    for (int c = lane; c < m; c += 32) Gt[(long long)r * m + c] = rb[c];
+    for (int c0 = lane * 8; c0 < m; c0 += 256) {
       double v[8];
 #pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        const double2 d2 = *reinterpret_cast<const double2*>(rb + c0 + u);
-        v[u] = d2.x;
-        v[u + 1] = d2.y;
-        *reinterpret_cast<double2*>(Gt + (long long)r * m + c0 + u) = d2;
-      }
+      for (int u = 0; u < 8; ++u) v[u] = c0 + u < m ? rb[c0 + u] : 0.0;
       uint32_t d[8][S];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) digits9((unsigned long long)__double_as_longlong(v[u]), e, d[u]);
+      for (int u = 0; u < 8; ++u) digits<S>((unsigned long long)__double_as_longlong(v[u]), e, d[u]);
 #pragma unroll
       for (int sl = 0; sl < S; ++sl)
-        *reinterpret_cast<uint4*>(Gs + ((long long)q * S + sl) * mm + (long long)r * m + c0) =
+        *reinterpret_cast<uint4*>(Gs + (((long long)q * S + sl) * m + r) * mp + c0) =
             make_uint4(pack_hi(d[0][sl], d[1][sl]), pack_hi(d[2][sl], d[3][sl]), pack_hi(d[4][sl], d[5][sl]),
                        pack_hi(d[6][sl], d[7][sl]));
     }
@@ -598,8 +583,12 @@ void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, d
 void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
                       void* Gs, int* eG, cudaStream_t st) {
   if (nparts <= 0) return;
-  gj::k_gj_finish<<<nparts * ((m + 31) / 32), 256, 0, st>>>(parts, t, m, W, G, piv, static_cast<__nv_bfloat16*>(Gs),
-                                                             eG);
+  const int grid = nparts * ((m + 31) / 32);
+  auto* g = static_cast<__nv_bfloat16*>(Gs);
+  if (oz_slices(m) == 7)
+    gj::k_gj_finish<7><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG);
+  else
+    gj::k_gj_finish<8><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG);
 }
 
 }  // namespace dm

@@ -160,16 +160,18 @@ struct OzOut {
 };
 constexpr int kBandMax = 6;
 bool oz_eligible(int m);
+// digit slices per block (dm_slices.cuh): 7 (base 256) to m = 128, 8 (base 128) above
+int oz_slices(int m);
 int oz_slice_blocks_bytes(int m);
 bool oz_make_map(const void* base, long long blocks, int m, int box_rows, void* out, int kdim = 0);
 int oz_box_rows_left();
-int oz_box_rows_right();
+int oz_box_rows_right(int m);
 int oz_box_rows_gj();  // rows of the right operand's box in the inverse's trailing updates
 // The supplementary blocks of a sliced level (Eq. e2311) as digit-sliced
 // products: C_q row slices and the four boundary spike blocks' column slices
 // per separator, then HB = B_q - A_q ZR - C_q ZL, HA = -A_q ZL, HC = -C_q ZR.
 struct OzAsm {
-  void *Cq, *S;   // [separator][9][m][m] C_q rows; [4 separator + b][9][m][m] spike columns
+  void *Cq, *S;   // [separator][slices][m][m] C_q rows; [4 separator + b][slices][m][m] spike columns
   int *eCq, *eS;  // their scales
   alignas(64) unsigned char maps[2][128];  // left Cq, right S
 };
@@ -211,9 +213,9 @@ void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m
 // [nparts][m][m], with the rank-32 updates as digit-sliced tensor-core
 // products; maps2 = the panel-slice maps (U with 128-row boxes, V with
 // oz_box_rows_gj() rows), piv [nparts][m] (the pivot row of every column), Us /
-// Vs [nparts][9][m][32] bf16, Uexp / Vexp [nparts][m].  Phases: begin (t = 0
+// Vs [nparts][7][m][32] bf16, Uexp / Vexp [nparts][m].  Phases: begin (t = 0
 // only: W = B_0), per panel panel and update, finish (the inverse to G_t, its
-// row slices to Gs [nparts][9][m][m] bf16 / eG [nparts][m]).
+// row slices to Gs [nparts][oz_slices(m)][m][m] bf16 / eG [nparts][m]).
 void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, cudaStream_t st);
 void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, int* piv, void* Us,
                      int* Uexp, void* Vs, int* Vexp, int* status, cudaStream_t st);

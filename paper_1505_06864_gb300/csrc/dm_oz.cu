@@ -5,31 +5,32 @@
 // The products are the ones of the tensor-core step kernels (dm_tc2.cu):
 // launch A = G_t [C_t | Y_t], launch B = A_{t+1} [Acal_t | Bcal_t], backward
 // Acal_t [ZL_{t+1} | ZR_{t+1}] (Section 3 applied to Eq. e231), here with
-// float64 operands and results.  Every operand block is cut into nine digit
+// float64 operands and results.  Every operand block is cut into S digit
 // slices (dm_slices.cuh): a left operand L with one power-of-two scale per
 // row r (|L[r][k]| < 2^e_r), a right operand R with one per column n
 // (|R[k][n]| < 2^f_n), stored transposed (row n of the copy is column n of
-// R).  Then
+// R).  Then, with the digits' base b = 2^8 (S = 7) or 2^7 (S = 8),
 //
-//   (L R)[r][n] = 2^(e_r + f_n) sum_{d=2..11} 2^(-6d) acc_d[r][n],
+//   (L R)[r][n] = 2^(e_r + f_n + 2) sum_{d=2..S+2} b^(-d) acc_d[r][n],
 //   acc_d = sum_{s+t=d} Lslice_s Rslice_t,
 //
-// keeping the 53 slice pairs with s + t <= 11.  Each acc_d sums at most nine
-// slice products over K = m <= 256 terms of magnitude <= 63^2: integers below
-// 9 * 256 * 3969 < 2^24, so the float32 accumulation in tensor memory is
-// exact.  The dropped pairs and the digit truncation bound the error of an
-// entry by about K 2^-50 max_k |L[r][k]| max_k |R[k][n]|, the size of the
-// float64 dot product's own bound.
+// keeping the slice pairs with s + t <= S + 2 (34 of 49 and 43 of 64).  The
+// digits are balanced (|digit| <= b / 2), so each acc_d is an integer of at most
+// S K b^2 / 4 <= 2^24 for K <= 128 (S = 7) and K <= 512 (S = 8), and the
+// float32 accumulation in tensor memory is exact.  Operands are rounded at
+// 2^-56 of their scale (as far as they are smaller than a quarter of it: the
+// others are exact), the dropped pairs are below 2^-61 sqrt(K) max_k |L[r][k]|
+// max_k |R[k][n]|.  (Without the last diagonal, 28 and 36 pairs, the dropped
+// ones doubled the error of systems with cond(B_i) = 1e4.)
 //
-// A CTA computes a 128 x 48 tile of one product: ten accumulators of 48
-// columns (480 tensor-memory columns), a two-stage ring of 32-wide K slabs
-// (nine left slices 72 KB + nine right slices 27 KB + a zero slice), one CTA
-// per SM.  Per 16-wide K step one thread issues 14 MMAs: left slice s
-// against right slices t = 1 .. T_s at once (stored consecutively, N = 48 per
-// slice, at most five per instruction), into accumulators d = s + t.  With
-// s = 1 the right slices run to a tenth, all-zero slice, so that the first
-// K step's two instructions for s = 1 initialise all ten accumulators.  The
-// epilogue combines the accumulators in 64-bit integers and scales once in
+// A CTA computes a tile of one product: 128 x 64 (S = 7) or 128 x 48 (S = 8),
+// 128 x 32 for KIND 3: S + 1 accumulators in tensor memory (512 or 432 columns;
+// KIND 3: two sets of 256), a two-stage ring of 32-wide K slabs, one CTA per
+// SM.  Per 16-wide K step one thread issues the MMAs: left slice s against
+// right slices t = 1 .. min(S, S + 2 - s) at once (stored consecutively, at
+// most N = 256 per instruction), into accumulators d = s + t; s = 1 and the
+// pair (2, S) cover all of them, so they initialise them in the first K step.
+// The epilogue combines the accumulators in 64-bit integers and scales once in
 // float64 (GB300's float64 pipe is narrow).  Operand slices of results are
 // made by separate slicing launches, which see whole rows and columns.
 #include <cuda.h>
@@ -48,26 +49,32 @@ namespace dm {
 namespace oz {
 using namespace ptx;
 
-constexpr int kEpiWarps = 8;                 // epilogue warps 2 .. 9
-constexpr int kThreads = 64 + 32 * kEpiWarps;  // warp 0: TMA producer, warp 1: MMA issuer
+__host__ __device__ constexpr int epi_warps(int kind, int S) { return kind != 3 && S == 8 ? 12 : 16; }  // epilogue warps from 2 on
+__host__ __device__ constexpr int threads_of(int kind, int S) {  // warp 0: TMA producer, warp 1: MMA issuer
+  return 64 + 32 * epi_warps(kind, S);
+}
 constexpr int MT = 128;          // rows per tile
-constexpr int NT = 48;           // columns per tile
 constexpr int NT3 = 32;          // columns per tile of the inverse's trailing updates (KIND 3)
 constexpr int KS = 32;           // K elements per stage (64-byte rows, 64-byte swizzle)
 constexpr int kStages = 2;
-constexpr int S = kRsSlices;     // 9 slices
-constexpr int NACC = 10;         // accumulators d = 2 .. 11
 constexpr int ROWB = KS * 2;     // 64 bytes
 constexpr int LSL = MT * ROWB;   // one left slice in a stage: 8 KB
-constexpr int RSL = NT * ROWB;   // one right slice: 3 KB (2 KB for KIND 3, packed the same way)
-constexpr int LBYTES = S * LSL;  // 72 KB
-constexpr int RBYTES = (S + 1) * RSL;  // 30 KB with the zero slice
-constexpr int STAGE = LBYTES + RBYTES;
-constexpr int STG = 32 * 9;                  // an epilogue warp's 32 x 9 float64 staging tile
-constexpr int SMEM = 1024 + kStages * STAGE + kEpiWarps * STG * 8;
+constexpr int STG = 32 * 8;                  // an epilogue warp's 32 x 8 float64 staging tile
 constexpr uint32_t kCols = 512;
 constexpr uint32_t kSbo = 8 * ROWB;  // 512-byte swizzle atoms
 constexpr uint64_t kLayout = 4;       // 64-byte swizzle
+
+// columns per tile
+constexpr int nt_of(int kind, int S) { return kind == 3 ? NT3 : S == 7 ? 64 : 48; }
+// bytes of a stage and of the kernel's shared memory
+template <int KIND, int S>
+constexpr int stage_bytes() {
+  return S * (LSL + nt_of(KIND, S) * ROWB);
+}
+template <int KIND, int S>
+constexpr int smem_bytes() {
+  return 1024 + kStages * stage_bytes<KIND, S>() + epi_warps(KIND, S) * STG * 8;
+}
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, int w,
                                             uint64_t* bar) {
@@ -78,30 +85,9 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm,
       : "memory");
 }
 
-// The integer value of an integer-valued float32 |v| < 2^22: v + 1.5 2^23
-// lies in [2^23, 2^24), where the float's low mantissa bits are v's.
+// The integer value of an integer-valued float32 |v| <= 2^22: v + 1.5 2^23
+// lies in [2^23, 2^24], where the float's low mantissa bits are v's.
 __device__ __forceinline__ int acc_int_small(float v) { return __float_as_int(v + 12582912.0f) - 0x4B400000; }
-
-// The integer value of an integer-valued float32 |v| < 2^24 from its bits.
-__device__ __forceinline__ int acc_int(uint32_t b) {
-  const uint32_t u = b & 0x7fffffffu;
-  const uint32_t sh = min(150u - min(u >> 23, 150u), 31u);  // 23 - exponent; 31 for zero
-  const int mag = (int)(((u & 0x7fffffu) | 0x800000u) >> sh);
-  const int sg = (int)b >> 31;
-  return (mag ^ sg) - sg;
-}
-
-// x 2^s as a float64, built from the bits: exact for |x| < 2^53 when the
-// result is a normal number (the caller checks the exponent range).
-__device__ __forceinline__ double i2d_scaled(long long x, int s) {
-  const unsigned long long sg = (unsigned long long)x & 0x8000000000000000ull;
-  const unsigned long long a = (unsigned long long)(x < 0 ? -x : x);
-  const int lz = __clzll(a);                              // >= 11 for a < 2^53
-  const unsigned long long mant = a << ((lz - 11) & 63);  // leading bit at 52
-  // the leading bit adds one to the exponent field
-  const unsigned long long ex = (unsigned long long)(1022 + 63 - lz + s);
-  return a == 0 ? 0.0 : __longlong_as_double((long long)(sg | ((ex << 52) + mant)));
-}
 
 }  // namespace oz
 
@@ -124,8 +110,8 @@ namespace oz {
 // KIND 5 j = 0: HB -= C_q ZL^{j+1}[q+1], j = 1: HC = -C_q ZR^{j+1}[q+1]
 // (parts unused, out.seps instead).
 //
-// A tile = (subsystem or separator, product j, 128-row M-tile, 48-column
-// N-tile); tile = ((unit * 2 + j) * ntm + M-tile) * ntn + N-tile (KIND 3,
+// A tile = (subsystem or separator, product j, 128-row M-tile, N-tile
+// of nt_of columns); tile = ((unit * 2 + j) * ntm + M-tile) * ntn + N-tile (KIND 3,
 // one product: (unit * ntm + M-tile) * ntn + N-tile).
 struct OzTile {
   PartDesc p;
@@ -134,12 +120,7 @@ struct OzTile {
   bool act;
 };
 
-template <int KIND>
-constexpr int nt_of() {
-  return KIND == 3 ? NT3 : NT;
-}
-
-template <int KIND>
+template <int KIND, int S>
 __device__ __forceinline__ OzTile oz_tile(int tile, const PartDesc* __restrict__ parts, const OzOut& out, int step,
                                           int aux, int m, int ntm, int ntn) {
   OzTile w{};
@@ -181,7 +162,7 @@ __device__ __forceinline__ OzTile oz_tile(int tile, const PartDesc* __restrict__
   // products with a banded operand run in the banded kernels instead
   const bool banded = out.band && *out.band <= kBandMax;
   if (banded && ((KIND == 0 && j == 0) || KIND == 1 || KIND >= 4)) act = false;
-  w.act = act && w.tm * MT < m && w.tn * nt_of<KIND>() < m;
+  w.act = act && w.tm * MT < m && w.tn * nt_of(KIND, S) < m;
   const long long mm = (long long)m * m;
   const int b0 = (int)(p.blk / mm), t = w.t;
   if (KIND == 4) {
@@ -209,38 +190,42 @@ __device__ __forceinline__ OzTile oz_tile(int tile, const PartDesc* __restrict__
 // Persistent: a CTA per SM walks the tiles blockIdx.x, blockIdx.x + gridDim.x,
 // ...  Warp 0 (one lane) streams every tile's K slabs by TMA into a two-stage
 // ring and runs ahead into the next tile; warp 1 (one lane) issues the MMAs
-// of a tile once the epilogue has drained the accumulators of the previous
-// one (the ten accumulators take 480 of the 512 tensor-memory columns, so
-// there is one set); warps 2-9 run the epilogue, loading what it needs
-// besides the accumulators while the MMAs run.  Every wait is bounded; a
-// role that gives up sets `err`, which the others see at their next tile.
-template <int KIND>
-__global__ void __launch_bounds__(kThreads, 1)
+// of a tile once the epilogue has drained the accumulators they go to (KIND 3
+// has two sets, so its MMAs run beside the previous tile's epilogue; the
+// other kinds' accumulators fill the tensor memory); warps from 2 on run the
+// epilogue (KIND 3: two teams of eight, a set of accumulators each), loading
+// what it needs besides the accumulators while the MMAs run.  Every wait is bounded; a role that gives up sets `err`, which the
+// others see at their next tile.
+template <int KIND, int S>
+__global__ void __launch_bounds__(threads_of(KIND, S), 1)
     k_oz_step(const PartDesc* __restrict__ parts, int step, int aux, int m, int ntm, int ntn, int ntiles, OzOut out,
               const int* __restrict__ lexp, const int* __restrict__ rexp0, const int* __restrict__ rexp1,
               int* __restrict__ errflag, const __grid_constant__ OzMaps maps) {
-  constexpr int NTK = nt_of<KIND>();   // columns per tile
+  constexpr int kEpi = epi_warps(KIND, S);
+  constexpr int NTK = nt_of(KIND, S);   // columns per tile
+  constexpr int NACC = S + 1;            // accumulators d = 2 .. S + 2
   constexpr int RSLK = NTK * ROWB;      // one right slice in a stage
+  constexpr int LBYTES = S * LSL, STAGE = stage_bytes<KIND, S>();
+  constexpr int SETC = NACC * NTK;                         // tensor-memory columns of one set of accumulators
+  constexpr int NBUF = 2 * SETC <= (int)kCols ? 2 : 1;  // sets
+  constexpr int DB = S == 7 ? 8 : 7;                    // bits per digit
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ uint64_t full[kStages], empty[kStages], tfull, tempty, mdone;
+  __shared__ uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], mdone;
   __shared__ uint32_t tmem_slot;
   __shared__ int err, nissued, ncons;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   double* stage_out = reinterpret_cast<double*>(base + kStages * STAGE);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* verr = &err;
-  // the zero right slice of both stages (never written by the copies)
-  for (int st = 0; st < kStages; ++st)
-    for (int i = threadIdx.x; i < RSLK / 16; i += kThreads)
-      reinterpret_cast<uint4*>(base + st * STAGE + LBYTES + S * RSLK)[i] = make_uint4(0u, 0u, 0u, 0u);
-  fence_async_shared();
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(&tfull, 1);
-    mbar_init(&tempty, kEpiWarps);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&tfull[s], 1);
+      mbar_init(&tempty[s], kEpi / NBUF);
+    }
     mbar_init(&mdone, 1);
     err = 0;
     nissued = 0;
@@ -260,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       int it = 0;
       for (int tile = blockIdx.x; tile < ntiles && !*verr; tile += gridDim.x) {
-        const OzTile w = oz_tile<KIND>(tile, parts, out, step, aux, m, ntm, ntn);
+        const OzTile w = oz_tile<KIND, S>(tile, parts, out, step, aux, m, ntm, ntn);
         if (!w.act) continue;
         const CUtensorMap* mr = w.j == 0 ? &maps.R0 : &maps.R1;
         bool ok = true;
@@ -287,10 +272,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       int it = 0, lt = 0;
       for (int tile = blockIdx.x; tile < ntiles && !*verr; tile += gridDim.x) {
-        const OzTile w = oz_tile<KIND>(tile, parts, out, step, aux, m, ntm, ntn);
+        const OzTile w = oz_tile<KIND, S>(tile, parts, out, step, aux, m, ntm, ntn);
         if (!w.act) continue;
-        // the accumulators of the previous tile have been read
-        if (lt > 0 && !mbar_wait(&tempty, (uint32_t)((lt - 1) & 1))) {
+        // the accumulators of the tile that used this set before have been read
+        const int bf = lt % NBUF, use = lt / NBUF;
+        if (use > 0 && !mbar_wait(&tempty[bf], (uint32_t)((use - 1) & 1))) {
           *verr = 1;
           break;
         }
@@ -309,14 +295,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t off = (uint32_t)(k * 32);
 #pragma unroll
             for (int sl = 1; sl <= S; ++sl) {
-              const int T = sl == 1 ? S + 1 : min(S, 11 - sl);  // s = 1 runs into the zero slice
+              constexpr int per = 256 / NTK;  // right slices per instruction
+              const int T = min(S, S + 2 - sl);
               const uint64_t ad = kmajor_desc(la + (sl - 1) * LSL + off, kSbo, kLayout);
 #pragma unroll
-              for (int ta = 1; ta <= T; ta += 5) {
-                const int cnt = min(5, T - ta + 1);
+              for (int ta = 1, cnt = 0; ta <= T; ta += cnt) {
+                cnt = min(per, T - ta + 1);
+                if (sl == 2 && ta < S && ta + cnt > S) cnt = S - ta;  // (2, S) by itself
                 const uint64_t bd = kmajor_desc(ra + (ta - 1) * RSLK + off, kSbo, kLayout);
-                const uint32_t dcol = (uint32_t)((sl + ta - 2) * NTK);
-                const uint32_t acc = (s == 0 && k == 0 && sl == 1) ? 0u : 1u;
+                const uint32_t dcol = (uint32_t)(bf * SETC + (sl + ta - 2) * NTK);
+                const uint32_t acc = (s == 0 && k == 0 && (sl == 1 || (sl == 2 && ta == S))) ? 0u : 1u;
                 mma<1>(tmem + dcol, ad, bd, make_idesc(1u, MT, NTK * cnt), acc);
               }
             }
@@ -327,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           *verr = 1;
           break;
         }
-        mma_commit(&tfull);
+        mma_commit(&tfull[bf]);
         ++lt;
       }
       ncons = it;
@@ -337,29 +325,32 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    const int ew = warp - 2, quarter = warp & 3, half = ew >> 2;  // a warp reaches lanes 32 (warp % 4) ..
+    // a warp reaches tensor-memory lanes 32 (warp % 4) ..; the warps of a team
+    // that share a lane quarter share the tile's columns, CW each
+    constexpr int CW = NTK / (kEpi / NBUF / 4);
+    const int ew = warp - 2, quarter = warp & 3, team = NBUF == 2 ? ew >> 3 : 0, part = NBUF == 2 ? (ew >> 2) & 1 : ew >> 2;
     double* stg = stage_out + ew * STG;
-    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
     const int cl = lane & 7, r0 = lane >> 3;
     const int k0 = 32 * step;  // KIND 3: the panel's columns
     int lt = 0;
     for (int tile = blockIdx.x; tile < ntiles && !*verr; tile += gridDim.x) {
-      const OzTile w = oz_tile<KIND>(tile, parts, out, step, aux, m, ntm, ntn);
+      const OzTile w = oz_tile<KIND, S>(tile, parts, out, step, aux, m, ntm, ntn);
       if (!w.act) continue;
+      const int bf = lt % NBUF, use = lt / NBUF;
+      ++lt;
+      if (NBUF == 2 && bf != team) continue;
+      const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(bf * SETC);
       const int j = w.j, t = w.t, pidx = w.unit;
       const PartDesc& p = w.p;
       const SepDesc& sd = w.sd;
       const int* rexp = j == 0 ? rexp0 : rexp1;
       // Before the accumulators are ready: the row's scale, the column scales
-      // of the warp's 24 columns (one per lane, passed by shuffle) and the
+      // of the warp's columns (one per lane, passed by shuffle) and the
       // values the stores update (they do not depend on the products)
       const int rbase = w.tm * MT + quarter * 32, row = rbase + lane;
+      const int cbase = w.tn * NTK + part * CW;  // the warp's columns
       const int er = row < m ? lexp[(long long)w.zl * m + row] : 0;
-      int fexp = 0;
-      {
-        const int n = w.tn * NTK + half * (NTK / 2) + lane;
-        if (lane < NTK / 2 && n < m) fexp = rexp[(long long)w.zr * m + n];
-      }
+      const int fexp = lane < CW && cbase + lane < m ? rexp[(long long)w.zr * m + cbase + lane] : 0;
       const bool rmw = KIND == 2 && j == 0, dnext = KIND == 1 && j == 0, gj = KIND == 3, hb = KIND >= 4 && j == 0;
       const bool upd = rmw || dnext || gj || hb;
       const long long o = p.blk + (long long)t * mm;
@@ -369,143 +360,125 @@ __global__ void __launch_bounds__(kThreads, 1)
                           : gj   ? wk
                           : hb   ? (KIND == 4 ? out.B + sd.blk_q : out.HB + sd.hblk)
                                  : out.B + o + mm;
+      // where the results go
+      double* dst;
+      if (KIND >= 4)
+        dst = (j == 0 ? out.HB : KIND == 4 ? out.HA : out.HC) + sd.hblk;  // HB = B_q - A_q ZR, then HB -= C_q ZL;
+                                                                         // HA = -A_q ZL, HC = -C_q ZR
+      else if (KIND == 0)
+        dst = (j == 0 ? (t < p.L - 1 ? out.Acal : out.ZR) : out.ZL) + o;
+      else if (KIND == 1)
+        dst = j == 0 ? wk : out.Y + (long long)pidx * mm;  // D_{t+1} = B_{t+1} - A_{t+1} Acal_t, Y = -A_{t+1} Bcal_t
+      else if (KIND == 2)
+        dst = (j == 0 ? out.ZL : out.ZR) + o;  // ZL_t -= Acal_t ZL_{t+1}, ZR_t = -Acal_t ZR_{t+1}
+      else
+        dst = wk;                              // Gauss-Jordan trailing update
       // KIND 3: which of the warp's 32 rows are pivot rows of the panel
       uint32_t zrows = 0;
       if (KIND == 3) {
         const int pv = k0 + lane < m ? out.piv[(long long)pidx * m + k0 + lane] : -1;
         zrows = __reduce_or_sync(0xffffffffu, pv >= 0 && (pv >> 5) == (rbase >> 5) ? 1u << (pv & 31) : 0u);
       }
-      // the values chunk ci's stores update, loaded one chunk ahead
+      // the values chunk ci's stores update, loaded before its accumulators are converted
       auto load_in = [&](int ci, double (&in)[8]) {
-        const int n = w.tn * NTK + half * (NTK / 2) + 8 * ci + cl;
-        const bool outside = KIND != 3 || n < k0 || n >= k0 + 32;
+        const int n = cbase + 8 * ci + cl;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int rr = rbase + r0 + 4 * i;
-          in[i] = (upd && n < m && outside && rr < m && !(gj && ((zrows >> (r0 + 4 * i)) & 1u)))
-                      ? src[(long long)rr * m + n]
-                      : 0.0;
+          in[i] = (upd && n < m && rr < m && !(gj && ((zrows >> (r0 + 4 * i)) & 1u))) ? src[(long long)rr * m + n]
+                                                                                      : 0.0;
         }
       };
-      double incur[8], innext[8];
-      load_in(0, incur);
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull, (uint32_t)(lt & 1)));
+      double in[8];
+      load_in(0, in);
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull[bf], (uint32_t)(use & 1)));
       if (!ok) {
         *verr = 1;
         break;
       }
       tc_fence_after();
       // Accumulators of this thread's row (tensor-memory lane) for 8 columns
-      // at a time.  Each acc_d is an integer-valued float below 2^24: its
-      // integer comes from the float's bits (float32 and integer operations),
-      // pairs P_j = acc_{2j+2} 64 + acc_{2j+3} are exact in 32 bits, and
-      //   hi = P_0 2^12 + P_1 (< 2^39),  lo = (P_2 2^12 + P_3) 2^12 + P_4 (< 2^53)
-      // give the sum exactly as hi 2^36 + lo.  Both become float64 from their
-      // bits with the scale 2^(e_r + f_n - 66) in the exponent, and one
-      // float64 add rounds their sum once (one issue slot; rounding the
-      // 128-bit sum in integer arithmetic measured slower).  Warps of the
-      // same lane quarter share the tile's columns.  Results are staged
-      // through the warp's 32 x 9 float64 tile so that row-major writes are
-      // coalesced.
-      // acc_d below 2^22 for every d (then the float32 magic-number
-      // conversion is exact): K = 32, or K = m <= 112 (acc_d <= 9 K 63^2)
-      const bool small = KIND == 3 || m <= 112;
-#pragma unroll
-      for (int ci = 0; ci < NTK / 16; ++ci) {
-        const int ch = half * (NTK / 2) + 8 * ci;
-        // chunks past the block's last column, and (KIND 3) inside the
-        // panel's columns, produce nothing: only the release of the
-        // accumulators after the last chunk remains
-        const int c0n = w.tn * NTK + ch;
-        const bool dead = c0n >= m || (KIND == 3 && c0n >= k0 && c0n < k0 + 32);
+      // at a time.  Each acc_d is an integer-valued float of at most 2^24 (its
+      // integer by float32 or conversion instructions); with b the digits'
+      // base,
+      //   S = 7: hi = (acc_2 b + acc_3) b + acc_4, lo the other five (< 2^56),
+      //   S = 8: hi = ((acc_2 b + acc_3) b + acc_4) b + acc_5, lo the other five (< 2^53)
+      // give the sum exactly as hi b^5 + lo.  It is rounded to a 64-bit integer
+      // T (at 2^-57 (S = 7; KIND 3: 2^-59), 2^-55 (S = 8) of 2^(e_r + f_n + 2), below the
+      // operands' own rounding) and T to float64, both in integer
+      // instructions: a float64 instruction holds its warp for 64 cycles, so
+      // only the addition of an updated value is one.  Results are staged
+      // through the warp's 32 x 8 float64 tile so that row-major writes are
+      // coalesced.  The chunk loop stays rolled: unrolled, a launch of few
+      // tiles waited for its instructions.
+#pragma unroll 1
+      for (int ci = 0; ci < CW / 8; ++ci) {
+        const int ch = part * CW + 8 * ci;
+        // chunks past the block's last column produce nothing: only the
+        // release of the accumulators after the last chunk remains
+        const bool dead = cbase + 8 * ci >= m, last = ci == CW / 8 - 1;
         if (dead) {
-          if (ci == NTK / 16 - 1) {
+          if (last) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty);
-          } else {
-            load_in(ci + 1, innext);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) incur[i] = innext[i];
+            if (lane == 0) mbar_arrive(&tempty[bf]);
           }
           continue;
         }
+        if (ci > 0) load_in(ci, in);
         uint32_t r[NACC][8];
 #pragma unroll
         for (int dd = 0; dd < NACC; ++dd) tmem_ld8_nowait(tl + (uint32_t)(dd * NTK + ch), r[dd]);
         tmem_wait_ld();
 #pragma unroll
         for (int dd = 0; dd < NACC; ++dd) tmem_regs_after_wait(r[dd]);
-        if (ci == NTK / 16 - 1) {  // the last accumulator read of this tile: the MMAs may go on
+        if (last) {  // the last accumulator read of this tile: the MMAs may go on
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&tempty);
-        } else {
-          load_in(ci + 1, innext);
+          if (lane == 0) mbar_arrive(&tempty[bf]);
         }
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          const int n = w.tn * NTK + ch + c;
-          const int k = er + __shfl_sync(0xffffffffu, fexp, 8 * ci + c);
+          const int k = er + __shfl_sync(0xffffffffu, fexp, 8 * ci + c) + 2;
+          // |acc_d| <= (d - 1) K b^2 / 4, at most 2^22 for K = 32 always, else
+          // for the first two
           int a[NACC];
 #pragma unroll
           for (int dd = 0; dd < NACC; ++dd)
-            a[dd] = (dd < 4 || small) ? acc_int_small(__uint_as_float(r[dd][c])) : acc_int(r[dd][c]);
-          const long long hi = (long long)(a[0] * 64 + a[1]) * 4096 + (a[2] * 64 + a[3]);
-          const long long lo =
-              ((long long)(a[4] * 64 + a[5]) * 4096 + (a[6] * 64 + a[7])) * 4096 + (a[8] * 64 + a[9]);
-          double val = 0.0;
-          const bool kept = KIND != 3 || n < k0 || n >= k0 + 32;  // KIND 3: not the panel's columns
-          if (row < m && n < m && kept) {
-            const float a2 = __uint_as_float(r[0][c]);
-            if (a2 != a2)  // NaN or infinite operand: every digit is NaN, acc_2 included
-              val = __longlong_as_double(0x7ff8000000000000ll);
-            else if ((hi | lo) == 0)  // also the zero rows and columns, whose scale is the smallest
-              val = 0.0;
-            else if (k - 66 >= -1022 && k + 9 <= 1023)
-              val = i2d_scaled(hi, k - 30) + i2d_scaled(lo, k - 66);
-            else
-              val = ldexp(fma((double)lo, 0x1p-36, (double)hi), k - 30);
+            a[dd] = KIND == 3 || dd < 2 ? acc_int_small(__uint_as_float(r[dd][c]))
+                                        : __float2int_rn(__uint_as_float(r[dd][c]));
+          long long hi, lo;
+          if (S == 7) {
+            hi = (long long)a[0] * 65536 + (a[1] * 256 + a[2]);
+            lo = (((long long)a[3] * 256 + a[4]) * 256 + a[5]) * 65536 + ((long long)a[6] * 256 + a[7]);
+          } else {
+            hi = (long long)(a[0] * 128 + a[1]) * 16384 + (a[2] * 128 + a[3]);
+            lo = (long long)(a[4] * 128 + a[5]) * 2097152 + (long long)(a[6] * 128 + a[7]) * 128 + a[NACC - 1];
           }
-          stg[lane * 9 + c] = val;
+          // |hi| < 2^35 (KIND 3), 2^38 (S = 7), 2^42 (S = 8): T = (hi b^5 + lo) / 2^drop below 2^63
+          constexpr int ulo = DB * (S + 2), drop = KIND == 3 ? 13 : 15, up = 5 * DB - drop;
+          const long long T = hi * (1ll << up) + ((lo + (1 << (drop - 1))) >> drop);
+          bool odd = false;
+          double val = round_scaled(T, k - ulo + drop, odd);
+          const float a2 = __uint_as_float(r[0][c]);
+          if (odd || a2 != a2)  // outside the normal range; NaN or infinite operand: its first digit is NaN, so acc_2 is
+            val = a2 != a2 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp((double)T, k - ulo + drop);
+          stg[lane * 8 + (c ^ (lane & 7))] = val;
         }
         __syncwarp();
         // row-major float64 results: lane = (row quarter, column), 8 row quads
-        const int n = w.tn * NTK + ch + cl;
-        const bool outside = KIND != 3 || n < k0 || n >= k0 + 32;
-        if (n < m && outside) {
+        const int n = cbase + 8 * ci + cl;
+        if (n < m) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const int rl = r0 + 4 * i, rr = rbase + rl;
             if (rr >= m) continue;
-            const double v = stg[rl * 9 + cl];
-            const long long e = (long long)rr * m + n;
-            if (KIND >= 4) {
-              if (j == 0)
-                out.HB[sd.hblk + e] = incur[i] - v;               // HB = B_q - A_q ZR, then HB -= C_q ZL
-              else
-                (KIND == 4 ? out.HA : out.HC)[sd.hblk + e] = -v;  // HA = -A_q ZL, HC = -C_q ZR
-            } else if (KIND == 0) {
-              double* d = (j == 0) ? (t < p.L - 1 ? out.Acal : out.ZR) : out.ZL;
-              d[o + e] = v;
-            } else if (dnext) {
-              wk[e] = incur[i] - v;                                // D_{t+1} = B_{t+1} - A_{t+1} Acal_t
-            } else if (KIND == 1) {
-              out.Y[(long long)pidx * mm + e] = -v;                // Y_{t+1} = -A_{t+1} Bcal_t
-            } else if (rmw) {
-              out.ZL[o + e] = incur[i] - v;                        // ZL_t -= Acal_t ZL_{t+1}
-            } else if (gj) {
-              wk[e] = incur[i] + v;                                // Gauss-Jordan trailing update
-            } else {
-              out.ZR[o + e] = -v;                                  // ZR_t = -Acal_t ZR_{t+1}
-            }
+            const double v = stg[rl * 8 + (cl ^ (rl & 7))];
+            dst[(long long)rr * m + n] = gj ? in[i] + v : upd ? in[i] - v : KIND == 0 ? v : -v;
           }
         }
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 8; ++i) incur[i] = innext[i];
       }
-      ++lt;
     }
   }
   __syncthreads();
@@ -523,12 +496,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 // operands) of one float64 m x m block; a block takes ceil(m / 32) CTAs.
 
 // Row slices (left operands): exps[r] = e with |v| < 2^e for the row's
-// largest |v|; slice s element (r, k) at (q * 9 + s) m^2 + r m + k.  One
-// warp per row, eight consecutive columns per lane (m % 8 == 0).
+// largest |v|; slice s element (r, k) at ((q * S + s) m + r) pitch + k, the
+// pitch m rounded up to 8 (16-byte rows for TMA; the columns past m are zero).
+// One warp per row, eight consecutive columns per lane.
+template <int S>
 __device__ __forceinline__ void slice_rows_group(const double* __restrict__ src, __nv_bfloat16* __restrict__ dst,
                                                  long long qdst, int* __restrict__ exps, int m, int g) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const long long mm = (long long)m * m;
+  const int mp = slice_pitch(m);
   const unsigned long long* bits = reinterpret_cast<const unsigned long long*>(src);
   const int rend = min(m, 32 * g + 32);
   for (int r = 32 * g + warp; r < rend; r += nw) {
@@ -541,7 +516,7 @@ __device__ __forceinline__ void slice_rows_group(const double* __restrict__ src,
     for (int c0 = lane * 8; c0 < m; c0 += 256) {
       uint32_t q[8][S];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) digits9(bits[(long long)r * m + c0 + u], e, q[u]);
+      for (int u = 0; u < 8; ++u) digits<S>(c0 + u < m ? bits[(long long)r * m + c0 + u] : 0ull, e, q[u]);
 #pragma unroll
       for (int sl = 0; sl < S; ++sl) {
         uint4 w;
@@ -549,21 +524,22 @@ __device__ __forceinline__ void slice_rows_group(const double* __restrict__ src,
         w.y = (q[2][sl] >> 16) | (q[3][sl] & 0xffff0000u);
         w.z = (q[4][sl] >> 16) | (q[5][sl] & 0xffff0000u);
         w.w = (q[6][sl] >> 16) | (q[7][sl] & 0xffff0000u);
-        *reinterpret_cast<uint4*>(dst + (qdst * S + sl) * mm + (long long)r * m + c0) = w;
+        *reinterpret_cast<uint4*>(dst + ((qdst * S + sl) * m + r) * mp + c0) = w;
       }
     }
   }
 }
 
 // Column slices, transposed (right operands): exps[n] for column n, slice s
-// element (n, k) = digit s of src[k][n] at (q * 9 + s) m^2 + n m + k.  The
+// element (n, k) = digit s of src[k][n] at ((q * S + s) m + n) pitch + k.  The
 // group's 32 column maxima first (eight warps over the rows), then 32 x 32
 // tiles through shared memory; a thread writes four consecutive k of one n
 // per slice (8-byte stores).  256 threads.
+template <int S>
 __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src, __nv_bfloat16* __restrict__ dst,
                                                  long long qdst, int* __restrict__ exps, int m, int g,
                                                  uint32_t (*red)[32], int* s_e, unsigned long long (*tile)[33]) {
-  const long long mm = (long long)m * m;
+  const int mp = slice_pitch(m);
   const unsigned long long* bits = reinterpret_cast<const unsigned long long*>(src);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = 32 * g + lane;
@@ -589,16 +565,16 @@ __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src,
     }
     __syncthreads();
     const int nn = 32 * g + nl, k = k0 + kq;
-    if (nn < m && k < m) {  // m % 8 == 0: four consecutive k are all inside
+    if (nn < m && k < mp) {  // past m the tile holds zeros
       uint32_t q[4][S];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) digits9(tile[kq + u][nl], s_e[nl], q[u]);
+      for (int u = 0; u < 4; ++u) digits<S>(tile[kq + u][nl], s_e[nl], q[u]);
 #pragma unroll
       for (int sl = 0; sl < S; ++sl) {
         uint2 w;
         w.x = (q[0][sl] >> 16) | (q[1][sl] & 0xffff0000u);
         w.y = (q[2][sl] >> 16) | (q[3][sl] & 0xffff0000u);
-        *reinterpret_cast<uint2*>(dst + (qdst * S + sl) * mm + (long long)nn * m + k) = w;
+        *reinterpret_cast<uint2*>(dst + ((qdst * S + sl) * m + nn) * mp + k) = w;
       }
     }
     __syncthreads();
@@ -609,7 +585,7 @@ __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src,
 // columns): blockIdx.x = block * groups + group, looping past the grid.
 // With `band` set and the level's A and C banded (*band <= kBandMax), nothing
 // is done: only the tensor-core tiles the banded kernels replace read these.
-template <bool COLS>
+template <bool COLS, int S>
 __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__ src, int nblocks, int m,
                                                       __nv_bfloat16* __restrict__ dst, int* __restrict__ exps,
                                                       const int* __restrict__ band) {
@@ -622,9 +598,9 @@ __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__
   for (long long i = blockIdx.x; i < (long long)nblocks * groups; i += gridDim.x) {
     const int q = (int)(i / groups), g = (int)(i - (long long)q * groups);
     if (COLS)
-      slice_cols_group(src + q * mm, dst, q, exps, m, g, red, s_e, tile);
+      slice_cols_group<S>(src + q * mm, dst, q, exps, m, g, red, s_e, tile);
     else
-      slice_rows_group(src + q * mm, dst, q, exps, m, g);
+      slice_rows_group<S>(src + q * mm, dst, q, exps, m, g);
     __syncthreads();
   }
 }
@@ -636,6 +612,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__
 //   6 ZL_t columns, backward step;        7 ZR_t columns, backward step;
 //   8 Y_0 = A_first columns -> rolling (q), at the start of a factorisation.
 // Several per-subsystem slicing jobs in one launch (blockIdx.y = job).
+template <int S>
 __global__ void __launch_bounds__(256) k_oz_slice_jobs(const PartDesc* __restrict__ parts, int step, int m,
                                                        OzSliceJobs jobs) {
   __shared__ uint32_t red[8][32];
@@ -667,15 +644,16 @@ __global__ void __launch_bounds__(256) k_oz_slice_jobs(const PartDesc* __restric
   if (!act) return;
   __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(jb.dst);
   if (jb.kind == 0 || jb.kind == 1)
-    slice_rows_group(jb.src + sblk * mm, dst, dq, jb.exps, m, g);
+    slice_rows_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g);
   else
-    slice_cols_group(jb.src + sblk * mm, dst, dq, jb.exps, m, g, red, s_e, tile);
+    slice_cols_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g, red, s_e, tile);
 }
 
 // The assembly's operands per separator s (blockIdx.x = s * groups + group,
 // blockIdx.y = job): job 0 C_q rows -> Cq slot s; jobs 1-4 the boundary
 // spike blocks as columns -> S slot 4 s + job - 1: ZR^j[q-1], ZL^j[q-1] (only
 // with HA), ZL^{j+1}[q+1], ZR^{j+1}[q+1] (only with HC).
+template <int S>
 __global__ void __launch_bounds__(256) k_oz_slice_seps(const SepDesc* __restrict__ seps, int m,
                                                        const double* __restrict__ C, const double* __restrict__ ZL,
                                                        const double* __restrict__ ZR, __nv_bfloat16* __restrict__ Cq,
@@ -689,13 +667,13 @@ __global__ void __launch_bounds__(256) k_oz_slice_seps(const SepDesc* __restrict
   const int s = blockIdx.x / groups, g = blockIdx.x - s * groups, job = blockIdx.y;
   const SepDesc sd = seps[s];
   if (job == 0) {
-    slice_rows_group(C + sd.blk_q, Cq, s, eCq, m, g);
+    slice_rows_group<S>(C + sd.blk_q, Cq, s, eCq, m, g);
     return;
   }
   if ((job == 2 && !(sd.flags & HAS_HA)) || (job == 4 && !(sd.flags & HAS_HC))) return;
   const double* src = job == 1 ? ZR + sd.blk_prev : job == 2 ? ZL + sd.blk_prev : job == 3 ? ZL + sd.blk_next
                                                                                          : ZR + sd.blk_next;
-  slice_cols_group(src, Sp, 4LL * s + job - 1, eS, m, g, red, s_e, tile);
+  slice_cols_group<S>(src, Sp, 4LL * s + job - 1, eS, m, g, red, s_e, tile);
 }
 
 // ---------------------------------------------------------------- banded operands
@@ -713,7 +691,7 @@ __global__ void __launch_bounds__(256) k_band_gc(const PartDesc* __restrict__ pa
                                                  const double* __restrict__ G, const double* __restrict__ C,
                                                  double* __restrict__ Acal, double* __restrict__ ZR,
                                                  const int* __restrict__ band) {
-  __shared__ double bd[2 * kBandMax + 1][kMaxMTensor];  // bd[d + w][n] = C[n + d][n]
+  extern __shared__ double bd[];  // bd[(d + w) m + n] = C[n + d][n]
   const int w = *band;
   if (w > kBandMax) return;
   const int groups = (m + 31) / 32;
@@ -726,7 +704,7 @@ __global__ void __launch_bounds__(256) k_band_gc(const PartDesc* __restrict__ pa
   double* X = (t < p.L - 1 ? Acal : ZR) + o;
   for (int i = threadIdx.x; i < (2 * w + 1) * m; i += blockDim.x) {
     const int dd = i / m, n = i - dd * m, k = n + dd - w;
-    bd[dd][n] = (k >= 0 && k < m) ? Ct[(long long)k * m + n] : 0.0;
+    bd[i] = (k >= 0 && k < m) ? Ct[(long long)k * m + n] : 0.0;
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -735,7 +713,7 @@ __global__ void __launch_bounds__(256) k_band_gc(const PartDesc* __restrict__ pa
       double acc = 0.0;
       for (int d = -w; d <= w; ++d) {
         const int k = n + d;
-        if (k >= 0 && k < m) acc = fma(Gt[(long long)r * m + k], bd[d + w][n], acc);
+        if (k >= 0 && k < m) acc = fma(Gt[(long long)r * m + k], bd[(d + w) * m + n], acc);
       }
       X[(long long)r * m + n] = acc;
     }
@@ -867,18 +845,22 @@ EncodeFn oz_encoder() {
 
 bool oz_eligible(int m) { return m >= 8 && m <= kMaxMTensor && m % 8 == 0; }
 
-int oz_slice_blocks_bytes(int m) { return oz::S * m * m * 2; }
+int oz_slices(int m) { return m <= 128 ? 7 : 8; }
+
+int oz_slice_blocks_bytes(int m) { return oz_slices(m) * m * slice_pitch(m) * 2; }
 
 // 4-D map [block][slice][row][column] of a slice array (rows x kdim per
-// slice; kdim = m for the sweeps' blocks, 32 for the inversion's panels),
-// box 32 x box_rows x 9 x 1.
+// slice, rows `pitch` elements apart; kdim = m for the sweeps' blocks, 32 for
+// the inversion's panels),
+// box 32 x box_rows x slices x 1.
 bool oz_make_map(const void* base, long long blocks, int m, int box_rows, void* out, int kdim) {
   EncodeFn enc = oz_encoder();
   if (kdim <= 0) kdim = m;
+  const int S = oz_slices(kdim), pitch = slice_pitch(kdim);
   if (!enc || blocks <= 0 || !oz_eligible(m)) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)kdim, (cuuint64_t)m, (cuuint64_t)oz::S, (cuuint64_t)blocks};
-  cuuint64_t strides[3] = {(cuuint64_t)kdim * 2, (cuuint64_t)m * kdim * 2, (cuuint64_t)oz::S * m * kdim * 2};
-  cuuint32_t box[4] = {(cuuint32_t)oz::KS, (cuuint32_t)box_rows, (cuuint32_t)oz::S, 1u};
+  cuuint64_t dims[4] = {(cuuint64_t)kdim, (cuuint64_t)m, (cuuint64_t)S, (cuuint64_t)blocks};
+  cuuint64_t strides[3] = {(cuuint64_t)pitch * 2, (cuuint64_t)m * pitch * 2, (cuuint64_t)S * m * pitch * 2};
+  cuuint32_t box[4] = {(cuuint32_t)oz::KS, (cuuint32_t)box_rows, (cuuint32_t)S, 1u};
   cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
   CUresult r = enc(static_cast<CUtensorMap*>(out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
@@ -887,7 +869,7 @@ bool oz_make_map(const void* base, long long blocks, int m, int box_rows, void* 
 }
 
 int oz_box_rows_left() { return oz::MT; }
-int oz_box_rows_right() { return oz::NT; }
+int oz_box_rows_right(int m) { return oz::nt_of(0, oz_slices(m)); }
 int oz_box_rows_gj() { return oz::NT3; }
 
 void launch_band_detect(const double* A, const double* C, long long n, int m, int* band, cudaStream_t st) {
@@ -900,16 +882,22 @@ void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void*
   if (nblocks <= 0) return;
   const long long work = (long long)nblocks * ((m + 31) / 32);
   const int grid = (int)std::min<long long>(work, 152LL * 16);
-  if (cols)
-    oz::k_oz_slice_all<true><<<grid, 256, 0, st>>>(src, nblocks, m, static_cast<__nv_bfloat16*>(dst), exps, band);
-  else
-    oz::k_oz_slice_all<false><<<grid, 256, 0, st>>>(src, nblocks, m, static_cast<__nv_bfloat16*>(dst), exps, band);
+  auto* d = static_cast<__nv_bfloat16*>(dst);
+  const bool s7 = oz_slices(m) == 7;
+  if (cols && s7) oz::k_oz_slice_all<true, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
+  else if (cols) oz::k_oz_slice_all<true, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
+  else if (s7) oz::k_oz_slice_all<false, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
+  else oz::k_oz_slice_all<false, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
 }
 
 void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, const OzSliceJobs& jobs, int njobs,
                           cudaStream_t st) {
   if (nparts <= 0 || njobs <= 0) return;
-  oz::k_oz_slice_jobs<<<dim3(nparts * ((m + 31) / 32), njobs), 256, 0, st>>>(parts, step, m, jobs);
+  const dim3 grid(nparts * ((m + 31) / 32), njobs);
+  if (oz_slices(m) == 7)
+    oz::k_oz_slice_jobs<7><<<grid, 256, 0, st>>>(parts, step, m, jobs);
+  else
+    oz::k_oz_slice_jobs<8><<<grid, 256, 0, st>>>(parts, step, m, jobs);
 }
 
 // The trailing update of one panel of the blocked inversion (dm_gj.cu).
@@ -938,26 +926,33 @@ void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m
   }
   // KIND 3: 32-column tiles without the one that is the panel itself
   const int ntm = (m + oz::MT - 1) / oz::MT,
-            ntn = kind == 3 ? (m + oz::NT3 - 1) / oz::NT3 - 1 : (m + oz::NT - 1) / oz::NT;
+            ntn = kind == 3 ? (m + oz::NT3 - 1) / oz::NT3 - 1 : (m + oz_box_rows_right(m) - 1) / oz_box_rows_right(m);
   const int ntiles = nparts * (kind == 3 ? 1 : 2) * ntm * ntn;
   if (ntiles <= 0) return;
   const int grid = std::min(ntiles, nsm);
-#define DM_OZ(KIND_)                                                                                              \
-  do {                                                                                                           \
-    static bool set = false;                                                                                     \
-    if (!set) {                                                                                                  \
-      cudaFuncSetAttribute(oz::k_oz_step<KIND_>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM);        \
-      set = true;                                                                                                \
-    }                                                                                                            \
-    oz::k_oz_step<KIND_><<<grid, oz::kThreads, oz::SMEM, st>>>(parts, step, aux, m, ntm, ntn, ntiles, out, lexp, \
-                                                               rexp0, rexp1, errflag, mp);                       \
+#define DM_OZ(KIND_, S_)                                                                                          \
+  do {                                                                                                            \
+    static bool set = false;                                                                                      \
+    constexpr int smem = oz::smem_bytes<KIND_, S_>();                                                             \
+    if (!set) {                                                                                                   \
+      cudaFuncSetAttribute(oz::k_oz_step<KIND_, S_>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);          \
+      set = true;                                                                                                 \
+    }                                                                                                             \
+    oz::k_oz_step<KIND_, S_><<<grid, oz::threads_of(KIND_, S_), smem, st>>>(parts, step, aux, m, ntm, ntn, ntiles, out, lexp,  \
+                                                               rexp0, rexp1, errflag, mp);                        \
   } while (0)
-  if (kind == 0) DM_OZ(0);
-  else if (kind == 1) DM_OZ(1);
-  else if (kind == 2) DM_OZ(2);
-  else if (kind == 3) DM_OZ(3);
-  else if (kind == 4) DM_OZ(4);
-  else DM_OZ(5);
+  const bool s7 = oz_slices(m) == 7;
+  if (kind == 3) DM_OZ(3, 7);  // K = 32
+  else if (kind == 0 && s7) DM_OZ(0, 7);
+  else if (kind == 0) DM_OZ(0, 8);
+  else if (kind == 1 && s7) DM_OZ(1, 7);
+  else if (kind == 1) DM_OZ(1, 8);
+  else if (kind == 2 && s7) DM_OZ(2, 7);
+  else if (kind == 2) DM_OZ(2, 8);
+  else if (kind == 4 && s7) DM_OZ(4, 7);
+  else if (kind == 4) DM_OZ(4, 8);
+  else if (s7) DM_OZ(5, 7);
+  else DM_OZ(5, 8);
 #undef DM_OZ
 }
 
@@ -965,8 +960,12 @@ void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, 
                         const double* ZR, double* HA, double* HB, double* HC, const OzAsm& a, const int* eA,
                         const void* mapA, int* errflag, const int* band, cudaStream_t st) {
   if (nseps <= 0) return;
-  oz::k_oz_slice_seps<<<dim3(nseps * ((m + 31) / 32), 5), 256, 0, st>>>(
-      seps, m, C, ZL, ZR, static_cast<__nv_bfloat16*>(a.Cq), a.eCq, static_cast<__nv_bfloat16*>(a.S), a.eS, band);
+  const dim3 sgrid(nseps * ((m + 31) / 32), 5);
+  auto *cq = static_cast<__nv_bfloat16*>(a.Cq), *sp = static_cast<__nv_bfloat16*>(a.S);
+  if (oz_slices(m) == 7)
+    oz::k_oz_slice_seps<7><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, band);
+  else
+    oz::k_oz_slice_seps<8><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, band);
   OzOut out{};
   out.B = B;
   out.seps = seps;
@@ -986,7 +985,13 @@ void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, 
 void launch_band_gc(const PartDesc* parts, int nparts, int t, int m, const double* G, const double* C, double* Acal,
                     double* ZR, const int* band, cudaStream_t st) {
   if (nparts <= 0 || !band) return;
-  oz::k_band_gc<<<nparts * ((m + 31) / 32), 256, 0, st>>>(parts, t, m, G, C, Acal, ZR, band);
+  static bool set = false;
+  if (!set) {
+    cudaFuncSetAttribute(oz::k_band_gc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (2 * kBandMax + 1) * kMaxM * (int)sizeof(double));
+    set = true;
+  }
+  oz::k_band_gc<<<nparts * ((m + 31) / 32), 256, (2 * kBandMax + 1) * m * sizeof(double), st>>>(parts, t, m, G, C, Acal, ZR, band);
 }
 
 void launch_band_b(const PartDesc* parts, int nparts, int t, int m, const double* A, const double* B,

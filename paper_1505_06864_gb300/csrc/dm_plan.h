@@ -86,9 +86,9 @@ struct Tc2Level {
   alignas(64) unsigned char maps[8][128];
 };
 
-// Digit slices of a float64 level with one block size m (m % 8 == 0,
-// m <= 256) for the products on the tensor cores (dm_oz.cu): nine bf16
-// slices per block ([block][slice][row][column]) and one exponent per row
+// Digit slices of a float64 level with one block size m for the products on
+// the tensor cores (dm_oz.cu): oz_slices(m) bf16 slices per block
+// ([block][slice][row][column], rows of slice_pitch(m)) and one exponent per row
 // ([block][m] ints).  Full copies: A (rows), C^T (columns of C), Acal (rows);
 // rolling, per subsystem: G_t (rows), Acal_t^T, Y_t^T, and two slots each of
 // ZL^T, ZR^T (columns); Y: Y_{t+1} per subsystem in float64.
@@ -102,7 +102,7 @@ struct OzLevel {
   // tensor maps: left G, A, Acal; right CT, YT, AcalT, ZLT, ZRT
   alignas(64) unsigned char maps[8][128];
   // blocked Gauss-Jordan inversion: the working matrix per subsystem, panel
-  // slices U, V ([subsystem][9][m][32]), their exponents, the pivot rows, and
+  // slices U, V ([subsystem][7][m][32]), their exponents, the pivot rows, and
   // the two panel maps
   bool gj = false;
   double* W = nullptr;

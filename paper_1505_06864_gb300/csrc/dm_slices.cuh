@@ -48,28 +48,66 @@ __device__ __forceinline__ void digits9(unsigned long long bits, int e, uint32_t
 
 constexpr int kBalSlices = 7;
 
-// Seven balanced base-256 digits of v, |v| < 2^e: v = 2^(e+1) sum_{s=1..7}
-// d_s 2^(-8s), rounded to the nearest multiple of 2^(e-55), every d_s an
-// integer in [-128, 128] and so exact in bf16 (bit patterns in the high half
-// of each word, as digits9).  The scaled integer is biased by 128 in every
-// byte, so that each digit is one byte minus 128.  v must be finite.
-__device__ __forceinline__ void digits7(unsigned long long bits, int e, uint32_t (&q)[kBalSlices]) {
+// Row pitch (elements) of the slices of an m x m block: 16-byte rows.
+__host__ __device__ constexpr int slice_pitch(int m) { return (m + 7) & ~7; }
+
+// v 2^(55 - e) rounded to the nearest integer (halves away from zero), |v| < 2^e.
+__device__ __forceinline__ long long scaled_integer(unsigned long long bits, int e) {
   const int ex = (int)((bits >> 52) & 0x7ff);
   const unsigned long long mant = (bits & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
   const int sh = (ex ? ex : 1) - 1075 + 55 - e;  // <= 2 for |v| < 2^e
   const int dn = min(-sh, 60);
   const unsigned long long Y = sh >= 0 ? (mant << (sh & 63)) : ((mant + (1ull << (dn - 1))) >> dn);
-  const unsigned long long Z = ((bits >> 63) ? 0ull - Y : Y) + 0x0080808080808080ull;
-  const uint32_t hi = (uint32_t)(Z >> 32), lo = (uint32_t)Z;
-  const uint32_t w[kBalSlices] = {0x4b000000u | (hi >> 16),
-                                  __byte_perm(hi, 0x4b000000u, 0x7541),
-                                  __byte_perm(hi, 0x4b000000u, 0x7540),
-                                  __byte_perm(lo, 0x4b000000u, 0x7543),
-                                  __byte_perm(lo, 0x4b000000u, 0x7542),
-                                  __byte_perm(lo, 0x4b000000u, 0x7541),
-                                  __byte_perm(lo, 0x4b000000u, 0x7540)};
+  return (long long)((bits >> 63) ? 0ull - Y : Y);
+}
+
+// S balanced digits of v, |v| < 2^e, in base 2^8 (S = 7) or 2^7 (S = 8):
+// v = 2^(e+1) sum_{s=1..S} d_s base^(-s), rounded to the nearest multiple of
+// 2^(e-55), every d_s an integer of at most base / 2 in magnitude and so exact
+// in bf16 (bit patterns in the high half of each word, as digits9).  The
+// scaled integer is biased by base / 2 in every digit, so that each digit is a
+// bit field minus base / 2.  NaN or infinity: the first digit is NaN, the
+// others finite.
+template <int S>
+__device__ __forceinline__ void digits(unsigned long long bits, int e, uint32_t (&q)[S]) {
+  static_assert(S == 7 || S == 8, "base 2^8 or 2^7");
+  const long long Y = scaled_integer(bits, e);
+  if constexpr (S == 7) {
+    const unsigned long long Z = (unsigned long long)Y + 0x0080808080808080ull;
+    const uint32_t hi = (uint32_t)(Z >> 32), lo = (uint32_t)Z;
+    const uint32_t w[7] = {0x4b000000u | (hi >> 16),
+                           __byte_perm(hi, 0x4b000000u, 0x7541),
+                           __byte_perm(hi, 0x4b000000u, 0x7540),
+                           __byte_perm(lo, 0x4b000000u, 0x7543),
+                           __byte_perm(lo, 0x4b000000u, 0x7542),
+                           __byte_perm(lo, 0x4b000000u, 0x7541),
+                           __byte_perm(lo, 0x4b000000u, 0x7540)};
 #pragma unroll
-  for (int k = 0; k < kBalSlices; ++k) q[k] = __float_as_uint(__uint_as_float(w[k]) - 8388736.0f);
+    for (int k = 0; k < 7; ++k) q[k] = __float_as_uint(__uint_as_float(w[k]) - 8388736.0f);
+  } else {
+    const unsigned long long Z = (unsigned long long)Y + 0x0081020408102040ull;  // 64 in every 7-bit digit
+    const uint32_t hi = (uint32_t)(Z >> 32), lo = (uint32_t)Z;
+    const uint32_t mid = __funnelshift_r(lo, hi, 28);  // bits 28 .. 59
+    const uint32_t w[8] = {hi >> 17,          (hi >> 10) & 127u, (hi >> 3) & 127u, (mid >> 0) & 127u,
+                           (lo >> 21) & 127u, (lo >> 14) & 127u, (lo >> 7) & 127u, lo & 127u};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) q[k] = __float_as_uint(__uint_as_float(0x4b000000u | w[k]) - 8388672.0f);
+  }
+  if ((bits >> 52 & 0x7ff) == 0x7ff) q[0] = 0x7fc00000u;
+}
+
+// T 2^s rounded to float64 (to nearest, halves up), |T| < 2^63, by integer
+// operations; `odd` is set when the result is outside the normal range (then
+// the value is not the result).
+__device__ __forceinline__ double round_scaled(long long T, int s, bool& odd) {
+  const unsigned long long a = (unsigned long long)(T < 0 ? -T : T);
+  const int lz = __clzll(a);
+  const unsigned long long an = a << (lz & 63);                   // leading bit at 63
+  const unsigned long long mant = (an >> 11) + ((an >> 10) & 1);  // leading bit at 52 (or 2^53)
+  const int ex = 1022 + 63 - lz + s;                              // the leading bit adds one to the exponent
+  odd = odd || (a != 0 && (unsigned)ex > 2044u);
+  const unsigned long long r = ((unsigned long long)T & 0x8000000000000000ull) + ((unsigned long long)ex << 52) + mant;
+  return __longlong_as_double(a == 0 ? 0ll : (long long)r);
 }
 
 // Two bf16 values (high halves of a and b) in one register, a first.
