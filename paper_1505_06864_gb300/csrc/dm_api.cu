@@ -299,7 +299,7 @@ static bool tc2_wanted(const Level& L) {
 }
 
 // Float64 products by digit slicing on the tensor cores: float64 levels
-// with one block size m % 8 == 0, m <= 256, unless the plan asked for the
+// with one block size m >= 16, unless the plan asked for the
 // FP64 pipe (DM_PLAN_FP64_FMA) or DM_FP64_PRODUCTS=fma is set.
 static bool oz_wanted(const Level& L) {
   const char* e = std::getenv("DM_FP64_PRODUCTS");
@@ -1138,15 +1138,26 @@ int Plan::init(const std::vector<SysSpec>& specs, int prec) {
   top.lazy_inputs = true;
   top.fp64_fma = !specs.empty() && (specs[0].flags & DM_PLAN_FP64_FMA) != 0;
   top.inv_column = !specs.empty() && (specs[0].flags & DM_PLAN_FP64_INV_COLUMN) != 0;
-  int rc = top.build(specs, prec != DM_FP64, prec == DM_TF32 ? 0 : (prec == DM_BF16X3 ? 1 : -1));
+  const int tmode = prec == DM_TF32 ? 0 : (prec == DM_BF16X3 ? 1 : -1);
+  int rc = top.build(specs, prec != DM_FP64, tmode);
   if (rc) return rc;
   {
     // admission: refuse cleanly, before allocating anything, when the device
     // lacks the plan's footprint plus a reserve
     size_t free_b = 0, total_b = 0;
     DM_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    const size_t need = top.bytes_needed() - 3 * top.nblk * sizeof(double) + 2 * top.nvec * sizeof(double);
+    auto footprint = [&] {
+      return top.bytes_needed() - 3 * top.nblk * sizeof(double) + 2 * top.nvec * sizeof(double);
+    };
+    size_t need = footprint();
     const size_t reserve = std::min<size_t>(total_b / 64, size_t(1) << 30);
+    if (need + reserve > free_b && !top.f32 && !top.fp64_fma && (top.max_m % 8 != 0 || top.max_m > kMaxMTensor)) {
+      // the digit slices about double a float64 plan's footprint: block sizes
+      // that have the float64 pipe's kernels as an equal in kind keep fitting
+      top.fp64_fma = true;
+      if ((rc = top.build(specs, prec != DM_FP64, tmode))) return rc;
+      need = footprint();
+    }
     if (need + reserve > free_b)
       return set_error(DM_ENOMEM, "admission refused: plan needs %zu bytes, %zu free (reserve %zu)", need, free_b,
                        reserve);

@@ -843,7 +843,10 @@ EncodeFn oz_encoder() {
 }
 }  // namespace
 
-bool oz_eligible(int m) { return m >= 8 && m <= kMaxMTensor && m % 8 == 0; }
+// From m = 16 on (float64 pipe / sliced, factor + solve of N = 511: m = 8 1143
+// / 1332 us, 12 1494 / 1675, 16 1851 / 1756, 24 2616 / 2058, 100 18.0 / 6.5 ms,
+// 200 97 / 18 ms; N = 127, m = 400 221 / 44 ms, 512 327 / 62 ms).
+bool oz_eligible(int m) { return m >= 16 && m <= kMaxM; }
 
 int oz_slices(int m) { return m <= 128 ? 7 : 8; }
 

@@ -39,7 +39,11 @@ def permuted_system(N, m, r, seed):
 # rows (one to 256, two above)
 @pytest.mark.parametrize("N,m,r,P,levels", [(9, 8, 1, 2, 1), (9, 24, 2, 3, 1), (9, 40, 1, 2, 1), (12, 64, 3, 3, 1),
                                             (9, 128, 1, 3, 1), (7, 136, 2, 2, 1), (7, 248, 1, 2, 1),
-                                            (7, 256, 1, 3, 1)])
+                                            (7, 256, 1, 3, 1),
+                                            # no multiples of 8 (padded slice rows, narrow last panels), above 256
+                                            (9, 9, 1, 2, 1), (12, 31, 3, 3, 1), (9, 33, 1, 2, 1), (9, 100, 2, 3, 1),
+                                            (9, 129, 1, 2, 1), (7, 201, 2, 3, 1), (7, 257, 1, 2, 1),
+                                            (7, 400, 2, 3, 1), (5, 511, 1, 2, 1), (5, 512, 1, 2, 1)])
 def test_every_pivot_exchanged(dm, N, m, r, P, levels):
     s = permuted_system(N, m, r, m + N)
     plan = dm.dm_plan(N, m, r, P, levels, "fp64")
@@ -53,3 +57,24 @@ def test_every_pivot_exchanged(dm, N, m, r, P, levels):
     assert np.all(np.isfinite(x))
     assert np.all(np.max(np.abs(x - xref), axis=(0, 1)) <= TOL * np.max(np.abs(xref), axis=(0, 1)))
     assert o.rel_err(x, xref) <= TOL
+
+
+def test_plan_without_room_for_slices_keeps_the_float64_pipe(dm):
+    """A float64 plan with m % 8 != 0 whose digit slices do not fit is planned without them."""
+    import torch
+    N, m = 2500, 100
+    entries = N * m * m
+    plan = dm.dm_plan(N, m, 1, 16, 1, "fp64")
+    sliced = dm.dm_plan_query(plan)["device_bytes"]
+    dm.dm_destroy(plan)
+    assert sliced > 70 * entries  # factors 32, slices 44 bytes per entry of a block
+    free, _ = torch.cuda.mem_get_info()
+    reserve = 1 << 30  # what dm_plan leaves free
+    hold = torch.empty(free - reserve - 55 * entries, dtype=torch.uint8, device="cuda")
+    try:
+        plan = dm.dm_plan(N, m, 1, 16, 1, "fp64")
+        assert dm.dm_plan_query(plan)["device_bytes"] < 40 * entries
+        dm.dm_destroy(plan)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
