@@ -62,7 +62,8 @@ extern "C" {
 /* How the residual r = b - T x is computed (dm_set_residual). */
 #define DM_RESIDUAL_FP64 0   /* float64 fused multiply-adds on the CUDA cores */
 #define DM_RESIDUAL_SLICED 1 /* exact bf16 slice products on the tensor cores, float64-accurate */
-#define DM_RESIDUAL_AUTO 2   /* SLICED for the systems where it is faster (m^2 nrhs >= 2^17), else FP64 */
+#define DM_RESIDUAL_AUTO 2   /* SLICED for the systems where it is faster (m nrhs >= 128; below 32 block rows
+                                m^2 nrhs >= 2^17), else FP64 */
 
 typedef struct dm_plan_s* dm_plan_t;
 
@@ -365,15 +366,15 @@ int dm_set_refinement(dm_plan_t plan, double tol, int max_iters); /* default 1e-
 /* Residual method (the paper has none: it stops at the direct solve; the
  * refinement of the mixed precisions needs r = b - T x in float64 accuracy).
  * DM_RESIDUAL_SLICED cuts every float64 entry of a block row [A_i B_i C_i]
- * and of [x_{i-1}; x_i; x_{i+1}] into nine 6-bit digits scaled by the row's
- * (column's) largest power of two, multiplies digit matrices exactly on the
- * bf16 tensor cores (integer partial sums below 2^24 in float32), and sums
- * the digit products in float64: error per entry below
+ * and of [x_{i-1}; x_i; x_{i+1}] into seven balanced base-256 digits scaled by
+ * the row's (column's) largest power of two, multiplies digit matrices exactly
+ * on the bf16 tensor cores (integer sums of at most 2^24 in float32), and sums
+ * the digit products in 64-bit integers: error per entry below
  * 3m 2^-50 max|row of [A B C]| max|column of x|, the float64 dot product's own
  * bound.  It serves systems with m <= 128 and nrhs <= 16; the others of the
  * plan use DM_RESIDUAL_FP64.  DM_RESIDUAL_AUTO picks SLICED per system where
- * it measured faster on GB300 (m^2 nrhs >= 2^17: m = 128 with nrhs >= 8,
- * m = 96 with nrhs >= 15): the float64 kernel's cost grows with nrhs, the
+ * it measured faster on GB300 (m nrhs >= 128; systems of fewer than 32 block
+ * rows: m^2 nrhs >= 2^17): the float64 kernel's cost grows with nrhs, the
  * sliced kernel's mostly with m^2.  Default: AUTO for DM_FP32 / DM_TF32 /
  * DM_BF16X3 plans, FP64 for DM_FP64 plans.  DM_EINVAL for other modes. */
 int dm_set_residual(dm_plan_t plan, int mode);

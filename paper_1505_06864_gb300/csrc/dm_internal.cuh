@@ -44,7 +44,8 @@ struct SysDesc {
   long long blk, vec;  // offsets of row 0
   int N, m, r;
   int row0;            // first row of the system when the rows of all systems are numbered consecutively
-  int sliced;          // residual on the tensor cores (k_residual_sliced) instead of float64 CUDA cores
+  int sliced;          // residual on the tensor cores (k_residual_digits) instead of float64 CUDA cores
+  int cta0[2];         // that kernel's first CTA of the system, per class of r (to 8, to 16 columns)
   int eoff;            // offset of the system's rows in the per-row scale arrays (sum of N m before it)
 };
 
@@ -99,6 +100,8 @@ void launch_residual(const SysDesc* sys, int nsys, int nrows, int max_m, int max
 // Residual b - T x of the systems with SysDesc::sliced set, float64-accurate
 // from exact bf16 slice products on the tensor cores (m <= 128, r <= 16).
 bool residual_sliced_fits(int m, int r);
+int residual_sliced_class(int r);         // 0: r <= 8, 1: r <= 16
+int residual_sliced_ctas(int N, int m);   // CTAs of one system
 // Per point row of the sliced systems: the largest high word (sign cleared)
 // of the row of [A_i B_i C_i] -- computed once per factorisation.
 void launch_row_scales(const SysDesc* sys, int nsys, int nrows, const double* A, const double* B,
@@ -106,9 +109,9 @@ void launch_row_scales(const SysDesc* sys, int nsys, int nrows, const double* A,
 // Per block row of the sliced systems: the largest high word of each column
 // of x_i ([global block row][16]), before each sliced residual.
 void launch_col_scales(const SysDesc* sys, int nsys, int nrows, const double* x, unsigned* colhi, cudaStream_t st);
-void launch_residual_sliced(const SysDesc* sys, int nsys, int nrows, const double* A, const double* B,
+void launch_residual_sliced(const SysDesc* sys, int nsys, const int (&ctas)[2], const double* A, const double* B,
                             const double* C, const double* x, const double* b, double* r, double* nrm,
-                            const unsigned* rowhi, const unsigned* colhi, int* errflag, cudaStream_t st);
+                            const unsigned* rowhi, const unsigned* colhi, cudaStream_t st);
 void launch_axpy_norms(const SysDesc* sys, int nsys, int nrows, int max_m, int max_r, const double* d,
                        double* x, double* nrm, cudaStream_t st);
 

@@ -153,6 +153,7 @@ struct Level {
   Cost c_asm_h, c_asm_f, c_backsub, c_resid, c_axpy, c_sepcopy;
   Cost c_resid_tc;     // the part of c_resid computed by the tensor-core residual
   int nres_tc = 0;     // systems whose residual runs on the tensor cores
+  int res_ctas[2] = {0, 0};  // CTAs of that residual's two kernels
   PartDesc* d_parts = nullptr;
   SepDesc* d_seps = nullptr;
   SysDesc* d_sys = nullptr;
@@ -224,7 +225,6 @@ struct Plan {
   int set_residual_mode(int mode);
   // r = b - T x (float64-accurate) with the column norms into nrm; all device pointers
   void residual(const double* x_dev, const double* b_dev, double* r_dev);
-  int check_residual_error();
   template <typename F>
   int run(GraphCache& g, F&& body);
 
