@@ -18,6 +18,7 @@
 #include <climits>
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <string>
@@ -1135,11 +1136,13 @@ __global__ void __launch_bounds__(kThreads) k_backsub(const PartDesc* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// Narrow products for right-hand sides (r <= 16 columns): one output row per
-// thread.  Each thread streams its row of the m x m block from global memory
-// (every load brings a whole line into L1, so a warp keeps 32 lines in flight
-// and the following k hit L1) against the panel R ([m][RB] in shared memory,
-// read as broadcasts); no cross-lane reduction.  RB is the CTA's own column
+// Narrow products for right-hand sides (r <= 16 columns): eight lanes per
+// output row, so that a row of the m x m block is read in whole 128-byte lines
+// (16-byte loads where the block's address and m allow them), against the
+// panel R (in shared memory), one to four rows per lane.  (One row per thread left every line to L1, which a full SM's
+// rows overflow: four times the L2 traffic, 865 us for the back-substitution
+// of N = 2048, m = 256, r = 1 in float64.)  A CTA takes 32 rows or a multiple,
+// several CTAs one block where a launch has few.  RB is the CTA's own column
 // bucket (1, 2, 4, 8 or 16 >= its r), so a batch with mixed right-hand-side
 // counts spends no multiply-add on another system's padding.
 __host__ __device__ constexpr int rbucket(int r) { return r <= 1 ? 1 : r <= 2 ? 2 : r <= 4 ? 4 : r <= 8 ? 8 : 16; }
@@ -1155,40 +1158,161 @@ __device__ __forceinline__ void with_rb(int r, F&& f) {
   if constexpr (RM >= 16) f(std::integral_constant<int, 16>());
 }
 
-template <typename T, typename TL1, typename TL2, int RB, typename Epi>
-__device__ __forceinline__ void rows_mm(int m, const TL1* __restrict__ L1, const T* __restrict__ R1,
-                                        const TL2* __restrict__ L2, const T* __restrict__ R2, Epi epi) {
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    T acc[RB];
+constexpr int kDotLanes = 8;
+constexpr int kDotRows = 256 / kDotLanes;  // row groups of a CTA
+
+// Rows per lane: a panel entry read from shared memory serves that many rows
+// (with one row, eight columns in float32 were bound by those reads).
+template <typename T, int RB>
+constexpr int dot_rt() {
+  return RB <= 2 ? RB : RB * (int)sizeof(T) <= 64 ? 4 : 2;
+}
+
+// Row pitch of a panel in shared memory (column-major [RB][pitch], so that the
+// eight lanes of a row read 128 consecutive bytes of a column).
+__host__ __device__ constexpr int dot_pitch(int m) { return (m + 3) & ~3; }
+
+// 16-byte loads of L's rows are possible (m in whole vectors, address aligned)
+template <typename TL>
+__device__ __forceinline__ bool dot_vec(const TL* L, int m) {
+  return (m * (int)sizeof(TL)) % 16 == 0 && (reinterpret_cast<uintptr_t>(L) & 15) == 0;
+}
+
+// acc[q][c] += this lane's part of sum_k L[i + 32 q][k] R[c][k], q < n (rows
+// of the block L): the lane takes every eighth vector (or entry) of a row.
+template <typename T, typename TL, int RB, int RT>
+__device__ __forceinline__ void dot_rows(const TL* __restrict__ L, const T* R, int m, int i, int n, int lane, bool vec,
+                                         T (&acc)[RT][RB]) {
+  const TL* l = L + (long long)i * m;
+  const long long rs = (long long)kDotRows * m;
+  const int ld = dot_pitch(m);
+  if (vec) {
+    constexpr int V = 16 / (int)sizeof(TL), U = RT >= 4 ? 2 : RT == 2 ? 4 : 8;  // vectors in flight per row
+    for (int k0 = lane * V; k0 < m; k0 += U * kDotLanes * V) {
+      uint4 qv[U][RT];
 #pragma unroll
-    for (int c = 0; c < RB; ++c) acc[c] = (T)0;
-    const TL1* l1 = L1 + (long long)i * m;
-#pragma unroll 4
-    for (int k = 0; k < m; ++k) {
-      const T lv = (T)l1[k];
+      for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int c = 0; c < RB; ++c) acc[c] = fma(lv, R1[k * RB + c], acc[c]);
-    }
-    if (L2 != nullptr) {
-      const TL2* l2 = L2 + (long long)i * m;
-#pragma unroll 4
-      for (int k = 0; k < m; ++k) {
-        const T lv = (T)l2[k];
+        for (int q = 0; q < RT; ++q) {
+          const int k = k0 + u * kDotLanes * V;
+          qv[u][q] = q < n && k < m ? __ldg(reinterpret_cast<const uint4*>(l + q * rs + k)) : make_uint4(0, 0, 0, 0);
+        }
 #pragma unroll
-        for (int c = 0; c < RB; ++c) acc[c] = fma(lv, R2[k * RB + c], acc[c]);
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * kDotLanes * V;
+        if (k < m)
+#pragma unroll
+          for (int c = 0; c < RB; ++c) {
+            T xv[V];
+            if constexpr (V * sizeof(T) == 16) {
+              const uint4 xq = *reinterpret_cast<const uint4*>(R + c * ld + k);
+              memcpy(xv, &xq, 16);
+            } else {
+              static_assert(V * sizeof(T) == 8, "float64 blocks times a float32 panel");
+              const uint2 xq = *reinterpret_cast<const uint2*>(R + c * ld + k);
+              memcpy(xv, &xq, 8);
+            }
+#pragma unroll
+            for (int q = 0; q < RT; ++q)
+              if (q < n) {
+                TL v[V];
+                memcpy(v, &qv[u][q], 16);
+#pragma unroll
+                for (int w = 0; w < V; ++w) acc[q][c] = fma((T)v[w], xv[w], acc[q][c]);
+              }
+          }
       }
     }
+  } else {
+#pragma unroll 2
+    for (int k = lane; k < m; k += kDotLanes) {
+      TL v[RT];
 #pragma unroll
-    for (int c = 0; c < RB; ++c) epi(i, c, acc[c]);
+      for (int q = 0; q < RT; ++q) v[q] = q < n ? __ldg(l + q * rs + k) : (TL)0;
+#pragma unroll
+      for (int q = 0; q < RT; ++q)
+        if (q < n)
+#pragma unroll
+          for (int c = 0; c < RB; ++c) acc[q][c] = fma((T)v[q], R[c * ld + k], acc[q][c]);
+    }
   }
 }
 
-// Rs[k][c] = src[k * r + c] for c < r, zero up to RB.
+// The lanes' parts of a row added up: each exchange halves the columns a lane
+// keeps, so RB columns cost RB - RB / 8 additions (not 3 RB).  The lane ends
+// with the sums of columns c0 .. c0 + max(1, RB / 8) - 1 in acc[0 ..]; of lanes
+// with the same columns the lowest has `mine` set.
+template <typename T, int RB>
+__device__ __forceinline__ void dot_sum(T (&acc)[RB], int lane, int& c0, bool& mine) {
+  c0 = 0;
+  mine = RB >= kDotLanes || lane < RB;
+  int n = RB;
+#pragma unroll
+  for (int w = 1; w < kDotLanes; w <<= 1) {
+    if (n > 1) {
+      n >>= 1;
+      const bool up = (lane & w) != 0;
+#pragma unroll
+      for (int c = 0; c < RB / 2; ++c)
+        if (c < n) {
+          const T send = up ? acc[c] : acc[c + n], keep = up ? acc[c + n] : acc[c];
+          acc[c] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+      if (up) c0 += n;
+    } else {
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], w);
+    }
+  }
+}
+
+// epi(i, c, sum_k L1[i][k] R1[c][k] + L2[i][k] R2[c][k]) for the rows lo <= i <
+// hi of an m x m block (L1 or L2 may be null); whole warps take part.
+template <typename T, typename TL1, typename TL2, int RB, int RT, typename Epi>
+__device__ __forceinline__ void rows_mm_rt(int m, int lo, int hi, const TL1* __restrict__ L1, const T* R1,
+                                           const TL2* __restrict__ L2, const T* R2, Epi epi) {
+  const int lane = threadIdx.x & (kDotLanes - 1), g = threadIdx.x / kDotLanes;
+  const bool v1 = L1 != nullptr && dot_vec(L1, m), v2 = L2 != nullptr && dot_vec(L2, m);
+  for (int i0 = lo; i0 < hi; i0 += kDotRows * RT) {
+    const int i = i0 + g, n = min(RT, (hi - i + kDotRows - 1) / kDotRows);  // rows i, i + 32, ..
+    T acc[RT][RB];
+#pragma unroll
+    for (int q = 0; q < RT; ++q)
+#pragma unroll
+      for (int c = 0; c < RB; ++c) acc[q][c] = (T)0;
+    if (n > 0) {
+      if (L1 != nullptr) dot_rows<T, TL1, RB, RT>(L1, R1, m, i, n, lane, v1, acc);
+      if (L2 != nullptr) dot_rows<T, TL2, RB, RT>(L2, R2, m, i, n, lane, v2, acc);
+    }
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+      if (i0 + kDotRows * q >= hi) break;  // the same for the whole CTA
+      int c0;
+      bool mine;
+      dot_sum<T, RB>(acc[q], lane, c0, mine);
+      if (q < n && mine)
+#pragma unroll
+        for (int c = 0; c < (RB + kDotLanes - 1) / kDotLanes; ++c) epi(i + kDotRows * q, c0 + c, acc[q][c]);
+    }
+  }
+}
+
+template <typename T, typename TL1, typename TL2, int RB, typename Epi>
+__device__ __forceinline__ void rows_mm(int m, int lo, int hi, const TL1* __restrict__ L1, const T* R1,
+                                        const TL2* __restrict__ L2, const T* R2, Epi epi) {
+  constexpr int RT = dot_rt<T, RB>();
+  if (RT > 1 && hi - lo <= kDotRows)  // a row per lane: more loads in flight
+    rows_mm_rt<T, TL1, TL2, RB, 1>(m, lo, hi, L1, R1, L2, R2, epi);
+  else
+    rows_mm_rt<T, TL1, TL2, RB, RT>(m, lo, hi, L1, R1, L2, R2, epi);
+}
+
+// Rs[c][k] = src[k * r + c] for c < r, zero up to RB (and up to the pitch).
 template <typename T, typename TS, int RB>
 __device__ __forceinline__ void load_narrow(T* Rs, const TS* __restrict__ src, int m, int r) {
-  for (int e = threadIdx.x; e < m * RB; e += blockDim.x) {
+  const int ld = dot_pitch(m);
+  for (int e = threadIdx.x; e < ld * RB; e += blockDim.x) {
     const int k = e / RB, c = e - k * RB;
-    Rs[e] = c < r ? (T)src[(long long)k * r + c] : (T)0;
+    Rs[c * ld + k] = c < r && k < m ? (T)src[(long long)k * r + c] : (T)0;
   }
 }
 
@@ -1370,7 +1494,8 @@ __global__ void __launch_bounds__(256) k_fwd_solve_n(const PartDesc* __restrict_
   with_rb<RM>(r, [&](auto rbc) {
     constexpr int RB = decltype(rbc)::value;
     T* Rs = reinterpret_cast<T*>(smem_raw);
-    T* Xs = Rs + m * RB;
+    const int ld = dot_pitch(m);
+    T* Xs = Rs + ld * RB;
     const long long mm = (long long)m * m, mr = (long long)m * r;
     const long long o = p.blk + (long long)t * mm, v = p.vec + (long long)t * mr;
     const double* Ft = F + v;
@@ -1379,14 +1504,14 @@ __global__ void __launch_bounds__(256) k_fwd_solve_n(const PartDesc* __restrict_
     } else {
       load_narrow<T, T, RB>(Xs, z + v - mr, m, r);
       __syncthreads();
-      rows_mm<T, double, double, RB>(m, A + o, Xs, (const double*)nullptr, (const T*)nullptr,
+      rows_mm<T, double, double, RB>(m, 0, m, A + o, Xs, (const double*)nullptr, (const T*)nullptr,
                                      [&](int row, int col, T val) {
-                                       Rs[row * RB + col] = col < r ? (T)Ft[(long long)row * r + col] - val : (T)0;
+                                       Rs[col * ld + row] = col < r ? (T)Ft[(long long)row * r + col] - val : (T)0;
                                      });
     }
     __syncthreads();
     T* dst = z + v;
-    rows_mm<T, T, T, RB>(m, G + o, Rs, (const T*)nullptr, (const T*)nullptr, [&](int row, int col, T val) {
+    rows_mm<T, T, T, RB>(m, 0, m, G + o, Rs, (const T*)nullptr, (const T*)nullptr, [&](int row, int col, T val) {
       if (col < r) dst[(long long)row * r + col] = val;
     });
   });
@@ -1408,7 +1533,7 @@ __global__ void __launch_bounds__(256) k_back_solve_n(const PartDesc* __restrict
     T* Y = z + v;
     load_narrow<T, T, RB>(Rs, Y + mr, m, r);
     __syncthreads();
-    rows_mm<T, T, T, RB>(m, Acal + o, Rs, (const T*)nullptr, (const T*)nullptr, [&](int row, int col, T val) {
+    rows_mm<T, T, T, RB>(m, 0, m, Acal + o, Rs, (const T*)nullptr, (const T*)nullptr, [&](int row, int col, T val) {
       if (col < r) {
         const long long e = (long long)row * r + col;
         Y[e] = Y[e] - val;
@@ -1425,17 +1550,19 @@ __global__ void __launch_bounds__(256) k_assemble_f_n(const SepDesc* __restrict_
                                                       const T* __restrict__ z, double* __restrict__ fh) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SepDesc sp = seps[blockIdx.x];
-  const int m = sp.m, r = sp.r;
+  const int m = sp.m, r = sp.r, lo = kDotRows * blockIdx.y;  // 32 rows per CTA
+  if (lo >= m) return;
   with_rb<RM>(r, [&](auto rbc) {
     constexpr int RB = decltype(rbc)::value;
     double* R1 = reinterpret_cast<double*>(smem_raw);
-    double* R2 = R1 + m * RB;
+    double* R2 = R1 + dot_pitch(m) * RB;
     load_narrow<double, T, RB>(R1, z + sp.vec_prev, m, r);
     load_narrow<double, T, RB>(R2, z + sp.vec_next, m, r);
     __syncthreads();
     const double* Fq = F + sp.vec_q;
     double* dst = fh + sp.hvec;
-    rows_mm<double, double, double, RB>(m, A + sp.blk_q, R1, C + sp.blk_q, R2, [&](int row, int col, double v) {
+    rows_mm<double, double, double, RB>(m, lo, min(m, lo + kDotRows), A + sp.blk_q, R1, C + sp.blk_q, R2,
+                                        [&](int row, int col, double v) {
       if (col < r) {
         const long long e = (long long)row * r + col;
         dst[e] = Fq[e] - v;
@@ -1444,23 +1571,23 @@ __global__ void __launch_bounds__(256) k_assemble_f_n(const SepDesc* __restrict_
   });
 }
 
-// Back-substitution for row t = blockIdx.x of subsystem blockIdx.y, in the
-// level's arithmetic (float32 levels: the spikes are float32, the products
+// Back-substitution for row t = blockIdx.x of subsystem blockIdx.y (rows
+// `chunk` blockIdx.z .. of the block), in the level's arithmetic (float32 levels: the spikes are float32, the products
 // too; x is written in float64).
 template <typename T, int RM>
 __global__ void __launch_bounds__(256) k_backsub_n(const PartDesc* __restrict__ parts,
                                                    const T* __restrict__ ZL, const T* __restrict__ ZR,
                                                    const T* __restrict__ z, const double* __restrict__ h,
-                                                   double* __restrict__ x) {
+                                                   double* __restrict__ x, int chunk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const PartDesc p = parts[blockIdx.y];
   const int t = blockIdx.x;
-  if (t >= p.L) return;
-  const int m = p.m, r = p.r;
+  const int m = p.m, r = p.r, lo = chunk * blockIdx.z, hi = min(m, lo + chunk);
+  if (t >= p.L || lo >= m) return;
   with_rb<RM>(r, [&](auto rbc) {
     constexpr int RB = decltype(rbc)::value;
     T* R1 = reinterpret_cast<T*>(smem_raw);
-    T* R2 = R1 + m * RB;
+    T* R2 = R1 + dot_pitch(m) * RB;
     const long long mm = (long long)m * m, mr = (long long)m * r;
     const long long o = p.blk + (long long)t * mm, v = p.vec + (long long)t * mr;
     const bool hl = p.flags & HAS_LEFT, hr = p.flags & HAS_RIGHT;
@@ -1476,13 +1603,13 @@ __global__ void __launch_bounds__(256) k_backsub_n(const PartDesc* __restrict__ 
       }
     };
     if (hl && hr) {
-      rows_mm<T, T, T, RB>(m, ZL + o, R1, ZR + o, R2, epi);
+      rows_mm<T, T, T, RB>(m, lo, hi, ZL + o, R1, ZR + o, R2, epi);
     } else if (hl) {
-      rows_mm<T, T, T, RB>(m, ZL + o, R1, (const T*)nullptr, (const T*)nullptr, epi);
+      rows_mm<T, T, T, RB>(m, lo, hi, ZL + o, R1, (const T*)nullptr, (const T*)nullptr, epi);
     } else if (hr) {
-      rows_mm<T, T, T, RB>(m, ZR + o, R2, (const T*)nullptr, (const T*)nullptr, epi);
+      rows_mm<T, T, T, RB>(m, lo, hi, ZR + o, R2, (const T*)nullptr, (const T*)nullptr, epi);
     } else {
-      for (long long e = threadIdx.x; e < mr; e += blockDim.x) xt[e] = (double)zt[e];
+      for (int e = lo * r + threadIdx.x; e < hi * r; e += blockDim.x) xt[e] = (double)zt[e];
     }
   });
 }
@@ -1497,8 +1624,8 @@ __global__ void k_sep_copy(const SepDesc* __restrict__ seps, const double* __res
 // ---------------------------------------------------------------------------
 // Residual r_i = b_i - A_i x_{i-1} - B_i x_i - C_i x_{i+1} in float64, one CTA
 // per block row of any system (rows of all systems numbered consecutively;
-// the CTA finds its system by binary search over their first rows).  One
-// output row per thread streaming the three block rows; x_{i-1}, x_i, x_{i+1}
+// the CTA finds its system by binary search over their first rows), `chunk`
+// point rows of it, as the narrow products above; x_{i-1}, x_i, x_{i+1}
 // staged in shared memory RB columns at a time (RB = the system's bucket).
 // Column sums of r^2 and b^2 go to nrm by atomics.
 __device__ __forceinline__ int find_sys(const SysDesc* __restrict__ sys, int nsys, int row) {
@@ -1519,7 +1646,7 @@ __global__ void __launch_bounds__(256) k_residual(const SysDesc* __restrict__ sy
                                                   const double* __restrict__ b,
                                                   double* __restrict__ rout,
                                                   double* __restrict__ nrm,
-                                                  const int* __restrict__ band) {
+                                                  const int* __restrict__ band, int chunk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[2 * kMaxR];
   // A and C banded (half-bandwidth w <= kBandMax, found by the factorisation
@@ -1527,72 +1654,83 @@ __global__ void __launch_bounds__(256) k_residual(const SysDesc* __restrict__ sy
   const int wb = band ? *band : kBandMax + 1;
   const int si = find_sys(sys, nsys, blockIdx.x);
   const SysDesc sd = sys[si];
-  if (sd.sliced) return;  // residual on the tensor cores (k_residual_sliced)
+  if (sd.sliced) return;  // residual on the tensor cores (k_residual_digits)
   const int i = blockIdx.x - sd.row0;
-  const int m = sd.m, r = sd.r;
+  const int m = sd.m, r = sd.r, lo = chunk * blockIdx.y, hi = min(m, lo + chunk);
+  if (lo >= m) return;
   const long long mm = (long long)m * m, mr = (long long)m * r;
   const long long o = sd.blk + i * mm, v = sd.vec + i * mr;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & (kDotLanes - 1), g = tid / kDotLanes;
   for (int e = tid; e < 2 * r; e += blockDim.x) red[e] = 0.0;
   const bool hasA = i > 0, hasC = i < sd.N - 1;
-  with_rb<RM>(r, [&](auto rbc) {
-    constexpr int RB = decltype(rbc)::value;
-    double* xs = reinterpret_cast<double*>(smem_raw);  // [3][m][RB]
+  const bool va = dot_vec(A + o, m), vb = dot_vec(B + o, m), vc = dot_vec(C + o, m);
+  auto run = [&](auto rbc, auto rtc) {
+    constexpr int RB = decltype(rbc)::value, RT = decltype(rtc)::value;
+    const int ld = dot_pitch(m);
+    double* xs = reinterpret_cast<double*>(smem_raw);  // [3][RB][ld]
     for (int c0 = 0; c0 < r; c0 += RB) {
       const int nc = min(RB, r - c0);
       __syncthreads();
-      for (int e = tid; e < 3 * m * RB; e += blockDim.x) {
-        const int which = e / (m * RB), rem = e - which * m * RB, k = rem / RB, c = rem - k * RB;
+      for (int e = tid; e < 3 * ld * RB; e += blockDim.x) {
+        const int which = e / (ld * RB), rem = e - which * ld * RB, k = rem / RB, c = rem - k * RB;
         const int row = i - 1 + which;
-        xs[e] = (row >= 0 && row < sd.N && c < nc) ? x[sd.vec + row * mr + (long long)k * r + c0 + c] : 0.0;
+        xs[(which * RB + c) * ld + k] = (row >= 0 && row < sd.N && c < nc && k < m) ? x[sd.vec + row * mr + (long long)k * r + c0 + c] : 0.0;
       }
       __syncthreads();
-      for (int row = tid; row < m; row += blockDim.x) {
-        double acc[RB];
+      for (int i0 = lo; i0 < hi; i0 += kDotRows * RT) {
+        const int row = i0 + g, n = min(RT, (hi - row + kDotRows - 1) / kDotRows);
+        double acc[RT][RB];
 #pragma unroll
-        for (int c = 0; c < RB; ++c) acc[c] = 0.0;
-        const double* ar = A + o + (long long)row * m;
-        const double* br = B + o + (long long)row * m;
-        const double* cr = C + o + (long long)row * m;
-        if (wb <= kBandMax) {
-#pragma unroll 2
-          for (int k = 0; k < m; ++k) {
-            const double bv = br[k];
-            const double* x0 = xs + (m + k) * RB;
+        for (int q = 0; q < RT; ++q)
 #pragma unroll
-            for (int c = 0; c < RB; ++c) acc[c] = fma(bv, x0[c], acc[c]);
-          }
-          for (int k = max(0, row - wb); k <= min(m - 1, row + wb); ++k) {
-            const double av = hasA ? ar[k] : 0.0, cv = hasC ? cr[k] : 0.0;
-            const double* xm = xs + k * RB;
-            const double* xp = xm + 2 * m * RB;
+          for (int c = 0; c < RB; ++c) acc[q][c] = 0.0;
+        if (n > 0) {
+          dot_rows<double, double, RB, RT>(B + o, xs + RB * ld, m, row, n, lane, vb, acc);
+          if (wb <= kBandMax) {
 #pragma unroll
-            for (int c = 0; c < RB; ++c) acc[c] = fma(av, xm[c], fma(cv, xp[c], acc[c]));
-          }
-        } else {
-#pragma unroll 2
-          for (int k = 0; k < m; ++k) {
-            const double av = hasA ? ar[k] : 0.0, bv = br[k], cv = hasC ? cr[k] : 0.0;
-            const double* xm = xs + k * RB;
-            const double* x0 = xm + m * RB;
-            const double* xp = x0 + m * RB;
+            for (int q = 0; q < RT; ++q) {
+              const int rq = row + kDotRows * q;
+              if (q < n)
+                for (int k = max(0, rq - wb) + lane; k <= min(m - 1, rq + wb); k += kDotLanes) {
+                  const double av = hasA ? A[o + (long long)rq * m + k] : 0.0, cv = hasC ? C[o + (long long)rq * m + k] : 0.0;
+                  const double* xm = xs + k;
+                  const double* xp = xm + 2 * RB * ld;
 #pragma unroll
-            for (int c = 0; c < RB; ++c) acc[c] = fma(av, xm[c], fma(bv, x0[c], fma(cv, xp[c], acc[c])));
+                  for (int c = 0; c < RB; ++c) acc[q][c] = fma(av, xm[c * ld], fma(cv, xp[c * ld], acc[q][c]));
+                }
+            }
+          } else {
+            if (hasA) dot_rows<double, double, RB, RT>(A + o, xs, m, row, n, lane, va, acc);
+            if (hasC) dot_rows<double, double, RB, RT>(C + o, xs + 2 * RB * ld, m, row, n, lane, vc, acc);
           }
         }
 #pragma unroll
-        for (int c = 0; c < RB; ++c) {
-          if (c < nc) {
-            const long long e = v + (long long)row * r + c0 + c;
-            const double bb = b[e];
-            const double rv = bb - acc[c];
-            rout[e] = rv;
-            atomicAdd(&red[c0 + c], rv * rv);
-            atomicAdd(&red[r + c0 + c], bb * bb);
-          }
+        for (int q = 0; q < RT; ++q) {
+          if (i0 + kDotRows * q >= hi) break;
+          int cl;
+          bool mine;
+          dot_sum<double, RB>(acc[q], lane, cl, mine);
+          if (q < n && mine)
+#pragma unroll
+            for (int c = 0; c < (RB + kDotLanes - 1) / kDotLanes; ++c)
+              if (cl + c < nc) {
+                const long long e = v + (long long)(row + kDotRows * q) * r + c0 + cl + c;
+                const double bb = b[e];
+                const double rv = bb - acc[q][c];
+                rout[e] = rv;
+                atomicAdd(&red[c0 + cl + c], rv * rv);
+                atomicAdd(&red[r + c0 + cl + c], bb * bb);
+              }
         }
       }
     }
+  };
+  with_rb<RM>(r, [&](auto rbc) {
+    constexpr int RT = dot_rt<double, decltype(rbc)::value>();
+    if (RT > 1 && hi - lo <= kDotRows)
+      run(rbc, std::integral_constant<int, 1>());
+    else
+      run(rbc, std::integral_constant<int, RT>());
   });
   __syncthreads();
   for (int c = tid; c < r; c += blockDim.x) {
@@ -1905,7 +2043,7 @@ void launch_fwd_solve(const PartDesc* parts, int nparts, int t, int max_m, int m
   if (nparts <= 0) return;
   if (narrow_dispatch(max_r, [&](auto rm) {
         constexpr int RM = decltype(rm)::value;
-        const size_t bytes = sizeof(T) * 2 * (size_t)max_m * RM;
+        const size_t bytes = sizeof(T) * 2 * (size_t)dot_pitch(max_m) * RM;
         allow_smem(k_fwd_solve_n<T, RM>, bytes);
         k_fwd_solve_n<T, RM><<<nparts, 256, bytes, st>>>(parts, t, A, G, F, z);
       }))
@@ -1929,7 +2067,7 @@ void launch_back_solve(const PartDesc* parts, int nparts, int s, int max_m, int 
   if (nparts <= 0) return;
   if (narrow_dispatch(max_r, [&](auto rm) {
         constexpr int RM = decltype(rm)::value;
-        const size_t bytes = sizeof(T) * (size_t)max_m * RM;
+        const size_t bytes = sizeof(T) * (size_t)dot_pitch(max_m) * RM;
         allow_smem(k_back_solve_n<T, RM>, bytes);
         k_back_solve_n<T, RM><<<nparts, 256, bytes, st>>>(parts, s, Acal, z);
       }))
@@ -2026,15 +2164,23 @@ void launch_assemble_h(const SepDesc* seps, int nseps, int max_m, const double* 
   }
 }
 
+// Rows per CTA of the narrow products over `blocks` blocks: 32 while that
+// leaves SMs idle, else up to 128 (the panel is loaded once per CTA).
+int dot_chunk(long long blocks, int max_m) {
+  int chunk = kDotRows;
+  while (chunk < 128 && blocks * ((max_m + chunk - 1) / chunk) > 8LL * device_sms()) chunk *= 2;
+  return chunk;
+}
+
 template <typename T>
 void launch_assemble_f(const SepDesc* seps, int nseps, int max_m, int max_r, const double* A,
                        const double* C, const double* F, const T* z, double* fh, cudaStream_t st) {
   if (nseps <= 0) return;
   if (narrow_dispatch(max_r, [&](auto rm) {
         constexpr int RM = decltype(rm)::value;
-        const size_t bytes = sizeof(double) * 2 * (size_t)max_m * RM;
+        const size_t bytes = sizeof(double) * 2 * (size_t)dot_pitch(max_m) * RM;
         allow_smem(k_assemble_f_n<T, RM>, bytes);
-        k_assemble_f_n<T, RM><<<nseps, 256, bytes, st>>>(seps, A, C, F, z, fh);
+        k_assemble_f_n<T, RM><<<dim3(nseps, (max_m + kDotRows - 1) / kDotRows), 256, bytes, st>>>(seps, A, C, F, z, fh);
       }))
     return;
   if (max_r <= 16) {
@@ -2056,9 +2202,11 @@ void launch_backsub(const PartDesc* parts, int nparts, int Lmax, int max_m, int 
   if (nparts <= 0 || Lmax <= 0) return;
   if (narrow_dispatch(max_r, [&](auto rm) {
         constexpr int RM = decltype(rm)::value;
-        const size_t bytes = sizeof(T) * 2 * (size_t)max_m * RM;
+        const size_t bytes = sizeof(T) * 2 * (size_t)dot_pitch(max_m) * RM;
         allow_smem(k_backsub_n<T, RM>, bytes);
-        k_backsub_n<T, RM><<<dim3(Lmax, nparts), 256, bytes, st>>>(parts, ZL, ZR, z, h, x);
+        const int chunk = dot_chunk((long long)Lmax * nparts, max_m);
+        k_backsub_n<T, RM><<<dim3(Lmax, nparts, (max_m + chunk - 1) / chunk), 256, bytes, st>>>(parts, ZL, ZR, z, h, x,
+                                                                                               chunk);
       }))
     return;
   if (max_r <= 16) {
@@ -2088,9 +2236,11 @@ void launch_residual(const SysDesc* sys, int nsys, int nrows, int max_m, int max
   if (nsys <= 0 || nrows <= 0) return;
   auto go = [&](auto rm) {
     constexpr int RM = decltype(rm)::value;
-    const size_t bytes = sizeof(double) * 3 * (size_t)max_m * RM;
+    const size_t bytes = sizeof(double) * 3 * (size_t)dot_pitch(max_m) * RM;
     allow_smem(k_residual<RM>, bytes);
-    k_residual<RM><<<nrows, 256, bytes, st>>>(sys, nsys, A, B, C, x, b, r, nrm, band);
+    const int chunk = dot_chunk(nrows, max_m);
+    k_residual<RM><<<dim3(nrows, (max_m + chunk - 1) / chunk), 256, bytes, st>>>(sys, nsys, A, B, C, x, b, r, nrm, band,
+                                                                                 chunk);
   };
   if (!narrow_dispatch(max_r, go)) go(std::integral_constant<int, 16>());
 }
