@@ -301,10 +301,21 @@ static bool tc2_wanted(const Level& L) {
 // Float64 products by digit slicing on the tensor cores: float64 levels
 // with one block size m >= 16, unless the plan asked for the
 // FP64 pipe (DM_PLAN_FP64_FMA) or DM_FP64_PRODUCTS=fma is set.
+static bool small_wanted(const Level& L);
+
 static bool oz_wanted(const Level& L) {
   const char* e = std::getenv("DM_FP64_PRODUCTS");
   return !L.f32 && !L.fp64_fma && !(e && std::strcmp(e, "fma") == 0) && uniform_m(L.spec, L.max_m) &&
-         oz_eligible(L.max_m);
+         oz_eligible(L.max_m) && !small_wanted(L);
+}
+
+// Small blocks: the whole factor sweep of a float64 level in one launch
+// (dm_small.cu), unless the plan asked for the float64-pipe step kernels or
+// the column inverse, or DM_SMALL_FACTOR=0 is set.
+static bool small_wanted(const Level& L) {
+  const char *e = std::getenv("DM_SMALL_FACTOR"), *f = std::getenv("DM_FP64_PRODUCTS"), *i = std::getenv("DM_FP64_INVERSE");
+  return !L.f32 && !L.fp64_fma && !L.inv_column && !(e && e[0] == '0') && !(f && std::strcmp(f, "fma") == 0) &&
+         !(i && std::strcmp(i, "cluster") == 0) && L.max_m <= kSmallM;
 }
 
 static size_t oz_bytes(long long nblk, int nparts, int nseps, int m) {
@@ -381,6 +392,24 @@ int Level::allocate() {
   DM_ALLOC(d_sys, std::max<size_t>(1, sysd.size()) * sizeof(SysDesc));
   DM_ALLOC(status, std::max(1, nsys) * sizeof(int));
   DM_ALLOC(d_err, sizeof(int));
+  // where the band of A and C is detected (unless DM_BANDED=0)
+  auto alloc_band = [&]() -> int {
+    OzLevel& Z = oz;
+    const char* eb = std::getenv("DM_BANDED");
+    if (!(eb && std::strcmp(eb, "0") == 0)) {
+      DM_ALLOC(Z.band, sizeof(int));
+      cudaMemset(Z.band, 0x7f, sizeof(int));  // "not banded" until a factorisation finds out
+      if (cudaHostAlloc(reinterpret_cast<void**>(&Z.band_host), sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(DM_ENOMEM, "cudaHostAlloc of 4 bytes failed");
+      }
+      *Z.band_host = kBandMax + 1;
+    }
+    return DM_OK;
+  };
+  small = small_wanted(*this);
+  // large enough that a band saves more than its detection costs
+  if (small && uniform_m(spec, max_m) && max_m >= 16 && (rc = alloc_band())) return rc;
   if (tc_mode >= 0 && tc2_wanted(*this)) {
     // operand copies and tensor maps of the tensor-core step kernels
     Tc2Level& T = tc2;
@@ -461,16 +490,7 @@ int Level::allocate() {
       if (!ok) return set_error(DM_ECUDA, "tensor map creation for the blocked inversion failed (m = %d)", m);
       Z.gj = true;
     }
-    const char* eb = std::getenv("DM_BANDED");
-    if (!(eb && std::strcmp(eb, "0") == 0)) {
-      DM_ALLOC(Z.band, sizeof(int));
-      cudaMemset(Z.band, 0x7f, sizeof(int));  // "not banded" until a factorisation finds out
-      if (cudaHostAlloc(reinterpret_cast<void**>(&Z.band_host), sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        return set_error(DM_ENOMEM, "cudaHostAlloc of 4 bytes failed");
-      }
-      *Z.band_host = kBandMax + 1;
-    }
+    if ((rc = alloc_band())) return rc;
     if (nseps > 0 && oz_asm_wanted()) {
       OzAsm& a = Z.as;
       DM_ALLOC(a.Cq, nseps * sl);
@@ -814,6 +834,31 @@ static void factor_level_t(Level& L, cudaStream_t st, Prof& pf, Aux* aux) {
   // With a side stream, the left-spike tiles of step t (type 1) run there,
   // overlapping the next inversion, which depends only on the type-0 tiles.
   if constexpr (std::is_same<T, double>::value) {
+    if (L.small) {
+      Cost c;
+      for (int t = 0; t < L.Lmax; ++t) {
+        c.flops += L.c_inv[t].flops + L.c_fwd[t].flops + L.c_back[t].flops;
+        c.bytes += L.c_inv[t].bytes + L.c_fwd[t].bytes + L.c_back[t].bytes;
+      }
+      // banded A and C (one block size): found before the sweep, used in it; the
+      // host's copy, of the factorisation before, names the profile class
+      const bool banded = L.oz.band && *L.oz.band_host <= kBandMax;
+      if (L.oz.band) {
+        Cost cd;
+        cd.bytes = 16.0 * L.nblk;
+        DM_LAUNCH(pf, st, K_TC_CONVERT, cd, 1,
+                  (cudaMemsetAsync(L.oz.band, 0, sizeof(int), st),
+                   launch_band_detect(L.A, L.C, L.nblk, L.max_m, L.oz.band, st),
+                   cudaMemcpyAsync(L.oz.band_host, L.oz.band, sizeof(int), cudaMemcpyDeviceToHost, st)));
+      }
+      DM_LAUNCH(pf, st, banded ? K_BANDED : K_FWD_FACTOR, c, L.nparts,
+                launch_small_factor(L.d_parts, L.nparts, L.A, L.B, L.C, G, Ac, ZL, ZR, L.status, L.oz.band, st));
+      if (L.supp)
+        DM_LAUNCH(pf, st, K_ASSEMBLE_H, L.c_asm_h, L.nseps,
+                  launch_assemble_h<T>(L.d_seps, L.nseps, L.max_m, L.A, L.B, L.C, ZL, ZR, L.supp->A, L.supp->B,
+                                       L.supp->C, st));
+      return;
+    }
     if (L.oz.on) {
       factor_level_oz(L, st, pf);
       if (L.supp && L.oz.asm_on) {

@@ -162,6 +162,11 @@ struct OzOut {
   const int* band;
 };
 constexpr int kBandMax = 6;
+// Factor sweeps of a float64 level with blocks of at most kSmallM in one
+// launch, a CTA per subsystem (dm_small.cu).
+constexpr int kSmallM = 32;
+void launch_small_factor(const PartDesc* parts, int nparts, const double* A, const double* B, const double* C, double* G,
+                         double* Acal, double* ZL, double* ZR, int* status, const int* band, cudaStream_t st);
 bool oz_eligible(int m);
 // digit slices per block (dm_slices.cuh): 7 (base 256) to m = 128, 8 (base 128) above
 int oz_slices(int m);

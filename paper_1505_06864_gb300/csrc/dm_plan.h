@@ -131,6 +131,7 @@ struct Level {
   bool has_tma = false;
   Tc2Level tc2;
   OzLevel oz;
+  bool small = false;  // the factor sweeps in one launch (dm_small.cu)
   bool fp64_fma = false;  // float64 products on the FP64 pipe even where digit slicing applies
   bool inv_column = false;  // the column-by-column float64 inverse even where the blocked one applies
   int nsys = 0;
