@@ -53,6 +53,11 @@ struct SysDesc {
 template <typename T>
 void launch_inv(const PartDesc* parts, int nparts, int t, const double* B, T* G, int* status,
                 int max_m, cudaStream_t st);
+// The float32 inverse of blocks to inv_f32_max_m() (dm_inv32.cu), which
+// launch_inv<float> takes unless DM_INV_KERNEL names another.
+int inv_f32_max_m();
+void launch_inv_f32(const PartDesc* parts, int nparts, int t, const double* B, float* G, int* status, int max_m,
+                    cudaStream_t st);
 // type_lo..type_hi-1 select the tile types: 0 = Acal_t and the next Schur
 // block (the inversion chain), 1 = left spike (off the chain).
 template <typename T>

@@ -1947,8 +1947,18 @@ template <typename T>
 void launch_inv(const PartDesc* parts, int nparts, int t, const double* B, T* G, int* status,
                 int max_m, cudaStream_t st) {
   if (nparts <= 0) return;
+  if constexpr (std::is_same<T, float>::value) {
+    // panels in shared memory: 85 against 163 us for 97 blocks of m = 128
+    // (register-resident), 67 against 113 for 42 of m = 88, 281 against 602
+    // where a batch fills the GPU (panel-blocked); above, a block and its
+    // panel don't fit in shared memory
+    if (inv_variant() == 1 && max_m <= inv_f32_max_m()) {
+      launch_inv_f32(parts, nparts, t, B, G, status, max_m, st);
+      return;
+    }
+  }
   const int cs = inv_cluster_size<T>(max_m);
-  // float32: the register-resident inverse while the blocks of a launch
+  // float32 above inv_f32_max_m() or with DM_INV_KERNEL: the register-resident inverse while the blocks of a launch
   // leave SMs idle (latency-bound, up to m = 128), the panel-blocked inverse
   // when there are enough blocks to fill the GPU several times over
   // (throughput-bound); float64: column by column, whose per-pivot update
