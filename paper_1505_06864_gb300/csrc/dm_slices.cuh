@@ -16,9 +16,9 @@ __host__ __device__ constexpr int slice_pitch(int m) { return (m + 7) & ~7; }
 __device__ __forceinline__ long long scaled_integer(unsigned long long bits, int e) {
   const int ex = (int)((bits >> 52) & 0x7ff);
   const unsigned long long mant = (bits & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
-  const int sh = (ex ? ex : 1) - 1075 + 55 - e;  // <= 2 for |v| < 2^e
-  const int dn = min(-sh, 60);
-  const unsigned long long Y = sh >= 0 ? (mant << (sh & 63)) : ((mant + (1ull << (dn - 1))) >> dn);
+  // (mant 8 >> n) / 2, rounded: |v| < 2^e leaves n >= 0, and from n = 56 on nothing is left
+  const int n = min(e + 1022 - (ex ? ex : 1), 62);
+  const unsigned long long Y = (((mant << 3) >> n) + 1) >> 1;
   return (long long)((bits >> 63) ? 0ull - Y : Y);
 }
 
