@@ -212,16 +212,16 @@ __device__ __forceinline__ void gj_control(int c0, int w, int nw, GjShared& sh, 
   }
 }
 
+// c += the product of two digit pairs (K = 16) or of one (K = 8): no side
+// effects, so the compiler may order the products of independent sums.
 __device__ __forceinline__ void mma_k16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                         uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(b0));
 }
@@ -232,110 +232,157 @@ __device__ __forceinline__ int bal_exponent(uint32_t hmax) {
   return hmax >= 0x7ff00000u ? kNotFinite : scale_exponent(hmax);
 }
 
+// The digits of a subpanel's pivot rows V (seven bf16 per value: [digit][column][row]) and
+// their columns' scales; the digits of its columns U by 16-row tile, in the
+// order in which gj_rank8's lanes hold them (two words more: a row's scale and
+// whether it is a pivot row).
+struct GjDigits {
+  uint32_t v[kBalSlices][PW][SW / 2];
+  int vexp[PW];
+  uint32_t pivots[kMaxM / 32];  // the subpanel's pivot rows
+};
+constexpr int kTileWords = 2 * kBalSlices + 2;
+
+// The digits of V = the rows piv[0 .. w - 1] of the panel; threads 0 .. 255, a value each.
+__device__ __forceinline__ void gj_digits_v(const double* P, const int* piv, int w, GjDigits& dg, int tid) {
+  const int c = tid >> 3, j = tid & 7;
+  const double v = j < w ? P[piv[min(j, w - 1)] * PS + c] : 0.0;
+  uint32_t h = abs_hi(v);
+  h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
+  h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
+  h = max(h, __shfl_xor_sync(0xffffffffu, h, 4));
+  const int e = bal_exponent(h);
+  uint32_t d[kBalSlices];
+  digits<7>((unsigned long long)__double_as_longlong(v), e, d);
+  unsigned short* dst = reinterpret_cast<unsigned short*>(dg.v);
+#pragma unroll
+  for (int k = 0; k < kBalSlices; ++k) dst[(k * PW + c) * SW + j] = (unsigned short)(d[k] >> 16);
+  if (j == 0) dg.vexp[c] = e;
+}
+
 // Rank-8 update of nq of the panel's 8-column groups (from column n0 on, wrapping) after
 // a subpanel's pivots: P[i][c] = (i a pivot row of the subpanel ? 0 : P[i][c])
 // + sum_j U[i][j] V[j][c], U the subpanel's columns, V its pivot rows before
-// the update; warp wi of nwk takes every nwk-th 16 x 8 tile.
+// the update; warp wi of nwk takes a run of the 16 x 8 tiles, row tile by row tile.
 // In float64 instructions it would cost twice the pivot chain itself, so it
 // runs on the tensor cores: seven balanced base-256 digits per operand (row
 // scales for U, column scales for V), the 28 digit products with s + t <= 8
 // in 16 mma.sync per 16 x 8 tile (two digit pairs share a K = 16
-// instruction), sums below 8 * 7 * 2^14 < 2^22, exact; one integer rounding
+// instruction), sums below 8 * 7 * 2^14 < 2^22, exact on top of the float
+// 1.5 2^23 they start from, whose bits then hold the integer; one integer rounding
 // and one float64 add per entry.  (tcgen05 has no use here: K = 8 and the
-// operands are in registers.)
-__device__ __noinline__ void gj_rank8(double* P, const double (*V)[PW], int mt, int c0, int n0, int nq,
-                                      const int* sub_piv, int w, int wi, int nwk) {
+// operands are in registers.)  A tile is a chain of dependent integer
+// instructions (3500 cycles when every warp made its digits of U and V
+// itself), so V's digits come from gj_digits_v, and U's are kept for the
+// helpers (keep: written to Ud; else read from there when `kept`).
+__device__ __noinline__ void gj_rank8(double* P, uint32_t* Ud, const GjDigits& dg, int mt, int c0, int n0, int nq,
+                                      bool keep, bool kept, int wi, int nwk) {
   const int lane = threadIdx.x & 31, g = lane >> 2, tg = lane & 3;
-  uint32_t b[kBalSlices];
-  int fe[2], qb = -1, nc = 0;
+  const int per = (mt * nq + nwk - 1) / nwk, i1 = min(mt * nq, (wi + 1) * per);
+  uint32_t a[2][kBalSlices];
+  int re[2];
+  bool z[2];
+  int rb = -1;
 #pragma unroll 1
-  for (int i = wi; i < mt * nq; i += nwk) {
+  for (int i = wi * per; i < i1; ++i) {
     __syncwarp();  // mma.sync below takes whole warps
-    const int q = i / mt, rt = i - q * mt;
-    if (q != qb) {  // the group's digits of V
-      qb = q;
-      nc = (n0 + SW * q) & (PW - 1);
-      const double v0 = V[2 * tg][nc + g], v1 = V[2 * tg + 1][nc + g];
-      uint32_t h = max(abs_hi(v0), abs_hi(v1));
-      h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
-      h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
-      const int e = bal_exponent(h);
-      uint32_t d0[kBalSlices], d1[kBalSlices];
-      digits<7>((unsigned long long)__double_as_longlong(v0), e, d0);
-      digits<7>((unsigned long long)__double_as_longlong(v1), e, d1);
+    const int rt = nq == 1 ? i : i / nq, nc = (n0 + SW * (i - rt * nq)) & (PW - 1);
+    uint32_t* ud = Ud + rt * (kTileWords * 32) + lane;
+    if (rt != rb) {
+      rb = rt;
+      if (kept) {
 #pragma unroll
-      for (int k = 0; k < kBalSlices; ++k) b[k] = pack_hi(d0[k], d1[k]);
-      fe[0] = __shfl_sync(0xffffffffu, e, 8 * tg);
-      fe[1] = __shfl_sync(0xffffffffu, e, 8 * tg + 4);
-    }
-    {
-      uint32_t a[2][kBalSlices];
-      int re[2];
-      bool z[2];
+        for (int h2 = 0; h2 < 2; ++h2) {
 #pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) {
-        const int row = 16 * rt + 8 * h2 + g;
-        const double v0 = P[row * PS + c0 + 2 * tg], v1 = P[row * PS + c0 + 2 * tg + 1];
-        uint32_t h = max(abs_hi(v0), abs_hi(v1));
-        h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
-        h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
-        re[h2] = bal_exponent(h);
-        uint32_t d0[kBalSlices], d1[kBalSlices];
-        digits<7>((unsigned long long)__double_as_longlong(v0), re[h2], d0);
-        digits<7>((unsigned long long)__double_as_longlong(v1), re[h2], d1);
+          for (int k = 0; k < kBalSlices; ++k) a[h2][k] = ud[32 * (h2 * kBalSlices + k)];
+          const int x = (int)ud[32 * (2 * kBalSlices + h2)];
+          re[h2] = x >> 1;
+          z[h2] = (x & 1) != 0;
+        }
+      } else {
 #pragma unroll
-        for (int k = 0; k < kBalSlices; ++k) a[h2][k] = pack_hi(d0[k], d1[k]);
-        z[h2] = false;
+        for (int h2 = 0; h2 < 2; ++h2) {
+          const int row = 16 * rt + 8 * h2 + g;
+          const double v0 = P[row * PS + c0 + 2 * tg], v1 = P[row * PS + c0 + 2 * tg + 1];
+          uint32_t h = max(abs_hi(v0), abs_hi(v1));
+          h = max(h, __shfl_xor_sync(0xffffffffu, h, 1));
+          h = max(h, __shfl_xor_sync(0xffffffffu, h, 2));
+          re[h2] = bal_exponent(h);
+          uint32_t d0[kBalSlices], d1[kBalSlices];
+          digits<7>((unsigned long long)__double_as_longlong(v0), re[h2], d0);
+          digits<7>((unsigned long long)__double_as_longlong(v1), re[h2], d1);
 #pragma unroll
-        for (int j = 0; j < SW; ++j) z[h2] = z[h2] || (j < w && sub_piv[j] == row);
-      }
-      int A[kBalSlices][4];  // acc_d, d = 2 .. 8
+          for (int k = 0; k < kBalSlices; ++k) a[h2][k] = pack_hi(d0[k], d1[k]);
+          z[h2] = ((dg.pivots[row >> 5] >> (row & 31)) & 1u) != 0;
+          if (keep) {
 #pragma unroll
-      for (int d = 2; d <= 8; ++d) {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-        int s = 1;
-#pragma unroll
-        for (; s + 1 <= d - 1; s += 2)
-          mma_k16(c, a[0][s - 1], a[1][s - 1], a[0][s], a[1][s], b[d - s - 1], b[d - s - 2]);
-        if (s <= d - 1) mma_k8(c, a[0][s - 1], a[1][s - 1], b[d - s - 1]);
-#pragma unroll
-        for (int o = 0; o < 4; ++o) A[d - 2][o] = __float_as_int(c[o] + 12582912.0f) - 0x4B400000;
-      }
-      double v[4];
-      bool odd = re[0] == kNotFinite || re[1] == kNotFinite || fe[0] == kNotFinite || fe[1] == kNotFinite;
-#pragma unroll
-      for (int o = 0; o < 4; ++o) {
-        // units 2^(e_r + f_c + 2 - 60): the last accumulator's low four bits are dropped
-        const long long T = (long long)(A[0][o] * 256 + A[1][o]) * (1ll << 36) +
-                            (long long)(A[2][o] * 256 + A[3][o]) * (1ll << 20) +
-                            (long long)(A[4][o] * 256 + A[5][o]) * 16 + (A[6][o] >> 4);
-        v[o] = round_scaled(T, re[o >> 1] + fe[o & 1] - 58, odd);
-      }
-      if (odd) {  // results outside the normal range, NaN and infinite operands
-#pragma unroll 1
-        for (int o = 0; o < 4; ++o) {
-          int t[kBalSlices];
-#pragma unroll
-          for (int k = 0; k < kBalSlices; ++k) t[k] = o == 0 ? A[k][0] : o == 1 ? A[k][1] : o == 2 ? A[k][2] : A[k][3];
-          const long long T = (long long)(t[0] * 256 + t[1]) * (1ll << 36) + (long long)(t[2] * 256 + t[3]) * (1ll << 20) +
-                              (long long)(t[4] * 256 + t[5]) * 16 + (t[6] >> 4);
-          const int er = o < 2 ? re[0] : re[1], ec = (o & 1) ? fe[1] : fe[0];
-          const double x = er == kNotFinite || ec == kNotFinite ? __longlong_as_double(0x7ff8000000000000ll)
-                                                                : ldexp((double)T, er + ec - 58);
-          if (o == 0) v[0] = x;
-          if (o == 1) v[1] = x;
-          if (o == 2) v[2] = x;
-          if (o == 3) v[3] = x;
+            for (int k = 0; k < kBalSlices; ++k) ud[32 * (h2 * kBalSlices + k)] = a[h2][k];
+            ud[32 * (2 * kBalSlices + h2)] = (uint32_t)(re[h2] * 2 + (z[h2] ? 1 : 0));
+          }
         }
       }
+    }
+    uint32_t b[kBalSlices];
 #pragma unroll
-      for (int o = 0; o < 4; ++o) {
-        double* d = P + (16 * rt + 8 * (o >> 1) + g) * PS + nc + 2 * tg + (o & 1);
-        *d = (z[o >> 1] ? 0.0 : *d) + v[o];
+    for (int k = 0; k < kBalSlices; ++k) b[k] = dg.v[k][nc + g][tg];
+    const int fe[2] = {dg.vexp[nc + 2 * tg], dg.vexp[nc + 2 * tg + 1]};
+    float c[kBalSlices][4];  // acc_d + 1.5 2^23, d = 2 .. 8
+#pragma unroll
+    for (int k = 0; k < kBalSlices; ++k)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) c[k][o] = 12582912.0f;
+#pragma unroll
+    for (int s = 1; s <= kBalSlices; s += 2)
+#pragma unroll
+      for (int d = s + 1; d <= 8; ++d) {
+        if (s + 1 <= d - 1)
+          mma_k16(c[d - 2], a[0][s - 1], a[1][s - 1], a[0][s], a[1][s], b[d - s - 1], b[d - s - 2]);
+        else
+          mma_k8(c[d - 2], a[0][s - 1], a[1][s - 1], b[d - s - 1]);
       }
+    // units 2^(e_r + f_c + 2 - 60): the last accumulator's low four bits are
+    // dropped; kBias is what the start leaves in 256 x + y
+    constexpr uint32_t kBias1 = 0x4B400000u, kBias = kBias1 * 257u;
+    auto total = [&](const uint32_t (&t)[kBalSlices]) {
+      return (long long)(int)(t[0] * 256u + t[1] - kBias) * (1ll << 36) +
+             (long long)(int)(t[2] * 256u + t[3] - kBias) * (1ll << 20) +
+             (long long)(int)(t[4] * 256u + t[5] - kBias) * 16 + ((int)(t[6] - kBias1) >> 4);
+    };
+    double v[4];
+    bool odd = re[0] == kNotFinite || re[1] == kNotFinite || fe[0] == kNotFinite || fe[1] == kNotFinite;
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      uint32_t t[kBalSlices];
+#pragma unroll
+      for (int k = 0; k < kBalSlices; ++k) t[k] = __float_as_uint(c[k][o]);
+      v[o] = round_scaled(total(t), re[o >> 1] + fe[o & 1] - 58, odd);
+    }
+    if (odd) {  // results outside the normal range, NaN and infinite operands
+#pragma unroll 1
+      for (int o = 0; o < 4; ++o) {
+        uint32_t t[kBalSlices];
+#pragma unroll
+        for (int k = 0; k < kBalSlices; ++k)
+          t[k] = __float_as_uint(o == 0 ? c[k][0] : o == 1 ? c[k][1] : o == 2 ? c[k][2] : c[k][3]);
+        const int er = o < 2 ? re[0] : re[1], ec = (o & 1) ? fe[1] : fe[0];
+        const double x = er == kNotFinite || ec == kNotFinite ? __longlong_as_double(0x7ff8000000000000ll)
+                                                              : ldexp((double)total(t), er + ec - 58);
+        if (o == 0) v[0] = x;
+        if (o == 1) v[1] = x;
+        if (o == 2) v[2] = x;
+        if (o == 3) v[3] = x;
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      double* d = P + (16 * rt + 8 * (o >> 1) + g) * PS + nc + 2 * tg + (o & 1);
+      *d = (z[o >> 1] ? 0.0 : *d) + v[o];
     }
   }
 }
+
+// Shared memory of k_gj_panel for mt 16-row tiles.
+constexpr size_t smem_bytes(int mt) { return (size_t)mt * (16 * PS * sizeof(double) + kTileWords * 32 * sizeof(uint32_t)); }
 
 // Eight values' digits to a slice array: slice sl at dst + sl * stride.
 __device__ __noinline__ void gj_slice8(double v0, double v1, double v2, double v3, double v4, double v5, double v6, double v7,
@@ -355,9 +402,11 @@ __device__ __noinline__ void gj_slice8(double v0, double v1, double v2, double v
 // eight chain warps (a row per lane; two rows above m = 256), the control
 // warp, and eight helpers.  Bound by the chain's float64 instructions and
 // barriers: about 1150 cycles per pivot to m = 128 (one warp per SM
-// sub-partition) and 1700 at m = 256 (two).  A cluster of CTAs with the rows
+// sub-partition) and 1800 at m = 256 (two), half of the kernel's time; the updates that the
+// chain waits for take a sixth, the slices at the end an eighth.  A cluster of CTAs with the rows
 // split and a cluster barrier per pivot took 83 / 90 / 98 us per panel at m =
-// 64 / 128 / 256, this one 40 / 47 / 76 us (34, 97, 64 blocks).  The loops
+// 64 / 128 / 256, this one with every warp making its own digits of U and V 40 / 48 / 74 us, and
+// 37 / 43 / 63 us (115 to 102 at m = 400) with the digits shared (34, 97, 64 blocks).  The loops
 // stay rolled: the code runs once per launch, and unrolled it waited for its
 // instructions.
 template <int CW, int RPL>
@@ -365,10 +414,10 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
     k_gj_panel(const PartDesc* __restrict__ parts, int t, int m, int panel, double* __restrict__ W,
                int* __restrict__ piv, __nv_bfloat16* __restrict__ Us, int* __restrict__ Uexp,
                __nv_bfloat16* __restrict__ Vs, int* __restrict__ Vexp, int* __restrict__ status) {
-  extern __shared__ __align__(16) double P[];  // [16 ceil(m / 16)][PS]
+  extern __shared__ __align__(16) double P[];  // [16 ceil(m / 16)][PS], then U's digits by tile
   __shared__ GjShared sh;
   constexpr int kWorkers = CW + kHelpers, kWarps = kWorkers + 1, kThreads = 32 * kWarps;  // the last: control
-  __shared__ double V[SW][PW];
+  __shared__ GjDigits dg;
   __shared__ int piv_s[PW];
   __shared__ uint32_t used[kMaxM / 32];
   const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -377,6 +426,7 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
   double* M = W + (long long)q * m * m;
   const int k0 = PW * panel, kw = min(PW, m - k0), mt = (m + 15) / 16;
   const int nw = min(CW, (m + 31) / 32);
+  uint32_t* Ud = reinterpret_cast<uint32_t*>(P + 16 * mt * PS);
   if (tid < kMaxM / 32) used[tid] = 0;
   __syncthreads();
   for (int k = tid; k < k0; k += kThreads) {
@@ -388,10 +438,10 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
     P[i * PS + lane] = (i < m && lane < kw) ? M[(long long)i * m + k0 + lane] : 0.0;
   __syncthreads();
   bool bad = false;
-  // Per subpanel: the pivots on warps 0-3 and the control warp while warps 4-7 finish the rank-8
-  // update of the subpanel before (its 16 columns that are not next); then
-  // all warps update the next subpanel's columns (after the last subpanel all
-  // other columns), which its chain waits for.
+  // Per subpanel: the pivots on the chain's warps and the control warp while the helpers
+  // finish the rank-8 update of the subpanel before (its 16 columns that are
+  // not next); then all of them but the control warp update the next subpanel's columns (after the
+  // last subpanel all other columns), which its chain waits for.
 #pragma unroll 1
   for (int c0 = 0; c0 < kw; c0 += SW) {
     const int w = min(SW, kw - c0);
@@ -400,14 +450,22 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
     else if (warp == kWorkers)
       gj_control(c0, w, nw, sh, piv_s, lane, bad);
     else if (warp >= CW && c0 > 0)
-      gj_rank8(P, V, mt, c0 - SW, c0 + SW, 2, piv_s + c0 - SW, SW, warp - CW, kHelpers);
+      gj_rank8(P, Ud, dg, mt, c0 - SW, c0 + SW, 2, false, true, warp - CW, kHelpers);
     __syncthreads();
-    // this subpanel's pivot rows of the other columns
-    if (warp < SW) V[warp][lane] = warp < w ? P[piv_s[c0 + min(warp, w - 1)] * PS + lane] : 0.0;
-    if (tid < w) atomicOr(&used[piv_s[c0 + tid] >> 5], 1u << (piv_s[c0 + tid] & 31));
+    // this subpanel's pivot rows
+    if (tid < SW * PW) gj_digits_v(P, piv_s + c0, w, dg, tid);
+    if (tid >= SW * PW && tid < SW * PW + kMaxM / 32) {
+      uint32_t bits = 0;
+      for (int j = 0; j < w; ++j)
+        if ((piv_s[c0 + j] >> 5) == tid - SW * PW) bits |= 1u << (piv_s[c0 + j] & 31);
+      dg.pivots[tid - SW * PW] = bits;
+      used[tid - SW * PW] |= bits;
+    }
     __syncthreads();
-    if (kw > SW && warp < kWorkers)
-      gj_rank8(P, V, mt, c0, c0 + SW, c0 + SW < kw ? 1 : 3, piv_s + c0, w, warp, kWorkers);
+    if (kw > SW && warp < kWorkers) {
+      const bool last = c0 + SW >= kw;
+      gj_rank8(P, Ud, dg, mt, c0, c0 + SW, last ? 3 : 1, !last, false, warp, kWorkers);
+    }
     __syncthreads();
   }
   if (tid < kw) piv[(long long)q * m + k0 + tid] = piv_s[tid];
@@ -526,13 +584,13 @@ void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const doub
 void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, int* piv, void* Us,
                      int* Uexp, void* Vs, int* Vexp, int* status, cudaStream_t st) {
   if (nparts <= 0) return;
-  const size_t smem = (size_t)16 * ((m + 15) / 16) * gj::PS * sizeof(double);
+  const size_t smem = gj::smem_bytes((m + 15) / 16);
 #define DM_GJ(C_, R_)                                                                                                   \
   do {                                                                                                              \
     static bool set = false;                                                                                        \
     if (!set) {                                                                                                     \
       cudaFuncSetAttribute(gj::k_gj_panel<C_, R_>, cudaFuncAttributeMaxDynamicSharedMemorySize,                         \
-                           32 * C_ * R_ * gj::PS * (int)sizeof(double));                                                \
+                           (int)gj::smem_bytes(2 * C_ * R_));                                                \
       set = true;                                                                                                   \
     }                                                                                                               \
     gj::k_gj_panel<C_, R_><<<nparts, 32 * (C_ + gj::kHelpers + 1), smem, st>>>(                                     \
