@@ -182,12 +182,14 @@ int Level::build(const std::vector<SysSpec>& specs, bool fp32_factors, int tenso
     active_back[s] = c;
   }
   // Both z sweeps in one persistent launch when every subsystem's cluster is
-  // resident at once (a second wave would serialise whole sweeps); with many
-  // subsystems the per-step launches keep the GPU busier.  DM_SOLVE_SWEEP=0
+  // resident at once (a second wave would serialise whole sweeps), or in a few
+  // waves when block sizes differ; with many subsystems the per-step launches
+  // keep the GPU busier.  DM_SOLVE_SWEEP=0
   // keeps the per-step kernels (for comparisons).
   {
     const char* e = std::getenv("DM_SOLVE_SWEEP");
-    sweep_cs = (e && e[0] == '0') ? 0 : sweep_cluster_choice(f32 ? 4 : 8, max_m, max_r, nparts);
+    const bool mixed = std::any_of(parts.begin(), parts.end(), [&](const PartDesc& p) { return p.m != max_m; });
+    sweep_cs = (e && e[0] == '0') ? 0 : sweep_cluster_choice(f32 ? 4 : 8, max_m, max_r, nparts, mixed);
     sweep = sweep_cs > 0;
   }
   compute_costs();

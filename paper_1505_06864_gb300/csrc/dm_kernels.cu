@@ -2128,8 +2128,19 @@ cudaLaunchConfig_t sweep_config(int nparts, int cs, int max_m, cudaStream_t st, 
 
 // Largest cluster size (about 16 rows per CTA, at most the portable 8) at
 // which all nparts clusters are resident together; 0 if none.
+//
+// Subsystems of several block sizes (`mixed`) may take more waves, with
+// clusters of at least 32 rows per CTA: the largest subsystems come first and
+// their chains, not the sum of the work, set the time, so a larger cluster for
+// them is worth the waves of the others.  Six waves where the arithmetic is
+// float64 (a CTA is bound by its SM's FP64 pipe), 3.5 in float32.  Measured (m = 32 .. 256, 1
+// to 16 right-hand sides, 40 systems): 255 float64 subsystems 12.2 ms with
+// one CTA each (resident), 3.6 with four (3.4 waves); 1010 float32 ones 6.6 step by step, 4.7 with two
+// (3.3 waves), 5.3 with four (6.8); 1016 float64 ones with one right-hand side 1.95
+// resident, 1.51 with four (3.4), 1.85 with eight (6.9).  With one block size the gain is
+// small or a loss (384 of m = 128, r = 8: 2.90 resident, 2.89 with two, 3.12 with four).
 template <typename T>
-int sweep_choice_t(int max_m, int max_r, int nparts) {
+int sweep_choice_t(int max_m, int max_r, int nparts, bool mixed) {
   if (max_r > 16 || sizeof(T) * 3 * (size_t)max_m * (size_t)rbucket(max_r) > 227 * 1024) return 0;
   if (nparts <= 0) return 0;
   int cs = 1;
@@ -2146,14 +2157,16 @@ int sweep_choice_t(int max_m, int max_r, int nparts) {
         cudaGetLastError();
         return;
       }
-      if (nclusters >= nparts) chosen = c;
+      const bool wide = mixed && 32 * c <= max_m;
+      if (nclusters >= nparts || (wide && (sizeof(T) == 8 ? 6.0 : 3.5) * nclusters >= nparts)) chosen = c;
     }
   });
   return chosen;
 }
 
-int sweep_cluster_choice(int elem_bytes, int max_m, int max_r, int nparts) {
-  return elem_bytes == 4 ? sweep_choice_t<float>(max_m, max_r, nparts) : sweep_choice_t<double>(max_m, max_r, nparts);
+int sweep_cluster_choice(int elem_bytes, int max_m, int max_r, int nparts, bool mixed) {
+  return elem_bytes == 4 ? sweep_choice_t<float>(max_m, max_r, nparts, mixed)
+                         : sweep_choice_t<double>(max_m, max_r, nparts, mixed);
 }
 
 template <typename T>
