@@ -279,11 +279,11 @@ def main():
     # roofline of the dominant kernel class (largest summed event time)
     top = max(prof.items(), key=lambda kv: kv[1]["ms"])
     kname, kd = top
-    roof = class_roofline(kname, kd, prof, mixed, clk, peaks, dev)
+    roof = class_roofline(kname, kd, prof, mixed, clk, peaks, dev, s.m)
     roof["timing"] = ("CUDA events around each launch in a second run of the same steps "
                       f"({prof_ms_step:.1f} ms/step instrumented vs {total_ms / args.steps:.1f} graph-replayed)")
     others = sorted(prof.items(), key=lambda kv: -kv[1]["ms"])[1:4]
-    roof["next"] = {k: {key: val for key, val in class_roofline(k, v, prof, mixed, clk, peaks, dev).items()
+    roof["next"] = {k: {key: val for key, val in class_roofline(k, v, prof, mixed, clk, peaks, dev, s.m).items()
                         if key in ("bound", "achieved", "peak", "unit", "frac", "share_of_step")}
                     for k, v in others}
     kernels = {k: {"launches": v["launches"], "ms_per_step": v["ms"] / args.steps,
@@ -351,14 +351,19 @@ def rel_err(x, xref):
 
 
 # float64 classes whose products run as digit-sliced bf16 tensor-core MMAs: per
-# float64 multiply-add, 54 slice-pair products (the 53 pairs with s + t <= 11
-# and one against the zero slice that initialises the accumulators)
+# float64 multiply-add, 34 slice-pair products with seven digits (K <= 128; the
+# inverse's updates have K = 32), 43 with eight
 SLICED_CLASSES = ("fwd_factor", "back_factor", "inv_update", "assemble_h")
-SLICE_PRODUCTS = 54
+
+
+def slice_products(base, m):
+    return 34 if base == "inv_update" or m <= 128 else 43
+
+
 HBM_CLASSES = ("inv", "tc_convert", "sweep_solve", "backsub", "sep_copy", "assemble_f", "axpy_norms")
 
 
-def class_roofline(kname, kd, prof, mixed, clk, peaks, dev):
+def class_roofline(kname, kd, prof, mixed, clk, peaks, dev, m):
     """Roofline of one kernel class: algorithmic flops (or bytes) of its
     launches over their summed CUDA-event time, against the peak of what
     bounds it: the derived float64 ALU peak for float64 CUDA-core kernels, the
@@ -374,9 +379,10 @@ def class_roofline(kname, kd, prof, mixed, clk, peaks, dev):
     if not mixed and base in SLICED_CLASSES:
         alg = kd["flops"] / secs / 1e12
         peak = mp.get("bf16_tflops") or 1900.0
-        return {**common, "bound": "tensor", "achieved": alg * SLICE_PRODUCTS, "peak": peak, "unit": "TFLOP/s",
-                "frac": alg * SLICE_PRODUCTS / peak, "achieved_algorithmic": alg,
-                "mma_flops_per_algorithmic": SLICE_PRODUCTS,
+        pairs = slice_products(base, m)
+        return {**common, "bound": "tensor", "achieved": alg * pairs, "peak": peak, "unit": "TFLOP/s",
+                "frac": alg * pairs / peak, "achieved_algorithmic": alg,
+                "mma_flops_per_algorithmic": pairs,
                 "peak_source": "bf16 dense, measured cuBLAS burst (MEASURED_PEAKS.json), of measured"}
     if base in HBM_CLASSES:
         ach = kd["bytes"] / secs / 1e9

@@ -152,7 +152,7 @@ bool tc2_eligible(int m);
 
 // Float64 products on the tensor cores by exact digit slicing (dm_oz.cu):
 // the step kernels' products with float64 operands and results, the operands
-// as nine bf16 digit slices with per-row (left) / per-column (right) scales.
+// as bf16 digit slices with per-row (left) / per-column (right) scales.
 struct OzOut {
   const double* B;
   double *G, *Acal, *ZL, *ZR, *Y;  // Y: Y_{t+1} per subsystem (rolling, float64)
