@@ -1973,8 +1973,9 @@ void launch_inv(const PartDesc* parts, int nparts, int t, const double* B, T* G,
     }
   }
   const int cs = inv_cluster_size<T>(max_m);
-  // float32 above inv_f32_max_m() or with DM_INV_KERNEL: the register-resident inverse while the blocks of a launch
-  // leave SMs idle (latency-bound, up to m = 128), the panel-blocked inverse
+  // float32 above inv_f32_max_m() or with DM_INV_KERNEL: the register-resident
+  // inverse while the blocks of a launch leave SMs idle (latency-bound, up to
+  // m = 128), the panel-blocked inverse
   // when there are enough blocks to fill the GPU several times over
   // (throughput-bound); float64: column by column, whose per-pivot update
   // spreads the FP64 work over every warp of the cluster.
