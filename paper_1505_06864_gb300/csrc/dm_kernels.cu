@@ -1378,6 +1378,9 @@ __device__ void sweep_body(const PartDesc& p, int rank, int cs, const double* __
                            const T* __restrict__ G, const T* __restrict__ Acal, const double* __restrict__ F,
                            T* __restrict__ z, T* Zp0, T* Zp1, T* Rs) {
   cg::cluster_group cl = cg::this_cluster();
+  // a CTA's shared memory may be written by a peer only once it has started:
+  // step 0 pushes its rows before any of the sweep's own barriers
+  if (cs > 1) cl.sync();
   const int m = p.m, r = p.r, L = p.L;
   const int rpc = (m + cs - 1) / cs;
   const int r0 = min(m, rank * rpc), r1 = min(m, r0 + rpc);
