@@ -194,18 +194,22 @@ __device__ __forceinline__ void gj_chain(double* P, int m, int c0, int w, int nw
   }
 }
 
-// The control warp's side of gj_chain.
-__device__ __forceinline__ void gj_control(int c0, int w, int nw, GjShared& sh, int* piv_s, int lane, bool& bad) {
+// The control warp's side of gj_chain.  Before the last pivot some row is
+// eligible, and an eligible row's key is at least 1, so a pivot is always
+// found; were none (key 0), it would count as singular, and the row stays
+// inside the block whatever a warp published.
+__device__ __forceinline__ void gj_control(int m, int c0, int w, int nw, GjShared& sh, int* piv_s, int lane, bool& bad) {
 #pragma unroll 1
   for (int j = 0; j < w; ++j) {
     asm volatile("bar.sync 1, %0;" ::"r"(32 * nw + 32) : "memory");
     const GjCand c = sh.cand[j & 1][min(lane, nw - 1)];
     const uint32_t kmax = __reduce_max_sync(0xffffffffu, c.key);
     const int best = (int)__reduce_min_sync(0xffffffffu, c.key == kmax ? (uint32_t)lane : 32u);
-    const double inv = pivot_unusable(c.v) ? 0.0 : pivot_recip(c.v);
+    const double inv = kmax == 0 || pivot_unusable(c.v) ? 0.0 : pivot_recip(c.v);
     if (lane == best) {
-      sh.piv[j & 1] = GjPivot{inv, c.idx, best};
-      piv_s[c0 + j] = c.idx;
+      const int row = min(c.idx, m - 1);
+      sh.piv[j & 1] = GjPivot{inv, row, best};
+      piv_s[c0 + j] = row;
       if (__double_as_longlong(inv) == 0) bad = true;
     }
     asm volatile("bar.sync 2, %0;" ::"r"(32 * nw + 32) : "memory");
@@ -448,7 +452,7 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
     if (warp < nw)
       gj_chain<CW, RPL>(P, m, c0, w, nw, used, sh, warp, lane);
     else if (warp == kWorkers)
-      gj_control(c0, w, nw, sh, piv_s, lane, bad);
+      gj_control(m, c0, w, nw, sh, piv_s, lane, bad);
     else if (warp >= CW && c0 > 0)
       gj_rank8(P, Ud, dg, mt, c0 - SW, c0 + SW, 2, false, true, warp - CW, kHelpers);
     __syncthreads();

@@ -42,7 +42,9 @@ struct Shared {
 // The pivots of the columns c0 .. c0 + w - 1 on warps 0 .. nw - 1: lane holds
 // rows 32 warp + lane + 128 i.  Register c holds column (j - 1 + c) mod 8
 // before pivot j; the pivot's own row takes part as zeros plus the reciprocal
-// times itself.
+// times itself.  While a pivot is left some row is eligible, with a key of at
+// least 1; were none, the pivot would count as unusable, and the row stays
+// inside the block.
 template <int RPL>
 __device__ __forceinline__ void chain(float* M, int ld, int m, int c0, int w, int nw, Shared& sh, int warp, int lane) {
   float a[RPL][SW], fn[RPL], s[SW];
@@ -94,9 +96,9 @@ __device__ __forceinline__ void chain(float* M, int ld, int m, int c0, int w, in
     for (int q = 1; q < kChain; ++q)
       if (q < nw && sh.key[buf][q] > kb) kb = sh.key[buf][q], best = q;
     const float4 lo = sh.row[buf][best][0], hi = sh.row[buf][best][1];
-    const int prow = sh.idx[buf][best];
+    const int prow = min(sh.idx[buf][best], m - 1);
     float inv = __frcp_rn(lo.x);
-    const bool unusable = !(fabsf(lo.x) > 0.f) || !isfinite(inv);
+    const bool unusable = kb == 0 || !(fabsf(lo.x) > 0.f) || !isfinite(inv);
     if (unusable) inv = 0.f;
     s[0] = 1.f;
     s[1] = lo.y, s[2] = lo.z, s[3] = lo.w, s[4] = hi.x, s[5] = hi.y, s[6] = hi.z, s[7] = hi.w;

@@ -58,7 +58,8 @@ __device__ __forceinline__ void invert(const double* D, double* G, int m, Shared
   for (int c = 0; c < CPW; ++c) a[c] = lane < m && c0 + c < m ? D[lane * LD + c0 + c] : 0.0;
   bool dead = lane >= m;
   int step = 0;  // the column this lane's row is the pivot of
-  // the search of column j on its owner warp, values v
+  // the search of column j on its owner warp, values v (the row is a lane's
+  // number, so it stays inside the 32 rows of every shared array)
   auto publish = [&](double v, int j) {
     const uint32_t key = dead ? 0u : abs_hi(v) + 1u;
     const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
