@@ -114,15 +114,23 @@ int dm_plan(dm_plan_t* out, int N, int m, int nrhs, int P, int levels, int preci
 #define DM_PLAN_EQUAL_TIME 1
 /* Float64 block products (DM_FP64 plans and every supplementary level) are by
  * default computed on the tensor cores by exact digit slicing where the level
- * has one block size m >= 16: every float64 operand is cut into balanced digit
- * slices (bf16; seven of base 2^8 to m = 128, eight of base 2^7 above) with a
+ * has one block size m > 32 (levels of smaller blocks run in one float64
+ * launch): every float64 operand is cut into balanced digit slices (bf16;
+ * seven of base 2^8 to m = 128, eight of base 2^7 above) with a
  * power-of-two scale per row (left operand) or column (right operand), the
  * digit products that matter (s + t <= slices + 2) are accumulated exactly
  * (integers of at most 2^24 in float32), and the sums are combined in 64-bit
- * integers -- an error bound of the size of the float64 dot product's.
- * DM_PLAN_FP64_FMA keeps them on the float64 pipe; so does a plan with m % 8
- * != 0 or m > 256 whose slices (about as much again as its factors) do not
- * fit the free device memory. */
+ * integers: an error per entry below m 2^-53 max|row| max|column|.  Before
+ * they are cut, the operands are balanced by exact powers of two, one per
+ * equation and one per unknown, found from the level's blocks at the start of
+ * dm_factor, and the blocks are inverted so equilibrated: equations and
+ * unknowns of different scale cost no accuracy (what is bounded by the largest
+ * entries is so after the scaling; an entry far below them is not resolved
+ * relative to itself, as in a float64 dot product of few terms it would be).
+ * DM_PLAN_FP64_FMA keeps the products on the float64 pipe; so does a plan with
+ * m % 8 != 0 or m > 256 whose slices (about as much again as its factors) do
+ * not fit the device memory free at dm_plan (several times slower, and in
+ * other roundings). */
 #define DM_PLAN_FP64_FMA 2
 /* The float64 block inverse of those levels is by default blocked
  * Gauss-Jordan (panels of 32 columns in float64, their rank-32 trailing

@@ -322,7 +322,7 @@ static bool small_wanted(const Level& L) {
 
 static size_t oz_bytes(long long nblk, int nparts, int nseps, int m) {
   const size_t mm = (size_t)m * m, sl = (size_t)oz_slice_blocks_bytes(m), nb = nblk / mm, np = std::max(1, nparts);
-  return (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + 2 * np * mm * sizeof(double) +
+  return 2 * nb * m * sizeof(int) + (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + 2 * np * mm * sizeof(double) +
          np * ((size_t)2 * 7 * m * 32 * 2 + 3 * m * sizeof(int));
 }
 
@@ -470,6 +470,8 @@ int Level::allocate() {
     DM_ALLOC(Z.eZLT, 2 * np * ex);
     DM_ALLOC(Z.eZRT, 2 * np * ex);
     DM_ALLOC(Z.Y, np * mm * sizeof(double));
+    DM_ALLOC(Z.gam, nb * ex);
+    DM_ALLOC(Z.rho, nb * ex);
     const void* lbase[3] = {Z.G, Z.A, Z.Acal};
     const long long lblk[3] = {np, nb, nb};
     const void* rbase[5] = {Z.CT, Z.YT, Z.AcalT, Z.ZLT, Z.ZRT};
@@ -696,7 +698,8 @@ static void factor_level_tc2(Level& L, cudaStream_t st, Prof& pf) {
 }
 
 // Forward and backward sweeps of a float64 level with its block products on
-// the tensor cores by digit slicing (dm_oz.cu): slices of A (rows), C^T and
+// the tensor cores by digit slicing (dm_oz.cu): the scales of its equations
+// and unknowns, slices of A (rows), C^T and
 // Y_0 = A_first^T (columns), then per step the float64 inversion, the row
 // slices of G_t, launch A = G_t [C_t | Y_t], slices of its results (Acal_t
 // rows and columns, Bcal_t columns, the right spike's seed), launch B =
@@ -715,6 +718,8 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
   out.ZR = static_cast<double*>(L.ZR);
   out.Y = Z.Y;
   out.W = Z.W;
+  out.gam = Z.gam;
+  out.rho = Z.rho;
   out.band = Z.band;
   // banded A and C as the previous factorisation found them (profiling costs
   // only: the kernels read the flag this factorisation's slicing sets)
@@ -735,21 +740,25 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
   const int* lexp[3] = {Z.eG, Z.eA, Z.eAcal};
   const int* r0exp[3] = {Z.eCT, Z.eAcalT, Z.eZLT};
   const int* r1exp[3] = {Z.eYT, Z.eZLT, Z.eZRT};
+  OzSliceJobs jobs0;
+  jobs0.gam = Z.gam;
+  jobs0.rho = Z.rho;
   auto job = [](const double* src, void* dst, int* e, int kind) { return OzSliceJob{src, dst, e, kind}; };
+  Cost cscale;
+  cscale.bytes = 48.0 * L.nblk;
+  DM_LAUNCH_K(pf, st, K_TC_CONVERT, cscale, 1, 2,
+              (Z.band ? (void)cudaMemsetAsync(Z.band, 0, sizeof(int), st) : (void)0,
+               launch_level_scales(L.d_sys, L.nsys, L.A, L.B, L.C, (int)nb, m, Z.gam, Z.rho, Z.band, st)));
   auto slice_inputs = [&] {
-    if (Z.band) {
-      cudaMemsetAsync(Z.band, 0, sizeof(int), st);
-      launch_band_detect(L.A, L.C, L.nblk, m, Z.band, st);
-    }
-    launch_oz_slice_all(false, L.A, (int)nb, m, Z.A, Z.eA, Z.band, st);
-    launch_oz_slice_all(true, L.C, (int)nb, m, Z.CT, Z.eCT, Z.band, st);
+    launch_oz_slice_all(false, L.A, (int)nb, m, Z.A, Z.eA, Z.gam, Z.rho, Z.band, st);
+    launch_oz_slice_all(true, L.C, (int)nb, m, Z.CT, Z.eCT, Z.gam, Z.rho, Z.band, st);
     if (Z.band) cudaMemcpyAsync(Z.band_host, Z.band, sizeof(int), cudaMemcpyDeviceToHost, st);
-    OzSliceJobs j0;
+    OzSliceJobs j0 = jobs0;
     j0.job[0] = job(L.A, Z.YT, Z.eYT, 8);
     launch_oz_slice_jobs(L.d_parts, L.nparts, 0, m, j0, 1, st);
   };
   Cost cslice = L.c_cvt;
-  DM_LAUNCH_K(pf, st, K_TC_CONVERT, cslice, 1, Z.band ? 4 : 3, slice_inputs());
+  DM_LAUNCH_K(pf, st, K_TC_CONVERT, cslice, 1, 3, slice_inputs());
   Cost cs;
   cs.bytes = (8.0 + 2.0 * oz_slices(m)) * m * m;  // one block: float64 read, its bf16 slices written
   for (int t = 0; t < L.Lmax; ++t) {
@@ -762,7 +771,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
       Cost cb, cf;
       cb.bytes = np * 16.0 * m * m;           // B_0 read, written to G
       cf.bytes = np * (16.0 + 2.0 * oz_slices(m)) * m * m;  // G_t read and written, its bf16 slices written
-      if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, Z.W, st));
+      if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, Z.W, Z.gam, Z.rho, st));
       for (int k0 = 0; k0 < m; k0 += 32) {
         const double kw = std::min(32, m - k0);
         Cost cp, cu;
@@ -776,10 +785,10 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
           DM_LAUNCH(pf, st, K_INV_UPDATE, cu, np,
                     launch_gj_update(L.d_parts, np, t, m, k0 / 32, Z.W, Z.piv, Z.eU, Z.eV, Z.gj_maps, L.d_err, st));
       }
-      DM_LAUNCH(pf, st, K_INV, cf, np, launch_gj_finish(L.d_parts, np, t, m, Z.W, G, Z.piv, Z.G, Z.eG, st));
+      DM_LAUNCH(pf, st, K_INV, cf, np, launch_gj_finish(L.d_parts, np, t, m, Z.W, G, Z.piv, Z.G, Z.eG, Z.gam, Z.rho, st));
     } else {
       DM_LAUNCH(pf, st, K_INV, L.c_inv[t], np, launch_inv<double>(L.d_parts, np, t, L.B, G, L.status, L.max_m, st));
-      OzSliceJobs jg;
+      OzSliceJobs jg = jobs0;
       jg.job[0] = job(G, Z.G, Z.eG, 0);
       Cost c0 = cs;
       c0.bytes *= np;
@@ -792,7 +801,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
     if (Z.band)  // G_t C_t when C is banded (the tiles above skip it then)
       DM_LAUNCH(pf, st, K_BANDED, band_cost(np, 1), np,
                 launch_band_gc(L.d_parts, np, t, m, G, L.C, out.Acal, out.ZR, Z.band, st));
-    OzSliceJobs ja;
+    OzSliceJobs ja = jobs0;
     ja.band = Z.band;
     ja.job[0] = job(out.Acal, Z.Acal, Z.eAcal, 1);
     ja.job[1] = job(out.Acal, Z.AcalT, Z.eAcalT, 2);
@@ -805,8 +814,8 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
               launch_oz_step(1, L.d_parts, nbk, t, m, out, lexp[1], r0exp[1], r1exp[1], maps[1], L.d_err, st));
     if (Z.band)  // both products of launch B when A is banded
       DM_LAUNCH(pf, st, K_BANDED, band_cost(nbk, 2), nbk,
-                launch_band_b(L.d_parts, nbk, t, m, L.A, L.B, out.Acal, out.ZL, G, Z.W, Z.Y, Z.band, st));
-    OzSliceJobs jy;
+                launch_band_b(L.d_parts, nbk, t, m, L.A, L.B, out.Acal, out.ZL, G, Z.W, Z.Y, Z.gam, Z.rho, Z.band, st));
+    OzSliceJobs jy = jobs0;
     jy.job[0] = job(Z.Y, Z.YT, Z.eYT, 5);
     Cost c2 = cs;
     c2.bytes *= nbk;
@@ -816,7 +825,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
     const int nbk = L.active_back[s];
     DM_LAUNCH(pf, st, K_BACK_FACTOR, L.c_back[s], nbk,
               launch_oz_step(2, L.d_parts, nbk, s, m, out, lexp[2], r0exp[2], r1exp[2], maps[2], L.d_err, st));
-    OzSliceJobs jb;
+    OzSliceJobs jb = jobs0;
     jb.job[0] = job(out.ZL, Z.ZLT, Z.eZLT, 6);
     jb.job[1] = job(out.ZR, Z.ZRT, Z.eZRT, 7);
     Cost c3 = cs;
@@ -867,7 +876,7 @@ static void factor_level_t(Level& L, cudaStream_t st, Prof& pf, Aux* aux) {
         const bool bh = L.oz.band && *L.oz.band_host <= kBandMax;
         DM_LAUNCH_K(pf, st, K_ASSEMBLE_H, bh ? Cost() : L.c_asm_h, L.nseps, 3,
                     launch_oz_assemble(L.d_seps, L.nseps, L.max_m, L.B, L.C, ZL, ZR, L.supp->A, L.supp->B, L.supp->C,
-                                       L.oz.as, L.oz.eA, L.oz.maps[1], L.d_err, L.oz.band, st));
+                                       L.oz.as, L.oz.eA, L.oz.maps[1], L.d_err, L.oz.gam, L.oz.band, st));
         if (L.oz.band) {  // the supplementary blocks when A and C are banded
           Cost cb;
           if (bh) {

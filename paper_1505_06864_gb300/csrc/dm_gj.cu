@@ -17,7 +17,9 @@
 // After the last panel the working matrix W satisfies D^{-1}[k][p_j] =
 // W[p_k][j]; k_gj_finish moves the entries there and writes the row slices of
 // the inverse.  The working matrix is a buffer per subsystem (rolling), so it
-// stays in L2 from step to step.
+// stays in L2 from step to step.  It holds D_t equilibrated, 2^-rho D 2^-gam with
+// the level's exponents per equation and unknown (dm_oz.cu), so that its digits
+// and its pivots see entries of one scale; k_gj_finish takes the exponents back.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -41,13 +43,15 @@ constexpr int kMaxChain = 8;           // most warps that run the pivot chain
 constexpr int kHelpers = 8;            // more warps for the rank-8 updates, beside the chain's
 
 __global__ void __launch_bounds__(256) k_gj_copy_b0(const PartDesc* __restrict__ parts, int m,
-                                                    const double* __restrict__ B, double* __restrict__ W) {
+                                                    const double* __restrict__ B, double* __restrict__ W,
+                                                    const int* __restrict__ gam, const int* __restrict__ rho) {
   const PartDesc p = parts[blockIdx.x];
   const long long mm = (long long)m * m;
   double* w = W + (long long)blockIdx.x * mm;
   const double* b = B + p.blk;
+  const int *gb = gam + p.blk / m, *rb = rho + p.blk / m;
   for (long long e = threadIdx.x + (long long)blockIdx.y * blockDim.x; e < mm; e += (long long)blockDim.x * gridDim.y)
-    w[e] = b[e];
+    w[e] = scale_pow2(b[e], -(rb[e / m] + gb[e % m]));
 }
 
 // What the chain's warps exchange per pivot (double-buffered by its parity).
@@ -518,7 +522,8 @@ __global__ void __launch_bounds__(32 * (CW + kHelpers + 1), 1)
   if (bad) atomicMin(status + p.sys, p.row0 + t + 1);
 }
 
-// After the last panel: D^{-1}[k][p_j] = W[p_k][j] moved to its place in G
+// After the last panel: X[k][p_j] = W[p_k][j], X = (2^-rho D 2^-gam)^{-1}, moved to its
+// place in G as D^{-1} = 2^-gam X 2^-rho
 // and the row slices of the block inverse G_t written (the left operand of
 // the next products), one pass: a CTA takes 32 rows of one block (blockIdx.x
 // = block * groups + group), a warp a row at a time: the row is read once,
@@ -528,8 +533,9 @@ template <int S>
 __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ parts, int t, int m,
                                                    const double* __restrict__ W, double* __restrict__ G,
                                                    const int* __restrict__ piv, __nv_bfloat16* __restrict__ Gs,
-                                                   int* __restrict__ eG) {
-  __shared__ int ip[kMaxM];
+                                                   int* __restrict__ eG, const int* __restrict__ gam,
+                                                   const int* __restrict__ rho) {
+  __shared__ int ip[kMaxM], rs[kMaxM];
   __shared__ double rowb[8][kMaxM];
   const int groups = (m + 31) / 32;
   const int q = blockIdx.x / groups, g = blockIdx.x - q * groups;
@@ -540,7 +546,9 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
   const double* M = W + (long long)q * mm;
   double* Gt = G + p.blk + (long long)t * mm;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int c = threadIdx.x; c < m; c += blockDim.x) ip[c] = piv[(long long)q * m + c];
+  const long long vt = p.blk / m + (long long)t * m;  // the block row's exponents
+  for (int c = threadIdx.x; c < m; c += blockDim.x) ip[c] = piv[(long long)q * m + c], rs[c] = rho[vt + c];
+  const int gv = 32 * g + lane < m ? gam[vt + 32 * g + lane] : 0;  // of the CTA's rows
   __syncthreads();
   double* rb = rowb[warp];
   const int rend = min(m, 32 * g + 32);
@@ -554,9 +562,11 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
     }
     hmax = __reduce_max_sync(0xffffffffu, hmax);
     const int e = scale_exponent(hmax);
-    if (lane == 0) eG[(long long)q * m + r] = e;
+    // the slices are of G_t 2^rho (dm_oz.cu) = 2^-gam X: X's digits
+    const int gr = __shfl_sync(0xffffffffu, gv, r - 32 * g);
+    if (lane == 0) eG[(long long)q * m + r] = e - gr;
     __syncwarp();
-    for (int c = lane; c < m; c += 32) Gt[(long long)r * m + c] = rb[c];
+    for (int c = lane; c < m; c += 32) Gt[(long long)r * m + c] = scale_pow2(rb[c], -(gr + rs[c]));
     for (int c0 = lane * 8; c0 < m; c0 += 256) {
       double v[8];
 #pragma unroll
@@ -580,9 +590,10 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
 // (working matrix W: D_t, written by launch B of the step before), as phases:
 // the copy of B_0, per panel of 32 columns the panel and its trailing update
 // (dm_oz.cu), and the finishing pass.
-void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, cudaStream_t st) {
+void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, const int* gam,
+                     const int* rho, cudaStream_t st) {
   if (nparts > 0 && t == 0)
-    gj::k_gj_copy_b0<<<dim3(nparts, std::max(1, m * m / 8192)), 256, 0, st>>>(parts, m, B, W);
+    gj::k_gj_copy_b0<<<dim3(nparts, std::max(1, m * m / 8192)), 256, 0, st>>>(parts, m, B, W, gam, rho);
 }
 
 void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, int* piv, void* Us,
@@ -608,14 +619,14 @@ void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, d
 }
 
 void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
-                      void* Gs, int* eG, cudaStream_t st) {
+                      void* Gs, int* eG, const int* gam, const int* rho, cudaStream_t st) {
   if (nparts <= 0) return;
   const int grid = nparts * ((m + 31) / 32);
   auto* g = static_cast<__nv_bfloat16*>(Gs);
   if (oz_slices(m) == 7)
-    gj::k_gj_finish<7><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG);
+    gj::k_gj_finish<7><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG, gam, rho);
   else
-    gj::k_gj_finish<8><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG);
+    gj::k_gj_finish<8><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG, gam, rho);
 }
 
 }  // namespace dm

@@ -158,6 +158,7 @@ struct OzOut {
   double *G, *Acal, *ZL, *ZR, *Y;  // Y: Y_{t+1} per subsystem (rolling, float64)
   double* W;       // working matrix of the blocked inversion per subsystem (rolling): D_{t+1} goes there (null: to G)
   const int* piv;  // the inversion's pivot rows [subsystem][m] (KIND 3)
+  const int *gam, *rho;  // exponents of the level's unknowns and equations [block][m]: D_{t+1} goes to W equilibrated
   // the supplementary blocks (Eq. e2311), one separator per CTA row
   const SepDesc* seps;
   double *HA, *HB, *HC;
@@ -190,9 +191,15 @@ struct OzAsm {
 };
 void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, const double* C, const double* ZL,
                         const double* ZR, double* HA, double* HB, double* HC, const OzAsm& a, const int* eA,
-                        const void* mapA, int* errflag, const int* band, cudaStream_t st);
-void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const int* band,
-                         cudaStream_t st);
+                        const void* mapA, int* errflag, const int* gam, const int* band, cudaStream_t st);
+void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const int* gam,
+                         const int* rho, const int* band, cudaStream_t st);
+// Exponents that equilibrate a level's unknowns (gam) and equations (rho),
+// both [block][m]: with the entries of A_i, B_i, C_i scaled by 2^-gam of their
+// unknown and 2^-rho of their equation every row's largest lies in [1/2, 1).
+// Folds the band of A and C into *band (null: not wanted; zeroed by the caller).
+void launch_level_scales(const SysDesc* sys, int nsys, const double* A, const double* B, const double* C, int nblocks,
+                         int m, int* gam, int* rho, int* band, cudaStream_t st);
 // The level's band into *band (atomicMax; the caller zeroes it first): the
 // largest |row - column| of a nonzero entry of the n entries of A and of C.
 void launch_band_detect(const double* A, const double* C, long long n, int m, int* band, cudaStream_t st);
@@ -202,8 +209,8 @@ void launch_band_detect(const double* A, const double* C, long long n, int m, in
 void launch_band_gc(const PartDesc* parts, int nparts, int t, int m, const double* G, const double* C, double* Acal,
                     double* ZR, const int* band, cudaStream_t st);
 void launch_band_b(const PartDesc* parts, int nparts, int t, int m, const double* A, const double* B,
-                   const double* Acal, const double* ZL, double* G, double* W, double* Y, const int* band,
-                   cudaStream_t st);
+                   const double* Acal, const double* ZL, double* G, double* W, double* Y, const int* gam,
+                   const int* rho, const int* band, cudaStream_t st);
 void launch_band_h(const SepDesc* seps, int nseps, int m, const double* A, const double* B, const double* C,
                    const double* ZL, const double* ZR, double* HA, double* HB, double* HC, const int* band,
                    cudaStream_t st);
@@ -216,6 +223,7 @@ struct OzSliceJob {
 struct OzSliceJobs {
   OzSliceJob job[4];
   const int* band = nullptr;  // kinds 2 and 3 (launch B's operands) are skipped when banded
+  const int *gam = nullptr, *rho = nullptr;  // the level's exponents (launch_level_scales)
 };
 void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, const OzSliceJobs& jobs, int njobs,
                           cudaStream_t st);
@@ -224,18 +232,19 @@ void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m
                     int aux = 0);
 // Blocked Gauss-Jordan inversion (dm_gj.cu) in the working matrices W
 // [nparts][m][m], with the rank-32 updates as digit-sliced tensor-core
-// products; maps2 = the panel-slice maps (U with 128-row boxes, V with
+// products; the blocks are inverted equilibrated, as 2^-rho D 2^-gam; maps2 = the panel-slice maps (U with 128-row boxes, V with
 // oz_box_rows_gj() rows), piv [nparts][m] (the pivot row of every column), Us /
 // Vs [nparts][7][m][32] bf16, Uexp / Vexp [nparts][m].  Phases: begin (t = 0
-// only: W = B_0), per panel panel and update, finish (the inverse to G_t, its
+// only: W = B_0, equilibrated), per panel panel and update, finish (the inverse to G_t, its
 // row slices to Gs [nparts][oz_slices(m)][m][m] bf16 / eG [nparts][m]).
-void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, cudaStream_t st);
+void launch_gj_begin(const PartDesc* parts, int nparts, int t, int m, const double* B, double* W, const int* gam,
+                     const int* rho, cudaStream_t st);
 void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, int* piv, void* Us,
                      int* Uexp, void* Vs, int* Vexp, int* status, cudaStream_t st);
 void launch_gj_update(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, const int* piv,
                       const int* Uexp, const int* Vexp, const void* maps2, int* errflag, cudaStream_t st);
 void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
-                      void* Gs, int* eG, cudaStream_t st);
+                      void* Gs, int* eG, const int* gam, const int* rho, cudaStream_t st);
 int tc2_ntile(int m);
 bool tc2_make_map(int mode, const void* base, long long blocks, int m, int box_rows, void* out);
 int tc2_map_bytes();

@@ -14,7 +14,18 @@
 //   (L R)[r][n] = 2^(e_r + f_n + 2) sum_{d=2..S+2} b^(-d) acc_d[r][n],
 //   acc_d = sum_{s+t=d} Lslice_s Rslice_t,
 //
-// keeping the slice pairs with s + t <= S + 2 (34 of 49 and 43 of 64).  The
+// The error of an entry is so bounded by the largest entries of the row and
+// the column, where a float64 dot product's is by its terms.  Where equations
+// or unknowns differ in scale, entry k of the row is large just where entry k
+// of the column is small, and one scale per row and column would lose the
+// small ones (m = 100, rows scaled over eight decades: solutions to 1e-11
+// against 1.5e-13).  So the operands are balanced along k by exact powers of
+// two, one per equation (rho) or unknown (gam) of a block row, found before
+// the sweeps (k_level_cols, k_level_rows): L[r][k] 2^(s_k) times 2^(-s_k) R[k][n],
+// inside the extraction of the digits.  The products' results, and all that is
+// stored in float64, are not scaled.
+//
+// Kept are the slice pairs with s + t <= S + 2 (34 of 49 and 43 of 64).  The
 // digits are balanced (|digit| <= b / 2), so each acc_d is an integer of at most
 // S K b^2 / 4 <= 2^24 for K <= 128 (S = 7) and K <= 512 (S = 8), and the
 // float32 accumulation in tensor memory is exact.  Operands are rounded at
@@ -349,8 +360,8 @@ __global__ void __launch_bounds__(threads_of(KIND, S), 1)
       // values the stores update (they do not depend on the products)
       const int rbase = w.tm * MT + quarter * 32, row = rbase + lane;
       const int cbase = w.tn * NTK + part * CW;  // the warp's columns
-      const int er = row < m ? lexp[(long long)w.zl * m + row] : 0;
-      const int fexp = lane < CW && cbase + lane < m ? rexp[(long long)w.zr * m + cbase + lane] : 0;
+      int er = row < m ? lexp[(long long)w.zl * m + row] : 0;
+      int fexp = lane < CW && cbase + lane < m ? rexp[(long long)w.zr * m + cbase + lane] : 0;
       const bool rmw = KIND == 2 && j == 0, dnext = KIND == 1 && j == 0, gj = KIND == 3, hb = KIND >= 4 && j == 0;
       const bool upd = rmw || dnext || gj || hb;
       const long long o = p.blk + (long long)t * mm;
@@ -360,6 +371,18 @@ __global__ void __launch_bounds__(threads_of(KIND, S), 1)
                           : gj   ? wk
                           : hb   ? (KIND == 4 ? out.B + sd.blk_q : out.HB + sd.hblk)
                                  : out.B + o + mm;
+      // D_{t+1} goes into the working matrix equilibrated (the exponents as the
+      // scales: of the lane's row, and a column of the warp's per lane): the
+      // product by its scales, B_{t+1} as it is loaded
+      const bool even = KIND == 1 && dnext && out.W != nullptr;
+      int rrow = 0, gcol = 0;
+      if (even) {
+        const long long v1 = (o + mm) / m;  // block row t + 1
+        if (row < m) rrow = out.rho[v1 + row];
+        if (lane < CW && cbase + lane < m) gcol = out.gam[v1 + cbase + lane];
+        er -= rrow;
+        fexp -= gcol;
+      }
       // where the results go
       double* dst;
       if (KIND >= 4)
@@ -387,6 +410,12 @@ __global__ void __launch_bounds__(threads_of(KIND, S), 1)
           const int rr = rbase + r0 + 4 * i;
           in[i] = (upd && n < m && rr < m && !(gj && ((zrows >> (r0 + 4 * i)) & 1u))) ? src[(long long)rr * m + n]
                                                                                       : 0.0;
+        }
+        if (even) {
+          const int gn = __shfl_sync(0xffffffffu, gcol, 8 * ci + cl);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            in[i] = scale_pow2(in[i], -(__shfl_sync(0xffffffffu, rrow, r0 + 4 * i) + gn));
         }
       };
       double in[8];
@@ -493,30 +522,50 @@ __global__ void __launch_bounds__(threads_of(KIND, S), 1)
 
 // ---------------------------------------------------------------- slicing
 // A CTA slices one group of 32 rows (left operands) or 32 columns (right
-// operands) of one float64 m x m block; a block takes ceil(m / 32) CTAs.
+// operands) of one float64 m x m block; a block takes ceil(m / 32) CTAs.  The
+// entries of index k (columns of a left operand, rows of a right one) take
+// part with 2^(sh.sign sh.kap[k]).  (Read beside the entries: staged in shared
+// memory, a load and a barrier ahead of them, they cost a launch of few blocks
+// 1 us.)
+struct Shift {
+  const int* kap;
+  int sign;
+  __device__ __forceinline__ int operator()(int k) const { return sign * __ldg(kap + k); }
+};
 
-// Row slices (left operands): exps[r] = e with |v| < 2^e for the row's
-// largest |v|; slice s element (r, k) at ((q * S + s) m + r) pitch + k, the
+// Key of the high word of an entry with shift s: keys are compared, and an
+// entry of key K is below 2^(K - 1022).
+constexpr int kNoKey = -(1 << 20);
+__device__ __forceinline__ int scale_key(uint32_t hi, int s) {
+  const int h = (int)(hi & 0x7fffffffu);
+  return h == 0 ? kNoKey : max(h >> 20, 1) + s;
+}
+__device__ __forceinline__ int key_exponent(int key) { return key == kNoKey ? 0 : key - 1022; }
+
+// Row slices (left operands): exps[r] = e with |v 2^shift| < 2^e for the row's
+// entries v; slice s element (r, k) at ((q * S + s) m + r) pitch + k, the
 // pitch m rounded up to 8 (16-byte rows for TMA; the columns past m are zero).
 // One warp per row, eight consecutive columns per lane.
 template <int S>
 __device__ __forceinline__ void slice_rows_group(const double* __restrict__ src, __nv_bfloat16* __restrict__ dst,
-                                                 long long qdst, int* __restrict__ exps, int m, int g) {
+                                                 long long qdst, int* __restrict__ exps, int m, int g,
+                                                 Shift sh) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int mp = slice_pitch(m);
   const unsigned long long* bits = reinterpret_cast<const unsigned long long*>(src);
   const int rend = min(m, 32 * g + 32);
   for (int r = 32 * g + warp; r < rend; r += nw) {
-    uint32_t hmax = 0;
-    for (int c = lane; c < m; c += 32) hmax = max(hmax, (uint32_t)(bits[(long long)r * m + c] >> 32) & 0x7fffffffu);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) hmax = max(hmax, __shfl_xor_sync(0xffffffffu, hmax, o));
-    const int e = scale_exponent(hmax);
+    int key = kNoKey;
+    for (int c = lane; c < m; c += 32) key = max(key, scale_key((uint32_t)(bits[(long long)r * m + c] >> 32), sh(c)));
+    const int e = key_exponent(__reduce_max_sync(0xffffffffu, key));
     if (lane == 0) exps[qdst * m + r] = e;
     for (int c0 = lane * 8; c0 < m; c0 += 256) {
       uint32_t q[8][S];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) digits<S>(c0 + u < m ? bits[(long long)r * m + c0 + u] : 0ull, e, q[u]);
+      for (int u = 0; u < 8; ++u) {
+        const bool in = c0 + u < m;
+        digits<S>(in ? bits[(long long)r * m + c0 + u] : 0ull, in ? e - sh(c0 + u) : e, q[u]);
+      }
 #pragma unroll
       for (int sl = 0; sl < S; ++sl) {
         uint4 w;
@@ -538,27 +587,30 @@ __device__ __forceinline__ void slice_rows_group(const double* __restrict__ src,
 template <int S>
 __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src, __nv_bfloat16* __restrict__ dst,
                                                  long long qdst, int* __restrict__ exps, int m, int g,
-                                                 uint32_t (*red)[32], int* s_e, unsigned long long (*tile)[33]) {
+                                                 Shift sh, int (*red)[32], int* s_e,
+                                                 unsigned long long (*tile)[33]) {
   const int mp = slice_pitch(m);
   const unsigned long long* bits = reinterpret_cast<const unsigned long long*>(src);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = 32 * g + lane;
-  uint32_t hmax = 0;
+  int key = kNoKey;
   if (n < m)
-    for (int k = warp; k < m; k += 8) hmax = max(hmax, (uint32_t)(bits[(long long)k * m + n] >> 32) & 0x7fffffffu);
-  red[warp][lane] = hmax;
+    for (int k = warp; k < m; k += 8) key = max(key, scale_key((uint32_t)(bits[(long long)k * m + n] >> 32), sh(k)));
+  red[warp][lane] = key;
   __syncthreads();
   if (warp == 0) {
-    uint32_t h = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) h = max(h, red[w][lane]);
-    const int e = scale_exponent(h);
+    for (int w = 0; w < 8; ++w) key = max(key, red[w][lane]);
+    const int e = key_exponent(key);
     s_e[lane] = e;
     if (n < m) exps[qdst * m + n] = e;
   }
   __syncthreads();
   const int nl = threadIdx.x >> 3, kq = (threadIdx.x & 7) * 4;
   for (int k0 = 0; k0 < m; k0 += 32) {
+    int sk[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sk[u] = sh(min(k0 + kq + u, m - 1));
     for (int y = warp; y < 32; y += 8) {
       const int k = k0 + y;
       tile[y][lane] = (k < m && n < m) ? bits[(long long)k * m + n] : 0ull;
@@ -568,7 +620,7 @@ __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src,
     if (nn < m && k < mp) {  // past m the tile holds zeros
       uint32_t q[4][S];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) digits<S>(tile[kq + u][nl], s_e[nl], q[u]);
+      for (int u = 0; u < 4; ++u) digits<S>(tile[kq + u][nl], s_e[nl] - sk[u], q[u]);
 #pragma unroll
       for (int sl = 0; sl < S; ++sl) {
         uint2 w;
@@ -581,16 +633,17 @@ __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src,
   }
 }
 
-// Slices of every block of a level's array (A as rows, C as transposed
-// columns): blockIdx.x = block * groups + group, looping past the grid.
+// Slices of every block of a level's array (A as rows, its columns the
+// unknowns of the block row before; C as transposed columns, its rows the
+// block row's equations): blockIdx.x = block * groups + group, looping past the grid.
 // With `band` set and the level's A and C banded (*band <= kBandMax), nothing
 // is done: only the tensor-core tiles the banded kernels replace read these.
 template <bool COLS, int S>
 __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__ src, int nblocks, int m,
                                                       __nv_bfloat16* __restrict__ dst, int* __restrict__ exps,
+                                                      const int* __restrict__ gam, const int* __restrict__ rho,
                                                       const int* __restrict__ band) {
-  __shared__ uint32_t red[8][32];
-  __shared__ int s_e[32];
+  __shared__ int red[8][32], s_e[32];
   __shared__ unsigned long long tile[32][33];
   if (band && *band <= kBandMax) return;
   const long long mm = (long long)m * m;
@@ -598,9 +651,9 @@ __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__
   for (long long i = blockIdx.x; i < (long long)nblocks * groups; i += gridDim.x) {
     const int q = (int)(i / groups), g = (int)(i - (long long)q * groups);
     if (COLS)
-      slice_cols_group<S>(src + q * mm, dst, q, exps, m, g, red, s_e, tile);
-    else
-      slice_rows_group<S>(src + q * mm, dst, q, exps, m, g);
+      slice_cols_group<S>(src + q * mm, dst, q, exps, m, g, Shift{rho + (long long)q * m, -1}, red, s_e, tile);
+    else  // the first block row has no unknowns before it
+      slice_rows_group<S>(src + q * mm, dst, q, exps, m, g, Shift{gam + (long long)max(q - 1, 0) * m, q > 0 ? -1 : 0});
     __syncthreads();
   }
 }
@@ -611,12 +664,14 @@ __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__
 //   4 ZR_{L-1} columns (last row, right spike) -> slot;  5 Y_{t+1} columns -> rolling (q);
 //   6 ZL_t columns, backward step;        7 ZR_t columns, backward step;
 //   8 Y_0 = A_first columns -> rolling (q), at the start of a factorisation.
+// Index k runs over the equations of block row t in G_t's columns and C_t's
+// and Y_t's rows, over the unknowns of block row t in the columns of A_{t+1}
+// and Acal_{t-1} and the rows of Acal_t, ZL_t, ZR_t.
 // Several per-subsystem slicing jobs in one launch (blockIdx.y = job).
 template <int S>
 __global__ void __launch_bounds__(256) k_oz_slice_jobs(const PartDesc* __restrict__ parts, int step, int m,
                                                        OzSliceJobs jobs) {
-  __shared__ uint32_t red[8][32];
-  __shared__ int s_e[32];
+  __shared__ int red[8][32], s_e[32];
   __shared__ unsigned long long tile[32][33];
   const OzSliceJob& jb = jobs.job[blockIdx.y];
   const int groups = (m + 31) / 32;
@@ -643,10 +698,16 @@ __global__ void __launch_bounds__(256) k_oz_slice_jobs(const PartDesc* __restric
   if (jobs.band && *jobs.band <= kBandMax && (jb.kind == 2 || (jb.kind == 3 && t < p.L - 1))) act = false;
   if (!act) return;
   __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(jb.dst);
+  const long long bt = p.blk / mm + t;  // the block row
+  const Shift sh = jb.kind == 0   ? Shift{jobs.rho + bt * m, 1}
+                   : jb.kind == 1 ? Shift{jobs.gam + (bt + 1) * m, -1}
+                   : jb.kind == 5 ? Shift{jobs.rho + (bt + 1) * m, -1}
+                   : jb.kind == 8 ? Shift{jobs.rho + sblk * m, -1}
+                                  : Shift{jobs.gam + bt * m, 1};
   if (jb.kind == 0 || jb.kind == 1)
-    slice_rows_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g);
+    slice_rows_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g, sh);
   else
-    slice_cols_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g, red, s_e, tile);
+    slice_cols_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g, sh, red, s_e, tile);
 }
 
 // The assembly's operands per separator s (blockIdx.x = s * groups + group,
@@ -658,22 +719,24 @@ __global__ void __launch_bounds__(256) k_oz_slice_seps(const SepDesc* __restrict
                                                        const double* __restrict__ C, const double* __restrict__ ZL,
                                                        const double* __restrict__ ZR, __nv_bfloat16* __restrict__ Cq,
                                                        int* __restrict__ eCq, __nv_bfloat16* __restrict__ Sp,
-                                                       int* __restrict__ eS, const int* __restrict__ band) {
-  __shared__ uint32_t red[8][32];
-  __shared__ int s_e[32];
+                                                       int* __restrict__ eS, const int* __restrict__ gam,
+                                                       const int* __restrict__ band) {
+  __shared__ int red[8][32], s_e[32];
   __shared__ unsigned long long tile[32][33];
   if (band && *band <= kBandMax) return;  // the banded assembly needs no slices
   const int groups = (m + 31) / 32;
   const int s = blockIdx.x / groups, g = blockIdx.x - s * groups, job = blockIdx.y;
   const SepDesc sd = seps[s];
+  const long long mm = (long long)m * m;
   if (job == 0) {
-    slice_rows_group<S>(C + sd.blk_q, Cq, s, eCq, m, g);
+    slice_rows_group<S>(C + sd.blk_q, Cq, s, eCq, m, g, Shift{gam + sd.blk_next / mm * m, -1});
     return;
   }
   if ((job == 2 && !(sd.flags & HAS_HA)) || (job == 4 && !(sd.flags & HAS_HC))) return;
   const double* src = job == 1 ? ZR + sd.blk_prev : job == 2 ? ZL + sd.blk_prev : job == 3 ? ZL + sd.blk_next
                                                                                          : ZR + sd.blk_next;
-  slice_cols_group<S>(src, Sp, 4LL * s + job - 1, eS, m, g, red, s_e, tile);
+  slice_cols_group<S>(src, Sp, 4LL * s + job - 1, eS, m, g,
+                      Shift{gam + (job <= 2 ? sd.blk_prev : sd.blk_next) / mm * m, 1}, red, s_e, tile);
 }
 
 // ---------------------------------------------------------------- banded operands
@@ -745,7 +808,8 @@ __global__ void __launch_bounds__(256) k_band_b(const PartDesc* __restrict__ par
                                                 const double* __restrict__ A, const double* __restrict__ B,
                                                 const double* __restrict__ Acal, const double* __restrict__ ZL,
                                                 double* __restrict__ G, double* __restrict__ W,
-                                                double* __restrict__ Y, const int* __restrict__ band) {
+                                                double* __restrict__ Y, const int* __restrict__ gam,
+                                                const int* __restrict__ rho, const int* __restrict__ band) {
   __shared__ double lb[32][2 * kBandMax + 1];
   const int w = *band;
   if (w > kBandMax) return;
@@ -763,8 +827,8 @@ __global__ void __launch_bounds__(256) k_band_b(const PartDesc* __restrict__ par
     for (int n = lane; n < m; n += 32) {
       const double v = band_row(lb[r - 32 * g], X, r, n, m, w);
       const long long e = (long long)r * m + n;
-      if (j == 0)
-        D[e] = B[o + mm + e] - v;           // D_{t+1}
+      if (j == 0)  // D_{t+1}, equilibrated in the working matrix
+        D[e] = W ? scale_pow2(B[o + mm + e] - v, -(rho[(o + mm) / m + r] + gam[(o + mm) / m + n])) : B[o + mm + e] - v;
       else
         Y[(long long)q * mm + e] = -v;      // Y_{t+1}
     }
@@ -800,6 +864,99 @@ __global__ void __launch_bounds__(256) k_band_h(const SepDesc* __restrict__ seps
       else
         HC[sd.hblk + e] = -band_row(cb[rl], ZR + sd.blk_next, r, n, m, w);
     }
+}
+
+// ---------------------------------------------------------------- scales of equations and unknowns
+// Exponents that equilibrate a level: gam per unknown, of the largest entry in
+// its column of [C_{i-1}; B_i; A_{i+1}], then rho per equation, of the largest
+// entry of its row of [A_i B_i C_i] with the columns so scaled.  Columns first,
+// since partial pivoting (down the columns) does not see their scales: with
+// them the digit-sliced elimination gave float64's errors or smaller ones for
+// dense, banded and Laplace blocks with rows, columns or both scaled over 0 to 12
+// decades (m = 33 to 129, a numpy restatement); rows first cost two digits where
+// the unknowns are scaled, one pass for both (or a 2^6 limit on the spread, as a
+// switch to float64 products) more.  Two passes over the blocks, each bound by
+// reading them.
+
+// Block row b = blockIdx.x, columns 32 blockIdx.y ..: a lane per column, eight
+// warps over the rows.  Also folds the largest |row - column| of a nonzero entry
+// (any bit but the sign set) of A and C into *band (if not null).
+__device__ __forceinline__ int sys_of_row(const SysDesc* __restrict__ sys, int nsys, int row) {
+  int lo = 0, hi = nsys - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (sys[mid].row0 <= row) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(256) k_level_cols(const SysDesc* __restrict__ sys, int nsys,
+                                                    const double* __restrict__ A, const double* __restrict__ B,
+                                                    const double* __restrict__ C, int m, int* __restrict__ gam,
+                                                    int* __restrict__ band) {
+  __shared__ int red[8][32], swid[8];
+  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = 32 * blockIdx.y + lane;
+  const SysDesc& sd = sys[sys_of_row(sys, nsys, b)];
+  const bool up = b > sd.row0, down = b < sd.row0 + sd.N - 1;
+  const long long mm = (long long)m * m;
+  int key = kNoKey, wid = 0;
+  auto column = [&](const double* M, bool banded) {
+    const unsigned long long* v = reinterpret_cast<const unsigned long long*>(M) + n;
+#pragma unroll 8
+    for (int k = warp; k < m; k += 8) {
+      const unsigned long long x = __ldg(v + (long long)k * m);
+      key = max(key, scale_key((uint32_t)(x >> 32), 0));
+      if (banded && (x << 1) != 0) wid = max(wid, abs(k - n));
+    }
+  };
+  if (n < m) {
+    column(B + b * mm, false);
+    if (up) column(C + (b - 1) * mm, true);
+    if (down) column(A + (b + 1) * mm, true);
+  }
+  red[warp][lane] = key;
+  wid = __reduce_max_sync(0xffffffffu, wid);
+  if (lane == 0) swid[warp] = wid;
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) key = max(key, red[w][lane]), wid = max(wid, swid[w]);
+    if (n < m) gam[(long long)b * m + n] = key_exponent(key);
+    if (band && lane == 0 && wid > *(volatile int*)band) atomicMax(band, wid);
+  }
+}
+
+// Block row b = blockIdx.x, rows 32 blockIdx.y ..: a warp a row at a time.
+__global__ void __launch_bounds__(256) k_level_rows(const SysDesc* __restrict__ sys, int nsys,
+                                                    const double* __restrict__ A, const double* __restrict__ B,
+                                                    const double* __restrict__ C, int m, const int* __restrict__ gam,
+                                                    int* __restrict__ rho) {
+  __shared__ int g[3][kMaxM];
+  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const SysDesc& sd = sys[sys_of_row(sys, nsys, b)];
+  const bool up = b > sd.row0, down = b < sd.row0 + sd.N - 1;
+  const long long mm = (long long)m * m;
+  for (int k = threadIdx.x; k < m; k += 256) {
+    const int* gb = gam + (long long)b * m + k;
+    g[0][k] = up ? gb[-m] : 0;
+    g[1][k] = gb[0];
+    g[2][k] = down ? gb[m] : 0;
+  }
+  __syncthreads();
+  const int r0 = 32 * blockIdx.y, rend = min(m, r0 + 32);
+  for (int r = r0 + warp; r < rend; r += 8) {
+    int key = kNoKey;
+    auto row = [&](const double* M, const int* gk) {
+      const unsigned long long* v = reinterpret_cast<const unsigned long long*>(M) + (long long)r * m;
+#pragma unroll 8
+      for (int c = lane; c < m; c += 32) key = max(key, scale_key((uint32_t)(__ldg(v + c) >> 32), -gk[c]));
+    };
+    row(B + b * mm, g[1]);
+    if (up) row(A + b * mm, g[0]);
+    if (down) row(C + b * mm, g[2]);
+    key = __reduce_max_sync(0xffffffffu, key);
+    if (lane == 0) rho[(long long)b * m + r] = key_exponent(key);
+  }
 }
 
 // The level's band: the largest |row - column| of a nonzero entry (any bit
@@ -880,17 +1037,25 @@ void launch_band_detect(const double* A, const double* C, long long n, int m, in
   oz::k_band_detect<<<152 * 8, 256, 0, st>>>(A, C, n, m, band);
 }
 
-void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const int* band,
-                         cudaStream_t st) {
+void launch_level_scales(const SysDesc* sys, int nsys, const double* A, const double* B, const double* C, int nblocks,
+                         int m, int* gam, int* rho, int* band, cudaStream_t st) {
+  if (nblocks <= 0) return;
+  const dim3 grid(nblocks, (m + 31) / 32);
+  oz::k_level_cols<<<grid, 256, 0, st>>>(sys, nsys, A, B, C, m, gam, band);
+  oz::k_level_rows<<<grid, 256, 0, st>>>(sys, nsys, A, B, C, m, gam, rho);
+}
+
+void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const int* gam,
+                         const int* rho, const int* band, cudaStream_t st) {
   if (nblocks <= 0) return;
   const long long work = (long long)nblocks * ((m + 31) / 32);
   const int grid = (int)std::min<long long>(work, 152LL * 16);
   auto* d = static_cast<__nv_bfloat16*>(dst);
   const bool s7 = oz_slices(m) == 7;
-  if (cols && s7) oz::k_oz_slice_all<true, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
-  else if (cols) oz::k_oz_slice_all<true, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
-  else if (s7) oz::k_oz_slice_all<false, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
-  else oz::k_oz_slice_all<false, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, band);
+  if (cols && s7) oz::k_oz_slice_all<true, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
+  else if (cols) oz::k_oz_slice_all<true, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
+  else if (s7) oz::k_oz_slice_all<false, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
+  else oz::k_oz_slice_all<false, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
 }
 
 void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, const OzSliceJobs& jobs, int njobs,
@@ -961,14 +1126,14 @@ void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m
 
 void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, const double* C, const double* ZL,
                         const double* ZR, double* HA, double* HB, double* HC, const OzAsm& a, const int* eA,
-                        const void* mapA, int* errflag, const int* band, cudaStream_t st) {
+                        const void* mapA, int* errflag, const int* gam, const int* band, cudaStream_t st) {
   if (nseps <= 0) return;
   const dim3 sgrid(nseps * ((m + 31) / 32), 5);
   auto *cq = static_cast<__nv_bfloat16*>(a.Cq), *sp = static_cast<__nv_bfloat16*>(a.S);
   if (oz_slices(m) == 7)
-    oz::k_oz_slice_seps<7><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, band);
+    oz::k_oz_slice_seps<7><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, gam, band);
   else
-    oz::k_oz_slice_seps<8><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, band);
+    oz::k_oz_slice_seps<8><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, gam, band);
   OzOut out{};
   out.B = B;
   out.seps = seps;
@@ -998,10 +1163,10 @@ void launch_band_gc(const PartDesc* parts, int nparts, int t, int m, const doubl
 }
 
 void launch_band_b(const PartDesc* parts, int nparts, int t, int m, const double* A, const double* B,
-                   const double* Acal, const double* ZL, double* G, double* W, double* Y, const int* band,
-                   cudaStream_t st) {
+                   const double* Acal, const double* ZL, double* G, double* W, double* Y, const int* gam,
+                   const int* rho, const int* band, cudaStream_t st) {
   if (nparts <= 0 || !band) return;
-  oz::k_band_b<<<dim3(nparts * ((m + 31) / 32), 2), 256, 0, st>>>(parts, t, m, A, B, Acal, ZL, G, W, Y, band);
+  oz::k_band_b<<<dim3(nparts * ((m + 31) / 32), 2), 256, 0, st>>>(parts, t, m, A, B, Acal, ZL, G, W, Y, gam, rho, band);
 }
 
 void launch_band_h(const SepDesc* seps, int nseps, int m, const double* A, const double* B, const double* C,

@@ -98,6 +98,10 @@ struct OzLevel {
   void *AcalT = nullptr, *YT = nullptr, *ZLT = nullptr, *ZRT = nullptr;
   int *eA = nullptr, *eCT = nullptr, *eAcal = nullptr, *eG = nullptr;
   int *eAcalT = nullptr, *eYT = nullptr, *eZLT = nullptr, *eZRT = nullptr;
+  // exponents of the unknowns and of the equations ([block][m]), found at the
+  // start of each factorisation: what the slices are balanced by and the
+  // blocks inverted with
+  int *gam = nullptr, *rho = nullptr;
   double* Y = nullptr;
   // tensor maps: left G, A, Acal; right CT, YT, AcalT, ZLT, ZRT
   alignas(64) unsigned char maps[8][128];

@@ -17,7 +17,8 @@ __device__ __forceinline__ long long scaled_integer(unsigned long long bits, int
   const int ex = (int)((bits >> 52) & 0x7ff);
   const unsigned long long mant = (bits & 0xfffffffffffffull) | (ex ? (1ull << 52) : 0ull);
   // (mant 8 >> n) / 2, rounded: |v| < 2^e leaves n >= 0, and from n = 56 on nothing is left
-  const int n = min(e + 1022 - (ex ? ex : 1), 62);
+  // (nor of a subnormal v where e < -1021)
+  const int n = (int)min((unsigned)(e + 1022 - (ex ? ex : 1)), 62u);
   const unsigned long long Y = (((mant << 3) >> n) + 1) >> 1;
   return (long long)((bits >> 63) ? 0ull - Y : Y);
 }
@@ -72,6 +73,14 @@ __device__ __forceinline__ double round_scaled(long long T, int s, bool& odd) {
   odd = odd || (a != 0 && (unsigned)ex > 2044u);
   const unsigned long long r = ((unsigned long long)T & 0x8000000000000000ull) + ((unsigned long long)ex << 52) + mant;
   return __longlong_as_double(a == 0 ? 0ll : (long long)r);
+}
+
+// v 2^k exactly (rounded where the result is subnormal), without float64
+// instructions while it is a normal number.
+__device__ __forceinline__ double scale_pow2(double v, int k) {
+  const int hi = __double2hiint(v), lo = __double2loint(v), ex = (hi >> 20) & 0x7ff;
+  if ((unsigned)(ex - 1) < 2046u && (unsigned)(ex + k - 1) < 2046u) return __hiloint2double(hi + k * (1 << 20), lo);
+  return ((hi << 1) | lo) == 0 ? v : ldexp(v, k);
 }
 
 // Two bf16 values (high halves of a and b) in one register, a first.
