@@ -122,11 +122,16 @@ int dm_plan(dm_plan_t* out, int N, int m, int nrhs, int P, int levels, int preci
  * (integers of at most 2^24 in float32), and the sums are combined in 64-bit
  * integers: an error per entry below m 2^-53 max|row| max|column|.  Before
  * they are cut, the operands are balanced by exact powers of two, one per
- * equation and one per unknown, found from the level's blocks at the start of
- * dm_factor, and the blocks are inverted so equilibrated: equations and
- * unknowns of different scale cost no accuracy (what is bounded by the largest
- * entries is so after the scaling; an entry far below them is not resolved
- * relative to itself, as in a float64 dot product of few terms it would be).
+ * equation and one per unknown, found from the largest entries of the level's
+ * blocks at the start of dm_factor, and the blocks are inverted equilibrated,
+ * so that equations and unknowns of different scale cost no accuracy.  Where
+ * the scales cannot be told from the largest entries (sparse blocks with
+ * fields of different units side by side), the level and those below it
+ * take the float64 products of DM_PLAN_FP64_FMA, several times slower: the
+ * first such factorisation of a plan runs twice, the following ones start
+ * there, and the result is the same.  Such a jump in opposite directions on
+ * equations and unknowns of less than 2^13 is not told from an ordinary
+ * block and can cost 40 times the float64 products' error (7e-14).
  * DM_PLAN_FP64_FMA keeps the products on the float64 pipe; so does a plan with
  * m % 8 != 0 or m > 256 whose slices (about as much again as its factors) do
  * not fit the device memory free at dm_plan (several times slower, and in

@@ -322,7 +322,7 @@ static bool small_wanted(const Level& L) {
 
 static size_t oz_bytes(long long nblk, int nparts, int nseps, int m) {
   const size_t mm = (size_t)m * m, sl = (size_t)oz_slice_blocks_bytes(m), nb = nblk / mm, np = std::max(1, nparts);
-  return 2 * nb * m * sizeof(int) + (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + 2 * np * mm * sizeof(double) +
+  return 4 * nb * m * sizeof(int) + (3 * nb + 7 * np + 5 * (size_t)nseps) * (sl + m * sizeof(int)) + 2 * np * mm * sizeof(double) +
          np * ((size_t)2 * 7 * m * 32 * 2 + 3 * m * sizeof(int));
 }
 
@@ -394,24 +394,28 @@ int Level::allocate() {
   DM_ALLOC(d_sys, std::max<size_t>(1, sysd.size()) * sizeof(SysDesc));
   DM_ALLOC(status, std::max(1, nsys) * sizeof(int));
   DM_ALLOC(d_err, sizeof(int));
-  // where the band of A and C is detected (unless DM_BANDED=0)
-  auto alloc_band = [&]() -> int {
+  // what a factorisation finds out about the level's blocks: whether their
+  // scales are uneven, and the band of A and C (unless DM_BANDED=0)
+  auto alloc_found = [&]() -> int {
     OzLevel& Z = oz;
     const char* eb = std::getenv("DM_BANDED");
+    DM_ALLOC(Z.uneven, 2 * sizeof(int));
+    if (cudaHostAlloc(reinterpret_cast<void**>(&Z.uneven_host), 2 * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+      cudaGetLastError();
+      return set_error(DM_ENOMEM, "cudaHostAlloc of 8 bytes failed");
+    }
+    Z.uneven_host[0] = 0;
     if (!(eb && std::strcmp(eb, "0") == 0)) {
-      DM_ALLOC(Z.band, sizeof(int));
+      Z.band = Z.uneven + 1;
+      Z.band_host = Z.uneven_host + 1;
       cudaMemset(Z.band, 0x7f, sizeof(int));  // "not banded" until a factorisation finds out
-      if (cudaHostAlloc(reinterpret_cast<void**>(&Z.band_host), sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        return set_error(DM_ENOMEM, "cudaHostAlloc of 4 bytes failed");
-      }
       *Z.band_host = kBandMax + 1;
     }
     return DM_OK;
   };
   small = small_wanted(*this);
   // large enough that a band saves more than its detection costs
-  if (small && uniform_m(spec, max_m) && max_m >= 16 && (rc = alloc_band())) return rc;
+  if (small && uniform_m(spec, max_m) && max_m >= 16 && (rc = alloc_found())) return rc;
   if (tc_mode >= 0 && tc2_wanted(*this)) {
     // operand copies and tensor maps of the tensor-core step kernels
     Tc2Level& T = tc2;
@@ -470,8 +474,10 @@ int Level::allocate() {
     DM_ALLOC(Z.eZLT, 2 * np * ex);
     DM_ALLOC(Z.eZRT, 2 * np * ex);
     DM_ALLOC(Z.Y, np * mm * sizeof(double));
-    DM_ALLOC(Z.gam, nb * ex);
-    DM_ALLOC(Z.rho, nb * ex);
+    DM_ALLOC(Z.sc.be, 4 * nb * ex);
+    Z.sc.gam = Z.sc.be + nb * m;
+    Z.sc.rho = Z.sc.gam + nb * m;
+    Z.sc.bu = Z.sc.rho + nb * m;
     const void* lbase[3] = {Z.G, Z.A, Z.Acal};
     const long long lblk[3] = {np, nb, nb};
     const void* rbase[5] = {Z.CT, Z.YT, Z.AcalT, Z.ZLT, Z.ZRT};
@@ -494,7 +500,7 @@ int Level::allocate() {
       if (!ok) return set_error(DM_ECUDA, "tensor map creation for the blocked inversion failed (m = %d)", m);
       Z.gj = true;
     }
-    if ((rc = alloc_band())) return rc;
+    if ((rc = alloc_found())) return rc;
     if (nseps > 0 && oz_asm_wanted()) {
       OzAsm& a = Z.as;
       DM_ALLOC(a.Cq, nseps * sl);
@@ -558,7 +564,7 @@ void Level::release(void* p) {
 
 Level::~Level() {
   for (void* p : owned) cudaFree(p);
-  if (oz.band_host) cudaFreeHost(oz.band_host);
+  if (oz.uneven_host) cudaFreeHost(oz.uneven_host);
 }
 
 // ---------------------------------------------------------------------------
@@ -697,6 +703,21 @@ static void factor_level_tc2(Level& L, cudaStream_t st, Prof& pf) {
               launch_tc2_step(mode, 2, L.d_parts, L.active_back[s], s, m, lo[2], out, maps[2], L.d_err, st));
 }
 
+// The scales and the band of a level whose products may be digit-sliced,
+// before anything else of its factorisation (also where it runs its float64
+// products, so that it is known whether they are needed still).
+static void scan_level(Level& L, cudaStream_t st, Prof& pf) {
+  OzLevel& Z = L.oz;
+  const int m = L.max_m;
+  Cost c;
+  c.bytes = 48.0 * L.nblk;
+  DM_LAUNCH_K(pf, st, K_TC_CONVERT, c, 1, 3,
+              (cudaMemsetAsync(Z.uneven, 0, 2 * sizeof(int), st),
+               launch_level_scales(L.d_sys, L.nsys, L.A, L.B, L.C, (int)(L.nblk / ((long long)m * m)), m, Z.sc, Z.uneven,
+                                   Z.band, st),
+               cudaMemcpyAsync(Z.uneven_host, Z.uneven, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)));
+}
+
 // Forward and backward sweeps of a float64 level with its block products on
 // the tensor cores by digit slicing (dm_oz.cu): the scales of its equations
 // and unknowns, slices of A (rows), C^T and
@@ -718,8 +739,8 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
   out.ZR = static_cast<double*>(L.ZR);
   out.Y = Z.Y;
   out.W = Z.W;
-  out.gam = Z.gam;
-  out.rho = Z.rho;
+  out.gam = Z.sc.gam;
+  out.rho = Z.sc.rho;
   out.band = Z.band;
   // banded A and C as the previous factorisation found them (profiling costs
   // only: the kernels read the flag this factorisation's slicing sets)
@@ -741,18 +762,13 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
   const int* r0exp[3] = {Z.eCT, Z.eAcalT, Z.eZLT};
   const int* r1exp[3] = {Z.eYT, Z.eZLT, Z.eZRT};
   OzSliceJobs jobs0;
-  jobs0.gam = Z.gam;
-  jobs0.rho = Z.rho;
+  jobs0.bu = Z.sc.bu;
+  jobs0.be = Z.sc.be;
   auto job = [](const double* src, void* dst, int* e, int kind) { return OzSliceJob{src, dst, e, kind}; };
-  Cost cscale;
-  cscale.bytes = 48.0 * L.nblk;
-  DM_LAUNCH_K(pf, st, K_TC_CONVERT, cscale, 1, 2,
-              (Z.band ? (void)cudaMemsetAsync(Z.band, 0, sizeof(int), st) : (void)0,
-               launch_level_scales(L.d_sys, L.nsys, L.A, L.B, L.C, (int)nb, m, Z.gam, Z.rho, Z.band, st)));
+  scan_level(L, st, pf);
   auto slice_inputs = [&] {
-    launch_oz_slice_all(false, L.A, (int)nb, m, Z.A, Z.eA, Z.gam, Z.rho, Z.band, st);
-    launch_oz_slice_all(true, L.C, (int)nb, m, Z.CT, Z.eCT, Z.gam, Z.rho, Z.band, st);
-    if (Z.band) cudaMemcpyAsync(Z.band_host, Z.band, sizeof(int), cudaMemcpyDeviceToHost, st);
+    launch_oz_slice_all(false, L.A, (int)nb, m, Z.A, Z.eA, Z.sc, Z.band, st);
+    launch_oz_slice_all(true, L.C, (int)nb, m, Z.CT, Z.eCT, Z.sc, Z.band, st);
     OzSliceJobs j0 = jobs0;
     j0.job[0] = job(L.A, Z.YT, Z.eYT, 8);
     launch_oz_slice_jobs(L.d_parts, L.nparts, 0, m, j0, 1, st);
@@ -771,7 +787,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
       Cost cb, cf;
       cb.bytes = np * 16.0 * m * m;           // B_0 read, written to G
       cf.bytes = np * (16.0 + 2.0 * oz_slices(m)) * m * m;  // G_t read and written, its bf16 slices written
-      if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, Z.W, Z.gam, Z.rho, st));
+      if (t == 0) DM_LAUNCH(pf, st, K_INV, cb, np, launch_gj_begin(L.d_parts, np, t, m, L.B, Z.W, Z.sc.gam, Z.sc.rho, st));
       for (int k0 = 0; k0 < m; k0 += 32) {
         const double kw = std::min(32, m - k0);
         Cost cp, cu;
@@ -785,7 +801,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
           DM_LAUNCH(pf, st, K_INV_UPDATE, cu, np,
                     launch_gj_update(L.d_parts, np, t, m, k0 / 32, Z.W, Z.piv, Z.eU, Z.eV, Z.gj_maps, L.d_err, st));
       }
-      DM_LAUNCH(pf, st, K_INV, cf, np, launch_gj_finish(L.d_parts, np, t, m, Z.W, G, Z.piv, Z.G, Z.eG, Z.gam, Z.rho, st));
+      DM_LAUNCH(pf, st, K_INV, cf, np, launch_gj_finish(L.d_parts, np, t, m, Z.W, G, Z.piv, Z.G, Z.eG, Z.sc, st));
     } else {
       DM_LAUNCH(pf, st, K_INV, L.c_inv[t], np, launch_inv<double>(L.d_parts, np, t, L.B, G, L.status, L.max_m, st));
       OzSliceJobs jg = jobs0;
@@ -814,7 +830,7 @@ static void factor_level_oz(Level& L, cudaStream_t st, Prof& pf) {
               launch_oz_step(1, L.d_parts, nbk, t, m, out, lexp[1], r0exp[1], r1exp[1], maps[1], L.d_err, st));
     if (Z.band)  // both products of launch B when A is banded
       DM_LAUNCH(pf, st, K_BANDED, band_cost(nbk, 2), nbk,
-                launch_band_b(L.d_parts, nbk, t, m, L.A, L.B, out.Acal, out.ZL, G, Z.W, Z.Y, Z.gam, Z.rho, Z.band, st));
+                launch_band_b(L.d_parts, nbk, t, m, L.A, L.B, out.Acal, out.ZL, G, Z.W, Z.Y, Z.sc.gam, Z.sc.rho, Z.band, st));
     OzSliceJobs jy = jobs0;
     jy.job[0] = job(Z.Y, Z.YT, Z.eYT, 5);
     Cost c2 = cs;
@@ -870,13 +886,14 @@ static void factor_level_t(Level& L, cudaStream_t st, Prof& pf, Aux* aux) {
                                        L.supp->C, st));
       return;
     }
-    if (L.oz.on) {
+    if (L.oz.on && L.oz.fp64_now) scan_level(L, st, pf);
+    if (L.oz.on && !L.oz.fp64_now) {
       factor_level_oz(L, st, pf);
       if (L.supp && L.oz.asm_on) {
         const bool bh = L.oz.band && *L.oz.band_host <= kBandMax;
         DM_LAUNCH_K(pf, st, K_ASSEMBLE_H, bh ? Cost() : L.c_asm_h, L.nseps, 3,
                     launch_oz_assemble(L.d_seps, L.nseps, L.max_m, L.B, L.C, ZL, ZR, L.supp->A, L.supp->B, L.supp->C,
-                                       L.oz.as, L.oz.eA, L.oz.maps[1], L.d_err, L.oz.gam, L.oz.band, st));
+                                       L.oz.as, L.oz.eA, L.oz.maps[1], L.d_err, L.oz.sc.bu, L.oz.band, st));
         if (L.oz.band) {  // the supplementary blocks when A and C are banded
           Cost cb;
           if (bh) {
@@ -1017,6 +1034,13 @@ void solve_level(Level& L, const double* F, double* X, cudaStream_t st, Prof& pf
     solve_level_t<float>(L, F, X, st, pf);
   else
     solve_level_t<double>(L, F, X, st, pf);
+}
+
+// The first level whose scales the last factorisation found too ambiguous for
+// digit products (its stream is synchronised); kNoLevel: none.
+static int first_uneven(const Level& L) {
+  if (L.oz.on && *L.oz.uneven_host) return L.depth;
+  return L.supp ? first_uneven(*L.supp) : kNoLevel;
 }
 
 // first failing block row per system (host check after a factorisation)
@@ -1274,7 +1298,7 @@ Plan::~Plan() {
 }
 
 void Plan::reset_graphs() {
-  for (GraphCache* g : {&g_factor, &g_solve, &g_iter_first, &g_iter_next}) {
+  for (GraphCache* g : {&g_factor, &g_factor64, &g_solve, &g_iter_first, &g_iter_next}) {
     if (g->exec) cudaGraphExecDestroy(g->exec);
     *g = GraphCache();
   }
@@ -1299,14 +1323,42 @@ int Plan::factor(const double* A, const double* B, const double* C) {
     if ((rc = copy_in(top.B, B, top.nblk * sizeof(double), st))) return rc;
     if ((rc = copy_in(top.C, C, top.nblk * sizeof(double), st))) return rc;
   }
-  rc = run(g_factor, [&] {
+  // Uneven levels, and those below them, need float64 products.  That is known
+  // once the factorisation has run; so it starts as the last one ended, which
+  // the next system of a sequence shares as a rule, and where that was wrong
+  // runs again: first with digit products on every level, then with float64
+  // ones from the first uneven level on (the levels above it, and so what its
+  // scan sees, are then the same).  The result does not depend on where it
+  // started.
+  factored = false;
+  auto completed = [&] { return rc == DM_OK || rc == DM_ESINGULAR; };
+  rc = run_factor(fp64_from);
+  if (completed() && fp64_from != kNoLevel && first_uneven(top) != fp64_from) {
+    fp64_from = kNoLevel;
+    rc = run_factor(kNoLevel);
+  }
+  if (completed() && fp64_from == kNoLevel && first_uneven(top) != kNoLevel) {
+    fp64_from = first_uneven(top);
+    rc = run_factor(fp64_from);
+  }
+  factored = (rc == DM_OK);
+  return rc;
+}
+
+// One factorisation, the digit-sliced levels from depth `from` on with float64
+// products, and its status.
+int Plan::run_factor(int from) {
+  for (Level* l = &top; l; l = l->supp.get()) l->oz.fp64_now = l->depth >= from;
+  if (from != kNoLevel && from != g_factor64_from) {
+    if (g_factor64.exec) cudaGraphExecDestroy(g_factor64.exec);
+    g_factor64 = GraphCache();
+    g_factor64_from = from;
+  }
+  const int rc = run(from == kNoLevel ? g_factor : g_factor64, [&] {
     factor_level(top, stream, prof, overlap ? &aux : nullptr);
     row_scales();
   });
-  if (rc) return rc;
-  rc = check_status(top, st, 0);
-  factored = (rc == DM_OK);
-  return rc;
+  return rc ? rc : check_status(top, stream, 0);
 }
 
 // per-system max over columns of sqrt(num/den) from the device norm array

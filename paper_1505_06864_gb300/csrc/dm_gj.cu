@@ -534,8 +534,8 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
                                                    const double* __restrict__ W, double* __restrict__ G,
                                                    const int* __restrict__ piv, __nv_bfloat16* __restrict__ Gs,
                                                    int* __restrict__ eG, const int* __restrict__ gam,
-                                                   const int* __restrict__ rho) {
-  __shared__ int ip[kMaxM], rs[kMaxM];
+                                                   const int* __restrict__ rho, const int* __restrict__ be) {
+  __shared__ int ip[kMaxM], rs[kMaxM], ds[kMaxM];
   __shared__ double rowb[8][kMaxM];
   const int groups = (m + 31) / 32;
   const int q = blockIdx.x / groups, g = blockIdx.x - q * groups;
@@ -547,22 +547,21 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
   double* Gt = G + p.blk + (long long)t * mm;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long vt = p.blk / m + (long long)t * m;  // the block row's exponents
-  for (int c = threadIdx.x; c < m; c += blockDim.x) ip[c] = piv[(long long)q * m + c], rs[c] = rho[vt + c];
+  for (int c = threadIdx.x; c < m; c += blockDim.x) ip[c] = piv[(long long)q * m + c], rs[c] = rho[vt + c], ds[c] = be[vt + c] - rs[c];
   const int gv = 32 * g + lane < m ? gam[vt + 32 * g + lane] : 0;  // of the CTA's rows
   __syncthreads();
   double* rb = rowb[warp];
   const int rend = min(m, 32 * g + 32);
   for (int r = 32 * g + warp; r < rend; r += 8) {
-    uint32_t hmax = 0;
+    int key = kNoKey;
     const double* src = M + (long long)ip[r] * m;
     for (int c = lane; c < m; c += 32) {
       const double v = src[c];
       rb[ip[c]] = v;
-      hmax = max(hmax, abs_hi(v));
+      key = max(key, scale_key(abs_hi(v), ds[ip[c]]));
     }
-    hmax = __reduce_max_sync(0xffffffffu, hmax);
-    const int e = scale_exponent(hmax);
-    // the slices are of G_t 2^rho (dm_oz.cu) = 2^-gam X: X's digits
+    // the slices are of G_t 2^be (dm_oz.cu) = 2^-gam X 2^(be - rho)
+    const int e = key_exponent(__reduce_max_sync(0xffffffffu, key));
     const int gr = __shfl_sync(0xffffffffu, gv, r - 32 * g);
     if (lane == 0) eG[(long long)q * m + r] = e - gr;
     __syncwarp();
@@ -573,7 +572,8 @@ __global__ void __launch_bounds__(256) k_gj_finish(const PartDesc* __restrict__ 
       for (int u = 0; u < 8; ++u) v[u] = c0 + u < m ? rb[c0 + u] : 0.0;
       uint32_t d[8][S];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) digits<S>((unsigned long long)__double_as_longlong(v[u]), e, d[u]);
+      for (int u = 0; u < 8; ++u)
+        digits<S>((unsigned long long)__double_as_longlong(v[u]), e - (c0 + u < m ? ds[c0 + u] : 0), d[u]);
 #pragma unroll
       for (int sl = 0; sl < S; ++sl)
         *reinterpret_cast<uint4*>(Gs + (((long long)q * S + sl) * m + r) * mp + c0) =
@@ -619,14 +619,14 @@ void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, d
 }
 
 void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
-                      void* Gs, int* eG, const int* gam, const int* rho, cudaStream_t st) {
+                      void* Gs, int* eG, const OzScales& sc, cudaStream_t st) {
   if (nparts <= 0) return;
   const int grid = nparts * ((m + 31) / 32);
   auto* g = static_cast<__nv_bfloat16*>(Gs);
   if (oz_slices(m) == 7)
-    gj::k_gj_finish<7><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG, gam, rho);
+    gj::k_gj_finish<7><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG, sc.gam, sc.rho, sc.be);
   else
-    gj::k_gj_finish<8><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG, gam, rho);
+    gj::k_gj_finish<8><<<grid, 256, 0, st>>>(parts, t, m, W, G, piv, g, eG, sc.gam, sc.rho, sc.be);
 }
 
 }  // namespace dm

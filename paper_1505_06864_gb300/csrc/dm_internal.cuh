@@ -49,6 +49,16 @@ struct SysDesc {
   int eoff;            // offset of the system's rows in the per-row scale arrays (sum of N m before it)
 };
 
+// The system of block row `row` of all systems.
+__device__ __forceinline__ int find_sys(const SysDesc* __restrict__ sys, int nsys, int row) {
+  int lo = 0, hi = nsys - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (sys[mid].row0 <= row) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
+
 // ---- launchers (dm_kernels.cu); T = double or float (factor storage type)
 template <typename T>
 void launch_inv(const PartDesc* parts, int nparts, int t, const double* B, T* G, int* status,
@@ -153,6 +163,12 @@ bool tc2_eligible(int m);
 // Float64 products on the tensor cores by exact digit slicing (dm_oz.cu):
 // the step kernels' products with float64 operands and results, the operands
 // as bf16 digit slices with per-row (left) / per-column (right) scales.
+// Exponents of a level, [block][m] each: the blocks are inverted as 2^-rho D
+// 2^-gam, the slices balanced by be (per equation) and bu (per unknown).
+// Consecutive arrays, be first.
+struct OzScales {
+  int *be = nullptr, *gam = nullptr, *rho = nullptr, *bu = nullptr;
+};
 struct OzOut {
   const double* B;
   double *G, *Acal, *ZL, *ZR, *Y;  // Y: Y_{t+1} per subsystem (rolling, float64)
@@ -191,15 +207,14 @@ struct OzAsm {
 };
 void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, const double* C, const double* ZL,
                         const double* ZR, double* HA, double* HB, double* HC, const OzAsm& a, const int* eA,
-                        const void* mapA, int* errflag, const int* gam, const int* band, cudaStream_t st);
-void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const int* gam,
-                         const int* rho, const int* band, cudaStream_t st);
-// Exponents that equilibrate a level's unknowns (gam) and equations (rho),
-// both [block][m]: with the entries of A_i, B_i, C_i scaled by 2^-gam of their
-// unknown and 2^-rho of their equation every row's largest lies in [1/2, 1).
-// Folds the band of A and C into *band (null: not wanted; zeroed by the caller).
+                        const void* mapA, int* errflag, const int* bu, const int* band, cudaStream_t st);
+void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const OzScales& sc,
+                         const int* band, cudaStream_t st);
+// The scales of a level's equations and unknowns (dm_oz.cu): *uneven set where
+// its products need float64, the band of A and C folded into *band (null: not
+// wanted; both zeroed by the caller).
 void launch_level_scales(const SysDesc* sys, int nsys, const double* A, const double* B, const double* C, int nblocks,
-                         int m, int* gam, int* rho, int* band, cudaStream_t st);
+                         int m, const OzScales& sc, int* uneven, int* band, cudaStream_t st);
 // The level's band into *band (atomicMax; the caller zeroes it first): the
 // largest |row - column| of a nonzero entry of the n entries of A and of C.
 void launch_band_detect(const double* A, const double* C, long long n, int m, int* band, cudaStream_t st);
@@ -223,7 +238,7 @@ struct OzSliceJob {
 struct OzSliceJobs {
   OzSliceJob job[4];
   const int* band = nullptr;  // kinds 2 and 3 (launch B's operands) are skipped when banded
-  const int *gam = nullptr, *rho = nullptr;  // the level's exponents (launch_level_scales)
+  const int *bu = nullptr, *be = nullptr;  // what the slices are balanced by (OzScales)
 };
 void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, const OzSliceJobs& jobs, int njobs,
                           cudaStream_t st);
@@ -244,7 +259,7 @@ void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, d
 void launch_gj_update(const PartDesc* parts, int nparts, int t, int m, int pnl, double* W, const int* piv,
                       const int* Uexp, const int* Vexp, const void* maps2, int* errflag, cudaStream_t st);
 void launch_gj_finish(const PartDesc* parts, int nparts, int t, int m, const double* W, double* G, const int* piv,
-                      void* Gs, int* eG, const int* gam, const int* rho, cudaStream_t st);
+                      void* Gs, int* eG, const OzScales& sc, cudaStream_t st);
 int tc2_ntile(int m);
 bool tc2_make_map(int mode, const void* base, long long blocks, int m, int box_rows, void* out);
 int tc2_map_bytes();

@@ -1631,15 +1631,6 @@ __global__ void k_sep_copy(const SepDesc* __restrict__ seps, const double* __res
 // point rows of it, as the narrow products above; x_{i-1}, x_i, x_{i+1}
 // staged in shared memory RB columns at a time (RB = the system's bucket).
 // Column sums of r^2 and b^2 go to nrm by atomics.
-__device__ __forceinline__ int find_sys(const SysDesc* __restrict__ sys, int nsys, int row) {
-  int lo = 0, hi = nsys - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (sys[mid].row0 <= row) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 template <int RM>
 __global__ void __launch_bounds__(256) k_residual(const SysDesc* __restrict__ sys, int nsys,
                                                   const double* __restrict__ A,

@@ -20,8 +20,8 @@
 // of the column is small, and one scale per row and column would lose the
 // small ones (m = 100, rows scaled over eight decades: solutions to 1e-11
 // against 1.5e-13).  So the operands are balanced along k by exact powers of
-// two, one per equation (rho) or unknown (gam) of a block row, found before
-// the sweeps (k_level_cols, k_level_rows): L[r][k] 2^(s_k) times 2^(-s_k) R[k][n],
+// two, one per equation (be) or unknown (bu) of a block row, found before
+// the sweeps (k_level_scan): L[r][k] 2^(s_k) times 2^(-s_k) R[k][n],
 // inside the extraction of the digits.  The products' results, and all that is
 // stored in float64, are not scaled.
 //
@@ -51,6 +51,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include "dm_internal.cuh"
 #include "dm_slices.cuh"
@@ -533,15 +534,6 @@ struct Shift {
   __device__ __forceinline__ int operator()(int k) const { return sign * __ldg(kap + k); }
 };
 
-// Key of the high word of an entry with shift s: keys are compared, and an
-// entry of key K is below 2^(K - 1022).
-constexpr int kNoKey = -(1 << 20);
-__device__ __forceinline__ int scale_key(uint32_t hi, int s) {
-  const int h = (int)(hi & 0x7fffffffu);
-  return h == 0 ? kNoKey : max(h >> 20, 1) + s;
-}
-__device__ __forceinline__ int key_exponent(int key) { return key == kNoKey ? 0 : key - 1022; }
-
 // Row slices (left operands): exps[r] = e with |v 2^shift| < 2^e for the row's
 // entries v; slice s element (r, k) at ((q * S + s) m + r) pitch + k, the
 // pitch m rounded up to 8 (16-byte rows for TMA; the columns past m are zero).
@@ -641,7 +633,7 @@ __device__ __forceinline__ void slice_cols_group(const double* __restrict__ src,
 template <bool COLS, int S>
 __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__ src, int nblocks, int m,
                                                       __nv_bfloat16* __restrict__ dst, int* __restrict__ exps,
-                                                      const int* __restrict__ gam, const int* __restrict__ rho,
+                                                      const int* __restrict__ bu, const int* __restrict__ be,
                                                       const int* __restrict__ band) {
   __shared__ int red[8][32], s_e[32];
   __shared__ unsigned long long tile[32][33];
@@ -651,9 +643,9 @@ __global__ void __launch_bounds__(256) k_oz_slice_all(const double* __restrict__
   for (long long i = blockIdx.x; i < (long long)nblocks * groups; i += gridDim.x) {
     const int q = (int)(i / groups), g = (int)(i - (long long)q * groups);
     if (COLS)
-      slice_cols_group<S>(src + q * mm, dst, q, exps, m, g, Shift{rho + (long long)q * m, -1}, red, s_e, tile);
+      slice_cols_group<S>(src + q * mm, dst, q, exps, m, g, Shift{be + (long long)q * m, -1}, red, s_e, tile);
     else  // the first block row has no unknowns before it
-      slice_rows_group<S>(src + q * mm, dst, q, exps, m, g, Shift{gam + (long long)max(q - 1, 0) * m, q > 0 ? -1 : 0});
+      slice_rows_group<S>(src + q * mm, dst, q, exps, m, g, Shift{bu + (long long)max(q - 1, 0) * m, q > 0 ? -1 : 0});
     __syncthreads();
   }
 }
@@ -699,11 +691,11 @@ __global__ void __launch_bounds__(256) k_oz_slice_jobs(const PartDesc* __restric
   if (!act) return;
   __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(jb.dst);
   const long long bt = p.blk / mm + t;  // the block row
-  const Shift sh = jb.kind == 0   ? Shift{jobs.rho + bt * m, 1}
-                   : jb.kind == 1 ? Shift{jobs.gam + (bt + 1) * m, -1}
-                   : jb.kind == 5 ? Shift{jobs.rho + (bt + 1) * m, -1}
-                   : jb.kind == 8 ? Shift{jobs.rho + sblk * m, -1}
-                                  : Shift{jobs.gam + bt * m, 1};
+  const Shift sh = jb.kind == 0   ? Shift{jobs.be + bt * m, 1}
+                   : jb.kind == 1 ? Shift{jobs.bu + (bt + 1) * m, -1}
+                   : jb.kind == 5 ? Shift{jobs.be + (bt + 1) * m, -1}
+                   : jb.kind == 8 ? Shift{jobs.be + sblk * m, -1}
+                                  : Shift{jobs.bu + bt * m, 1};
   if (jb.kind == 0 || jb.kind == 1)
     slice_rows_group<S>(jb.src + sblk * mm, dst, dq, jb.exps, m, g, sh);
   else
@@ -719,7 +711,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_seps(const SepDesc* __restrict
                                                        const double* __restrict__ C, const double* __restrict__ ZL,
                                                        const double* __restrict__ ZR, __nv_bfloat16* __restrict__ Cq,
                                                        int* __restrict__ eCq, __nv_bfloat16* __restrict__ Sp,
-                                                       int* __restrict__ eS, const int* __restrict__ gam,
+                                                       int* __restrict__ eS, const int* __restrict__ bu,
                                                        const int* __restrict__ band) {
   __shared__ int red[8][32], s_e[32];
   __shared__ unsigned long long tile[32][33];
@@ -729,14 +721,14 @@ __global__ void __launch_bounds__(256) k_oz_slice_seps(const SepDesc* __restrict
   const SepDesc sd = seps[s];
   const long long mm = (long long)m * m;
   if (job == 0) {
-    slice_rows_group<S>(C + sd.blk_q, Cq, s, eCq, m, g, Shift{gam + sd.blk_next / mm * m, -1});
+    slice_rows_group<S>(C + sd.blk_q, Cq, s, eCq, m, g, Shift{bu + sd.blk_next / mm * m, -1});
     return;
   }
   if ((job == 2 && !(sd.flags & HAS_HA)) || (job == 4 && !(sd.flags & HAS_HC))) return;
   const double* src = job == 1 ? ZR + sd.blk_prev : job == 2 ? ZL + sd.blk_prev : job == 3 ? ZL + sd.blk_next
                                                                                          : ZR + sd.blk_next;
   slice_cols_group<S>(src, Sp, 4LL * s + job - 1, eS, m, g,
-                      Shift{gam + (job <= 2 ? sd.blk_prev : sd.blk_next) / mm * m, 1}, red, s_e, tile);
+                      Shift{bu + (job <= 2 ? sd.blk_prev : sd.blk_next) / mm * m, 1}, red, s_e, tile);
 }
 
 // ---------------------------------------------------------------- banded operands
@@ -867,96 +859,127 @@ __global__ void __launch_bounds__(256) k_band_h(const SepDesc* __restrict__ seps
 }
 
 // ---------------------------------------------------------------- scales of equations and unknowns
-// Exponents that equilibrate a level: gam per unknown, of the largest entry in
-// its column of [C_{i-1}; B_i; A_{i+1}], then rho per equation, of the largest
-// entry of its row of [A_i B_i C_i] with the columns so scaled.  Columns first,
-// since partial pivoting (down the columns) does not see their scales: with
-// them the digit-sliced elimination gave float64's errors or smaller ones for
-// dense, banded and Laplace blocks with rows, columns or both scaled over 0 to 12
-// decades (m = 33 to 129, a numpy restatement); rows first cost two digits where
-// the unknowns are scaled, one pass for both (or a 2^6 limit on the spread, as a
-// switch to float64 products) more.  Two passes over the blocks, each bound by
-// reading them.
+// Exponents that equilibrate a level, estimated in two ways from the largest
+// entries: per unknown of its column of [C_{i-1}; B_i; A_{i+1}] (gam), then per
+// equation of its row of [A_i B_i C_i] with the columns so scaled (rho); and
+// rows first, then columns.  The blocks are inverted with the first (partial
+// pivoting, down the columns, does not see the columns' scales).  The products
+// are balanced by the mean of both: where equations alone or unknowns alone
+// are scaled one estimate is right, and for sparse blocks the other may be off
+// by the whole range at the border of two fields of different scale.  Where
+// they differ by more than 2^kAmbiguous inside a block row, or by more than
+// 2^kDoubt where the largest entries spread over more than 2^kWide, the scales
+// are not to be had from the largest entries, and the level keeps float64
+// products (*uneven).  Relative errors, float64 / digits with columns first /
+// with the mean (block Thomas in numpy, m = 64): dense, rows scaled over 12
+// decades 1.1e-13 / 1.5e-14 / 5e-16; banded with a jump between the halves of
+// the blocks of 2^40 5e-16 / 4e-6 / 1e-11 (estimates 2^42 apart), of 2^10 5e-16 /
+// 3e-15 / 7e-16; Laplace blocks with equations and unknowns jumping oppositely
+// by 2^20 9e-16 / 3e-14 / 3e-14 (2^7 apart, spread 2^18).  Blocks of one scale are
+// 2^2 apart at most, dense blocks of condition 1e4 with graded singular vectors
+// 2^8, spread over 2^11; digits serve those with smaller errors than float64
+// products (6.5e-14 against 2.8e-13 at m = 128).  What stays on digits with an
+// opposite jump of less than 2^13 has up to 40 times float64's error, at most
+// 7e-14.  Two passes over the blocks, each bound by reading them.
+constexpr int kAmbiguous = 11, kDoubt = 4, kWide = 13;
+constexpr int kKeyBias = 4096;
 
-// Block row b = blockIdx.x, columns 32 blockIdx.y ..: a lane per column, eight
-// warps over the rows.  Also folds the largest |row - column| of a nonzero entry
-// (any bit but the sign set) of A and C into *band (if not null).
-__device__ __forceinline__ int sys_of_row(const SysDesc* __restrict__ sys, int nsys, int row) {
-  int lo = 0, hi = nsys - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (sys[mid].row0 <= row) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__global__ void __launch_bounds__(256) k_level_cols(const SysDesc* __restrict__ sys, int nsys,
+// One pass over the blocks: blockIdx.x = block row, y = 0 A, 1 B, 2 C, z =
+// `rpc` rows of it; a warp a row at a time, a lane every 32nd column (at most
+// CPL).  First pass: the largest exponent of every row to rowkey and of every
+// column to colkey ([block row][m], zeroed before; a column of A_i belongs to
+// the unknowns of block row i - 1, one of C_i to those of i + 1), and the
+// largest |row - column| of a nonzero entry (any bit but the sign set) of A
+// and C to *band (if not null).  Second pass: the same with every entry
+// divided by its column's (for the rows) or its row's (for the columns) first
+// result, in rowkey2 and colkey2.
+template <int CPL, bool SECOND>
+__global__ void __launch_bounds__(256) k_level_scan(const SysDesc* __restrict__ sys, int nsys,
                                                     const double* __restrict__ A, const double* __restrict__ B,
-                                                    const double* __restrict__ C, int m, int* __restrict__ gam,
-                                                    int* __restrict__ band) {
-  __shared__ int red[8][32], swid[8];
-  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n = 32 * blockIdx.y + lane;
-  const SysDesc& sd = sys[sys_of_row(sys, nsys, b)];
-  const bool up = b > sd.row0, down = b < sd.row0 + sd.N - 1;
-  const long long mm = (long long)m * m;
-  int key = kNoKey, wid = 0;
-  auto column = [&](const double* M, bool banded) {
-    const unsigned long long* v = reinterpret_cast<const unsigned long long*>(M) + n;
-#pragma unroll 8
-    for (int k = warp; k < m; k += 8) {
-      const unsigned long long x = __ldg(v + (long long)k * m);
-      key = max(key, scale_key((uint32_t)(x >> 32), 0));
-      if (banded && (x << 1) != 0) wid = max(wid, abs(k - n));
-    }
-  };
-  if (n < m) {
-    column(B + b * mm, false);
-    if (up) column(C + (b - 1) * mm, true);
-    if (down) column(A + (b + 1) * mm, true);
+                                                    const double* __restrict__ C, int m, int rpc, int* __restrict__ rowkey,
+                                                    int* __restrict__ colkey, int* __restrict__ rowkey2,
+                                                    int* __restrict__ colkey2, int* __restrict__ band) {
+  __shared__ int cmax[8][32 * CPL], swid[8];
+  const int b = blockIdx.x, part = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const SysDesc& sd = sys[find_sys(sys, nsys, b)];
+  const int cb = b + part - 1;
+  if (cb < sd.row0 || cb >= sd.row0 + sd.N) return;  // A_1, C_N
+  const unsigned long long* M =
+      reinterpret_cast<const unsigned long long*>(part == 0 ? A : part == 1 ? B : C) + (long long)b * m * m;
+  int* rk = rowkey + (long long)b * m;
+  int* ck = colkey + (long long)cb * m;
+  int cm[CPL], cs[CPL], wid = 0;
+#pragma unroll
+  for (int q = 0; q < CPL; ++q) {
+    cm[q] = 0;
+    cs[q] = SECOND && lane + 32 * q < m ? kKeyBias - ck[lane + 32 * q] : 0;
   }
-  red[warp][lane] = key;
+  const int rend = min(m, (int)(blockIdx.z + 1) * rpc);
+#pragma unroll 2
+  for (int r = blockIdx.z * rpc + warp; r < rend; r += 8) {
+    unsigned long long v[CPL];
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) v[q] = lane + 32 * q < m ? __ldg(M + (long long)r * m + lane + 32 * q) : 0ull;
+    const int rs = SECOND ? kKeyBias - rk[r] : 0;
+    int rm = 0;
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) {
+      const int h = (int)(v[q] >> 32) & 0x7fffffff, ex = max(h >> 20, 1);
+      if (h != 0) {
+        rm = max(rm, ex + cs[q]);
+        cm[q] = max(cm[q], ex + rs);
+      }
+      if (!SECOND && (v[q] << 1) != 0) wid = max(wid, abs(r - lane - 32 * q));
+    }
+    rm = __reduce_max_sync(0xffffffffu, rm);
+    if (lane == 0 && rm > 0) atomicMax((SECOND ? rowkey2 + (long long)b * m : rk) + r, rm);
+  }
+#pragma unroll
+  for (int q = 0; q < CPL; ++q) cmax[warp][lane + 32 * q] = cm[q];
   wid = __reduce_max_sync(0xffffffffu, wid);
   if (lane == 0) swid[warp] = wid;
   __syncthreads();
-  if (warp == 0) {
+  for (int c = threadIdx.x; c < m; c += 256) {
+    int h = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) key = max(key, red[w][lane]), wid = max(wid, swid[w]);
-    if (n < m) gam[(long long)b * m + n] = key_exponent(key);
-    if (band && lane == 0 && wid > *(volatile int*)band) atomicMax(band, wid);
+    for (int w = 0; w < 8; ++w) h = max(h, cmax[w][c]);
+    if (h > 0) atomicMax((SECOND ? colkey2 + (long long)cb * m : ck) + c, h);
+  }
+  if (!SECOND && band && part != 1 && threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) wid = max(wid, swid[w]);
+    if (wid > *(volatile int*)band) atomicMax(band, wid);
   }
 }
 
-// Block row b = blockIdx.x, rows 32 blockIdx.y ..: a warp a row at a time.
-__global__ void __launch_bounds__(256) k_level_rows(const SysDesc* __restrict__ sys, int nsys,
-                                                    const double* __restrict__ A, const double* __restrict__ B,
-                                                    const double* __restrict__ C, int m, const int* __restrict__ gam,
-                                                    int* __restrict__ rho) {
-  __shared__ int g[3][kMaxM];
-  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const SysDesc& sd = sys[sys_of_row(sys, nsys, b)];
-  const bool up = b > sd.row0, down = b < sd.row0 + sd.N - 1;
-  const long long mm = (long long)m * m;
-  for (int k = threadIdx.x; k < m; k += 256) {
-    const int* gb = gam + (long long)b * m + k;
-    g[0][k] = up ? gb[-m] : 0;
-    g[1][k] = gb[0];
-    g[2][k] = down ? gb[m] : 0;
+// The exponents from the keys, in place, a warp per block row: rowkey2 -> rho,
+// colkey -> gam, rowkey -> be (equations), colkey2 -> bu (unknowns).
+__global__ void __launch_bounds__(256) k_level_exponents(int nblocks, int m, int* __restrict__ rowkey,
+                                                         int* __restrict__ colkey, int* __restrict__ rowkey2,
+                                                         int* __restrict__ colkey2, int* __restrict__ uneven) {
+  const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (b >= nblocks) return;
+  // the differences of the estimates and the estimates from all entries, of
+  // the equations and the unknowns
+  int lo[4] = {1 << 20, 1 << 20, 1 << 20, 1 << 20}, hi[4] = {-(1 << 20), -(1 << 20), -(1 << 20), -(1 << 20)};
+  auto take = [&](int i, int v) { lo[i] = min(lo[i], v), hi[i] = max(hi[i], v); };
+  for (int k = lane; k < m; k += 32) {
+    const long long i = (long long)b * m + k;
+    const bool row = rowkey[i] != 0, col = colkey[i] != 0;  // not all zeros
+    const int rho2 = row ? rowkey[i] - 1022 : 0, gam = col ? colkey[i] - 1022 : 0;
+    const int rho = row ? rowkey2[i] - kKeyBias : 0, gam2 = col ? colkey2[i] - kKeyBias : 0;
+    if (row) take(0, rho - rho2), take(2, rho2);
+    if (col) take(1, gam - gam2), take(3, gam);
+    rowkey2[i] = rho;
+    colkey[i] = gam;
+    rowkey[i] = (rho + rho2) >> 1;
+    colkey2[i] = (gam + gam2) >> 1;
   }
-  __syncthreads();
-  const int r0 = 32 * blockIdx.y, rend = min(m, r0 + 32);
-  for (int r = r0 + warp; r < rend; r += 8) {
-    int key = kNoKey;
-    auto row = [&](const double* M, const int* gk) {
-      const unsigned long long* v = reinterpret_cast<const unsigned long long*>(M) + (long long)r * m;
-#pragma unroll 8
-      for (int c = lane; c < m; c += 32) key = max(key, scale_key((uint32_t)(__ldg(v + c) >> 32), -gk[c]));
-    };
-    row(B + b * mm, g[1]);
-    if (up) row(A + b * mm, g[0]);
-    if (down) row(C + b * mm, g[2]);
-    key = __reduce_max_sync(0xffffffffu, key);
-    if (lane == 0) rho[(long long)b * m + r] = key_exponent(key);
-  }
+  int sp[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) sp[i] = __reduce_max_sync(0xffffffffu, hi[i]) - __reduce_min_sync(0xffffffffu, lo[i]);
+  const int apart = max(sp[0], sp[1]), wide = max(sp[2], sp[3]);
+  if (lane == 0 && (apart > kAmbiguous || (apart > kDoubt && wide > kWide))) *uneven = 1;
 }
 
 // The level's band: the largest |row - column| of a nonzero entry (any bit
@@ -1038,24 +1061,36 @@ void launch_band_detect(const double* A, const double* C, long long n, int m, in
 }
 
 void launch_level_scales(const SysDesc* sys, int nsys, const double* A, const double* B, const double* C, int nblocks,
-                         int m, int* gam, int* rho, int* band, cudaStream_t st) {
+                         int m, const OzScales& sc, int* uneven, int* band, cudaStream_t st) {
   if (nblocks <= 0) return;
-  const dim3 grid(nblocks, (m + 31) / 32);
-  oz::k_level_cols<<<grid, 256, 0, st>>>(sys, nsys, A, B, C, m, gam, band);
-  oz::k_level_rows<<<grid, 256, 0, st>>>(sys, nsys, A, B, C, m, gam, rho);
+  cudaMemsetAsync(sc.be, 0, 4 * (size_t)nblocks * m * sizeof(int), st);
+  const int rpc = 3 * nblocks >= 304 ? m : 32;  // a few blocks: more CTAs each
+  const dim3 grid(nblocks, 3, (m + rpc - 1) / rpc);
+  auto pass = [&](auto second) {
+    constexpr bool S2 = decltype(second)::value;
+#define DM_SCAN(CPL_) oz::k_level_scan<CPL_, S2><<<grid, 256, 0, st>>>(sys, nsys, A, B, C, m, rpc, sc.be, sc.gam, sc.rho, sc.bu, band)
+    if (m <= 64) DM_SCAN(2);
+    else if (m <= 128) DM_SCAN(4);
+    else if (m <= 256) DM_SCAN(8);
+    else DM_SCAN(16);
+#undef DM_SCAN
+  };
+  pass(std::false_type());
+  pass(std::true_type());
+  oz::k_level_exponents<<<(nblocks + 7) / 8, 256, 0, st>>>(nblocks, m, sc.be, sc.gam, sc.rho, sc.bu, uneven);
 }
 
-void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const int* gam,
-                         const int* rho, const int* band, cudaStream_t st) {
+void launch_oz_slice_all(bool cols, const double* src, int nblocks, int m, void* dst, int* exps, const OzScales& sc,
+                         const int* band, cudaStream_t st) {
   if (nblocks <= 0) return;
   const long long work = (long long)nblocks * ((m + 31) / 32);
   const int grid = (int)std::min<long long>(work, 152LL * 16);
   auto* d = static_cast<__nv_bfloat16*>(dst);
   const bool s7 = oz_slices(m) == 7;
-  if (cols && s7) oz::k_oz_slice_all<true, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
-  else if (cols) oz::k_oz_slice_all<true, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
-  else if (s7) oz::k_oz_slice_all<false, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
-  else oz::k_oz_slice_all<false, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, gam, rho, band);
+  if (cols && s7) oz::k_oz_slice_all<true, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, sc.bu, sc.be, band);
+  else if (cols) oz::k_oz_slice_all<true, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, sc.bu, sc.be, band);
+  else if (s7) oz::k_oz_slice_all<false, 7><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, sc.bu, sc.be, band);
+  else oz::k_oz_slice_all<false, 8><<<grid, 256, 0, st>>>(src, nblocks, m, d, exps, sc.bu, sc.be, band);
 }
 
 void launch_oz_slice_jobs(const PartDesc* parts, int nparts, int step, int m, const OzSliceJobs& jobs, int njobs,
@@ -1126,14 +1161,14 @@ void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m
 
 void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, const double* C, const double* ZL,
                         const double* ZR, double* HA, double* HB, double* HC, const OzAsm& a, const int* eA,
-                        const void* mapA, int* errflag, const int* gam, const int* band, cudaStream_t st) {
+                        const void* mapA, int* errflag, const int* bu, const int* band, cudaStream_t st) {
   if (nseps <= 0) return;
   const dim3 sgrid(nseps * ((m + 31) / 32), 5);
   auto *cq = static_cast<__nv_bfloat16*>(a.Cq), *sp = static_cast<__nv_bfloat16*>(a.S);
   if (oz_slices(m) == 7)
-    oz::k_oz_slice_seps<7><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, gam, band);
+    oz::k_oz_slice_seps<7><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, bu, band);
   else
-    oz::k_oz_slice_seps<8><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, gam, band);
+    oz::k_oz_slice_seps<8><<<sgrid, 256, 0, st>>>(seps, m, C, ZL, ZR, cq, a.eCq, sp, a.eS, bu, band);
   OzOut out{};
   out.B = B;
   out.seps = seps;

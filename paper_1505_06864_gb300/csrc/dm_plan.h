@@ -98,10 +98,14 @@ struct OzLevel {
   void *AcalT = nullptr, *YT = nullptr, *ZLT = nullptr, *ZRT = nullptr;
   int *eA = nullptr, *eCT = nullptr, *eAcal = nullptr, *eG = nullptr;
   int *eAcalT = nullptr, *eYT = nullptr, *eZLT = nullptr, *eZRT = nullptr;
-  // exponents of the unknowns and of the equations ([block][m]), found at the
-  // start of each factorisation: what the slices are balanced by and the
-  // blocks inverted with
-  int *gam = nullptr, *rho = nullptr;
+  // found at the start of each factorisation: the exponents of the equations
+  // and unknowns; whether they are too ambiguous for digit products (host copy
+  // valid once the factorisation is), and whether this factorisation
+  // therefore runs the level's float64 products
+  OzScales sc;
+  int* uneven = nullptr;
+  int* uneven_host = nullptr;
+  bool fp64_now = false;
   double* Y = nullptr;
   // tensor maps: left G, A, Acal; right CT, YT, AcalT, ZLT, ZRT
   alignas(64) unsigned char maps[8][128];
@@ -116,8 +120,8 @@ struct OzLevel {
   // the supplementary blocks on the tensor cores (levels with a supplementary level)
   bool asm_on = false;
   OzAsm as;
-  // banded A and C: the largest |row - column| of a nonzero entry, found by
-  // the input slicing on the device (null: detection off, DM_BANDED=0), and
+  // banded A and C: the largest |row - column| of a nonzero entry, found with
+  // the scales on the device (null: detection off, DM_BANDED=0), and
   // its copy in page-locked host memory after each factorisation (for the
   // profiling costs of the next one; the device decides the path)
   int* band = nullptr;
@@ -191,6 +195,8 @@ struct GraphCache {
   bool broken = false;     // capture failed: stay eager
 };
 
+constexpr int kNoLevel = 1 << 20;
+
 struct Plan {
   int precision = 0;
   int device = 0;  // the CUDA device current at dm_plan: every launch of the plan goes there
@@ -210,7 +216,12 @@ struct Plan {
   Prof prof;
   Aux aux;
   bool use_graphs = true;
-  GraphCache g_factor, g_solve, g_iter_first, g_iter_next;
+  GraphCache g_factor, g_factor64, g_solve, g_iter_first, g_iter_next;
+  // the first level (depth) whose digit products give way to float64 ones
+  // (kNoLevel: none): as the last factorisation found it, where the next one
+  // starts from, and the one g_factor64 was captured with
+  int fp64_from = kNoLevel, g_factor64_from = kNoLevel;
+  int run_factor(int from);
   bool borrow = false;  // use the caller's device A, B, C in place (no copy)
   bool overlap = false;  // left-spike tiles on the side stream
   const double *bA = nullptr, *bB = nullptr, *bC = nullptr;

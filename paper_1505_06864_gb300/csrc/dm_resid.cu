@@ -40,21 +40,12 @@ static_assert(kMaxMRow <= 16 * kWarps, "a block row's 16-row tiles in one CTA");
 
 __device__ __forceinline__ uint32_t abs_hi(unsigned long long bits) { return (uint32_t)(bits >> 32) & 0x7fffffffu; }
 
-__device__ __forceinline__ int find_row(const SysDesc* __restrict__ sys, int nsys, int row) {
-  int lo = 0, hi = nsys - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (sys[mid].row0 <= row) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // Largest high word (sign cleared) of every point row of [A_i B_i C_i] of the
 // sliced systems: a warp per point row, one CTA per block row.
 __global__ void __launch_bounds__(kThreads) k_row_scales(const SysDesc* __restrict__ sys, int nsys,
                                                          const double* __restrict__ A, const double* __restrict__ B,
                                                          const double* __restrict__ C, unsigned* __restrict__ rowhi) {
-  const int si = find_row(sys, nsys, blockIdx.x);
+  const int si = find_sys(sys, nsys, blockIdx.x);
   const SysDesc sd = sys[si];
   if (!sd.sliced) return;
   const int i = blockIdx.x - sd.row0, m = sd.m;
@@ -85,7 +76,7 @@ __global__ void __launch_bounds__(kThreads) k_col_scales(const SysDesc* __restri
   const int row = blockIdx.x * kWarps + (threadIdx.x >> 5);
   if (row >= nrows) return;
   const int lane = threadIdx.x & 31;
-  const SysDesc sd = sys[find_row(sys, nsys, row)];
+  const SysDesc sd = sys[find_sys(sys, nsys, row)];
   if (!sd.sliced) return;
   const int i = row - sd.row0, m = sd.m, r = sd.r;
   const int c = lane & 15, par = lane >> 4;

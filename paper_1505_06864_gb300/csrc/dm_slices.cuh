@@ -93,4 +93,13 @@ __device__ __forceinline__ int scale_exponent(uint32_t hmax) {
   return E == 0 ? -1021 : E - 1022;
 }
 
+// Key of the high word of an entry with shift s: keys are compared, and an
+// entry of key K is below 2^(K - 1022).
+constexpr int kNoKey = -(1 << 20);
+__device__ __forceinline__ int scale_key(uint32_t hi, int s) {
+  const int h = (int)(hi & 0x7fffffffu);
+  return h == 0 ? kNoKey : max(h >> 20, 1) + s;
+}
+__device__ __forceinline__ int key_exponent(int key) { return key == kNoKey ? 0 : key - 1022; }
+
 }  // namespace dm
