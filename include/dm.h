@@ -383,8 +383,11 @@ int dm_set_refinement(dm_plan_t plan, double tol, int max_iters); /* default 1e-
  * the row's (column's) largest power of two, multiplies digit matrices exactly
  * on the bf16 tensor cores (integer sums of at most 2^24 in float32), and sums
  * the digit products in 64-bit integers: error per entry below
- * 3m 2^-50 max|row of [A B C]| max|column of x|, the float64 dot product's own
- * bound.  It serves systems with m <= 128 and nrhs <= 16; the others of the
+ * 3m 2^-50 max|row of [A B C]| max|column of x|.  An entry whose terms are all
+ * far below those maxima (unknowns of different scale, a solution that decays
+ * within three block rows) is found by a product of the magnitudes and computed
+ * again in float64, so that the error is also below 3m 2^-49 sum |row| |column|,
+ * a float64 dot product's bound but for a factor of 16.  It serves systems with m <= 128 and nrhs <= 16; the others of the
  * plan use DM_RESIDUAL_FP64.  DM_RESIDUAL_AUTO picks SLICED per system where
  * it measured faster on GB300 (m nrhs >= 128; systems of fewer than 32 block
  * rows: m^2 nrhs >= 2^17): the float64 kernel's cost grows with nrhs, the

@@ -1398,8 +1398,8 @@ int Plan::set_residual_mode(int mode) {
     // r = 4 62 / 30, 32,1 47 / 51, 32,8 217 / 57, 64,1 131 / 122, 64,2 160 /
     // 130, 96,1 268 / 288, 96,8 1007 / 304, 128,1 458 / 367, 128,8 1698 / 385,
     // 128,16 3340 / 754: the line is near m r = 128.  Systems of fewer than 32
-    // block rows (at most 0.3 ms either way) keep the line m^2 r >= 2^17 that
-    // the interface states for them.
+    // block rows take at most 0.3 ms either way and keep the higher line m^2 r >=
+    // 2^17.
     const bool faster = (long long)d.m * d.m * d.r >= (1ll << 17) || (d.N >= 32 && d.m * d.r >= 128);
     d.cta0[0] = top.res_ctas[0];
     d.cta0[1] = top.res_ctas[1];

@@ -8,8 +8,17 @@
 // Each acc_d sums at most seven products over K <= 128 (one of the three
 // blocks) of magnitude <= 2^14: integers below 2^24, exact in float32; after
 // each block they are added up in 64-bit integers.  Operand rounding and the
-// dropped pairs bound the error of an entry by 3m 2^-50 max|row| max|column|,
-// the float64 dot product's own bound.
+// dropped pairs bound the error of an entry by 3m 2^-55 times its scales 2^(e+f).
+//
+// A float64 dot product's bound is 3m 2^-53 sum |row| |column|, far below that
+// where the row weights small entries of x only (unknowns of different scale, a
+// solution that decays within three block rows).  So every entry is certified: one
+// more product, of |L| and |x| rounded to bf16 (down, so from below), gives the
+// sum, and an entry with less than 2^-6 of its scales is computed again by
+// float64 multiply-adds, a warp per entry.  Dense and banded blocks with
+// solutions of one scale have 2^-4.5 of them and more (none is recomputed: the
+// magnitudes cost 60 us of a residual of N = 4096, m = 128, r = 8).  The error of
+// an entry is then at most 3m 2^-49 sum |row| |column|.
 //
 // Bound by the digit extraction (about 40 instructions per entry of L, once
 // per residual) beside reading L: so the digits stay in registers.  A warp
@@ -35,6 +44,8 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int S = kBalSlices;
 constexpr int NACC = S + 1;  // d = 2 .. 9
+constexpr int SX = S + 1;    // an entry of x in shared memory: its digits and its magnitude
+constexpr float kCertified = 0x1p-6f;
 constexpr int kMaxMRow = 128, kMaxCols = 16;
 static_assert(kMaxMRow <= 16 * kWarps, "a block row's 16-row tiles in one CTA");
 
@@ -119,18 +130,28 @@ __device__ __forceinline__ void load_tile(const double* __restrict__ L, int m, i
   }
 }
 
-// acc += the 16 rows of L (one block, m columns) times the digits xd of x.
+// |v| 2^-e, |v| < 2^e, as bf16 rounded down (in the high half of the word); for
+// e below -896 less than that.
+__device__ __forceinline__ uint32_t magnitude(unsigned long long bits, int e) {
+  const int h = (int)(bits >> 32) & 0x7fffffff;
+  return (uint32_t)max((h >> 13) - ((max(e, -896) + 896) << 7), 0) << 16;
+}
+
+// acc += the 16 rows of L (one block, m columns) times the digits xd of x, sum
+// += the product of the magnitudes.
 template <int NT, bool V2>
 __device__ __forceinline__ void tile_products(const double* __restrict__ L, int m, int r0, int tg, const int (&er)[2],
-                                              const uint2* xd, int lane, float (&acc)[NACC][NT][4]) {
+                                              const uint2* xd, int lane, float (&acc)[NACC][NT][4],
+                                              float (&sum)[NT][4]) {
   const int nks = (m + 15) / 16;
   unsigned long long v[8];
   load_tile<V2>(L, m, r0, 2 * tg, v);
 #pragma unroll 1
   for (int ks = 0; ks < nks; ++ks) {
-    uint32_t a[S][4];
+    uint32_t a[S][4], am[4];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
+      am[h] = pack_hi(magnitude(v[2 * h], er[h & 1]), magnitude(v[2 * h + 1], er[h & 1]));
       uint32_t d0[S], d1[S];
       digits<S>(v[2 * h], er[h & 1], d0);
       digits<S>(v[2 * h + 1], er[h & 1], d1);
@@ -141,8 +162,9 @@ __device__ __forceinline__ void tile_products(const double* __restrict__ L, int 
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       uint2 b[S];
+      mma_k16(sum[nt], am, xd[((ks * SX + S) * NT + nt) * 32 + lane]);
 #pragma unroll
-      for (int t = 0; t < S; ++t) b[t] = xd[((ks * S + t) * NT + nt) * 32 + lane];
+      for (int t = 0; t < S; ++t) b[t] = xd[((ks * SX + t) * NT + nt) * 32 + lane];
 #pragma unroll
       for (int s = 1; s <= S; ++s)
 #pragma unroll
@@ -150,6 +172,29 @@ __device__ __forceinline__ void tile_products(const double* __restrict__ L, int 
           if (s + t <= S + 2) mma_k16(acc[s + t - 2][nt], a[s - 1], b[t - 1]);
     }
   }
+}
+
+// sum_k L[k] x[k r] over the m entries of one point row of a block (lanes
+// together; this lane's part).
+__device__ __forceinline__ double row_part(const double* __restrict__ L, const double* __restrict__ x, int m, int r,
+                                           int lane) {
+  double acc = 0.0;
+#pragma unroll 4
+  for (int k = lane; k < m; k += 32) acc = fma(__ldg(L + k), __ldg(x + (long long)k * r), acc);
+  return acc;
+}
+
+// One entry of L X in float64 by a warp: o the row in A, B, C, xi its column in
+// x_i (mr entries from one x_i to the next).
+__device__ __noinline__ double float64_entry(const double* __restrict__ A, const double* __restrict__ B,
+                                             const double* __restrict__ C, long long o, const double* __restrict__ xi,
+                                             long long mr, int m, int r, bool hasA, bool hasC, int lane) {
+  double acc = row_part(B + o, xi, m, r, lane);
+  if (hasA) acc += row_part(A + o, xi - mr, m, r, lane);
+  if (hasC) acc += row_part(C + o, xi + mr, m, r, lane);
+#pragma unroll
+  for (int w = 16; w; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
+  return acc;
 }
 
 // One CTA per group of block rows of a sliced system with 8 (NT - 1) < r <= 8
@@ -160,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
                       const double* __restrict__ B, const double* __restrict__ C, const double* __restrict__ x,
                       const double* __restrict__ b, double* __restrict__ rout, double* __restrict__ nrm,
                       const unsigned* __restrict__ rowhi, const unsigned* __restrict__ colhi) {
-  extern __shared__ __align__(16) uint2 xd[];  // [block row of the group][k16 step][digit][NT][lane]
+  extern __shared__ __align__(16) uint2 xd[];  // [block row of the group][k16 step][digit, magnitude][NT][lane]
   __shared__ double red[2 * kMaxCols];
   __shared__ int fcol[kWarps][kMaxCols];
   int lo = 0, hi = nsys - 1;
@@ -175,7 +220,7 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
   const int sub = warp / mt, i = i0 + sub, r0 = 16 * (warp - sub * mt) + g;
   const bool active = sub < rows;
   const long long mm = (long long)m * m, mr = (long long)m * r;
-  const int xw = mt * S * NT * 32;  // words of one block row's digits
+  const int xw = mt * SX * NT * 32;  // words of one block row's digits
   if (tid < 2 * kMaxCols) red[tid] = 0.0;
   if (tid < kMaxCols * rows) {
     const int q = tid / kMaxCols, c = tid - q * kMaxCols, ii = i0 + q;
@@ -195,11 +240,12 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
   const bool v2 = (m & 1) == 0 && (((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B) |
                                      reinterpret_cast<uintptr_t>(C)) & 15) | (sd.blk & 1)) == 0;
   long long T[NT][4];  // (L X) 2^(54 - e - f)
+  float sum[NT][4];  // sum |L| |X| 2^(-e - f), from below
   uint32_t nan = 0;
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) T[nt][q] = 0;
+    for (int q = 0; q < 4; ++q) T[nt][q] = 0, sum[nt][q] = 0.f;
 #pragma unroll 1
   for (int part = 0; part < 3; ++part) {  // A_i x_{i-1}, B_i x_i, C_i x_{i+1}
     __syncthreads();
@@ -209,16 +255,18 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
       const int ii = i0 + q - 1 + part, c = 8 * nt + (ln >> 2), k = 16 * ks + 2 * (ln & 3);
       const double* xp = x + sd.vec + (long long)ii * mr + c;
       const bool in = ii >= 0 && ii < sd.N && c < r;
-      uint32_t d[4][S];
+      uint32_t d[4][S], mg[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int kk = k + (u & 1) + 8 * (u >> 1);
         const double val = in && kk < m ? xp[(long long)kk * r] : 0.0;
         digits<S>((unsigned long long)__double_as_longlong(val), fcol[q][c], d[u]);
+        mg[u] = magnitude((unsigned long long)__double_as_longlong(val), fcol[q][c]);
       }
 #pragma unroll
       for (int t = 0; t < S; ++t)
-        xd[q * xw + ((ks * S + t) * NT + nt) * 32 + ln] = make_uint2(pack_hi(d[0][t], d[1][t]), pack_hi(d[2][t], d[3][t]));
+        xd[q * xw + ((ks * SX + t) * NT + nt) * 32 + ln] = make_uint2(pack_hi(d[0][t], d[1][t]), pack_hi(d[2][t], d[3][t]));
+      xd[q * xw + ((ks * SX + S) * NT + nt) * 32 + ln] = make_uint2(pack_hi(mg[0], mg[1]), pack_hi(mg[2], mg[3]));
     }
     __syncthreads();
     if (!active || (part == 0 && i == 0) || (part == 2 && i == sd.N - 1)) continue;
@@ -231,9 +279,9 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[d][nt][q] = 0.f;
     if (v2)
-      tile_products<NT, true>(L, m, r0, tg, er, xd + sub * xw, lane, acc);
+      tile_products<NT, true>(L, m, r0, tg, er, xd + sub * xw, lane, acc, sum);
     else
-      tile_products<NT, false>(L, m, r0, tg, er, xd + sub * xw, lane, acc);
+      tile_products<NT, false>(L, m, r0, tg, er, xd + sub * xw, lane, acc, sum);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -250,6 +298,29 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
   if (active) {
     const double* bi = b + sd.vec + (long long)i * mr;
     double* ri = rout + sd.vec + (long long)i * mr;
+    double val[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int row = r0 + 8 * (q >> 1), c = 8 * nt + 2 * tg + (q & 1);
+        const int s = er[q >> 1] + fcol[sub][c] - 54;
+        bool odd = false;
+        double v = round_scaled(T[nt][q], s, odd);
+        if (odd) v = ldexp((double)T[nt][q], s);
+        if ((nan >> (4 * nt + q)) & 1u) v = __longlong_as_double(0x7ff8000000000000ll);
+        // a sum of 0: no term above 2^-126 of the scales
+        uint32_t left = __ballot_sync(0xffffffffu, row < m && c < r && sum[nt][q] != 0.f && !(sum[nt][q] >= kCertified));
+        while (left) {
+          const int src = __ffs(left) - 1;
+          left &= left - 1;
+          const int lrow = r0 - g + (src >> 2) + 8 * (q >> 1), lc = 8 * nt + 2 * (src & 3) + (q & 1);
+          const double w = float64_entry(A, B, C, o + (long long)lrow * m, x + sd.vec + (long long)i * mr + lc, mr, m, r,
+                                         i > 0, i < sd.N - 1, lane);
+          if (lane == src) v = w;
+        }
+        val[nt][q] = v;
+      }
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -260,13 +331,8 @@ __global__ void __launch_bounds__(kThreads, NT == 1 ? 2 : 1)
         for (int h = 0; h < 2; ++h) {
           const int row = r0 + 8 * h, q = 2 * h + cc;
           if (row < m && c < r) {
-            const int s = er[h] + fcol[sub][c] - 54;
-            bool odd = false;
-            double v = round_scaled(T[nt][q], s, odd);
-            if (odd) v = ldexp((double)T[nt][q], s);
-            if ((nan >> (4 * nt + q)) & 1u) v = __longlong_as_double(0x7ff8000000000000ll);
             const long long e = (long long)row * r + c;
-            const double bb = bi[e], rv = bb - v;
+            const double bb = bi[e], rv = bb - val[nt][q];
             ri[e] = rv;
             sr = fma(rv, rv, sr);
             sb = fma(bb, bb, sb);
@@ -319,7 +385,7 @@ void launch_residual_sliced(const SysDesc* sys, int nsys, const int (&ctas)[2], 
                             const double* C, const double* x, const double* b, double* r, double* nrm,
                             const unsigned* rowhi, const unsigned* colhi, cudaStream_t st) {
   // the group's block rows have at most 16 kWarps = 128 point rows together
-  constexpr int smem1 = resid::kWarps * resid::S * 32 * (int)sizeof(uint2);
+  constexpr int smem1 = resid::kWarps * resid::SX * 32 * (int)sizeof(uint2);
   if (ctas[0] > 0)
     resid::k_residual_digits<1><<<ctas[0], resid::kThreads, smem1, st>>>(sys, nsys, A, B, C, x, b, r, nrm, rowhi, colhi);
   if (ctas[1] > 0)

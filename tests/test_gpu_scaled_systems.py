@@ -128,3 +128,25 @@ def test_blocks_outside_the_system_are_not_read(dm, which):  # noqa: F811
         C[-1] = np.nan
     x = solution(dm, dm.dm_plan(12, 40, 1, 3, 1, "fp64"), A, s.B, C, s.b)
     assert o.rel_err(x, o.dm(s.A, s.B, s.C, s.b, 3)) <= 1e-12
+
+
+@pytest.mark.parametrize("m,r,N", [(64, 2, 40), (128, 1, 40), (88, 3, 33), (16, 8, 64), (128, 8, 12)])
+def test_refinement_of_scaled_unknowns(dm, m, r, N):  # noqa: F811
+    """Refined plans, default residual: unknowns over eight decades to the mixed path's 1e-10 of the largest, each in
+    its scale, in as many iterations as with the float64 residual (give or take one)."""
+    s = w.dominant_system(N, m, r, m)
+    A, B, C, b, q = scaled(s, m, 0, 27)
+    ref = o.thomas(s.A, s.B, s.C, s.b)
+    iters = []
+    for mode in ("auto", "fp64"):
+        plan = dm.dm_plan(N, m, r, 3, 1, "fp32")
+        try:
+            dm.dm_set_residual(plan, mode)
+            dm.dm_factor(plan, A, B, C)
+            x = np.zeros_like(b)
+            dm.dm_solve(plan, b, x)
+            iters.append(dm.dm_plan_query(plan)["last_iters"])
+        finally:
+            dm.dm_destroy(plan)
+        assert np.max(np.abs(x * q - ref)) <= 1e-10 * np.max(np.abs(ref)), mode
+    assert abs(iters[0] - iters[1]) <= 1
