@@ -602,12 +602,7 @@ void launch_gj_panel(const PartDesc* parts, int nparts, int t, int m, int pnl, d
   const size_t smem = gj::smem_bytes((m + 15) / 16);
 #define DM_GJ(C_, R_)                                                                                                   \
   do {                                                                                                              \
-    static bool set = false;                                                                                        \
-    if (!set) {                                                                                                     \
-      cudaFuncSetAttribute(gj::k_gj_panel<C_, R_>, cudaFuncAttributeMaxDynamicSharedMemorySize,                         \
-                           (int)gj::smem_bytes(2 * C_ * R_));                                                \
-      set = true;                                                                                                   \
-    }                                                                                                               \
+    allow_smem(gj::k_gj_panel<C_, R_>, smem);                                                                       \
     gj::k_gj_panel<C_, R_><<<nparts, 32 * (C_ + gj::kHelpers + 1), smem, st>>>(                                     \
         parts, t, m, pnl, W, piv, static_cast<__nv_bfloat16*>(Us), Uexp, static_cast<__nv_bfloat16*>(Vs), Vexp,     \
         status);                                                                                                    \

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "dm_grants.h"
+
 namespace dm {
 
 constexpr int kMaxM = 512;
@@ -57,6 +59,27 @@ __device__ __forceinline__ int find_sys(const SysDesc* __restrict__ sys, int nsy
     if (sys[mid].row0 <= row) lo = mid; else hi = mid - 1;
   }
   return lo;
+}
+
+// Raise a kernel's dynamic shared memory limit on the current device once (to
+// the largest size asked for so far), so that launches inside a stream capture
+// make no attribute calls; `carveout` also prefers the largest shared memory.
+inline Grants& smem_grants() {
+  static Grants g;
+  return g;
+}
+template <typename K>
+void allow_smem(K kernel, size_t bytes, bool carveout = false) {
+  // the default limit (48 KB) covers static + dynamic shared memory together;
+  // no kernel has more than 16 KB of static
+  if (bytes + 16 * 1024 <= 48 * 1024 && !carveout) return;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  smem_grants().ensure(dev, reinterpret_cast<const void*>(kernel), bytes, [&] {
+    if (carveout)
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+  });
 }
 
 // ---- launchers (dm_kernels.cu); T = double or float (factor storage type)

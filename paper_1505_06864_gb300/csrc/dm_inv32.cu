@@ -232,19 +232,12 @@ void launch_inv_f32(const PartDesc* parts, int nparts, int t, const double* B, f
                     cudaStream_t st) {
   if (nparts <= 0) return;
   const size_t smem = (size_t)max_m * (max_m | 1) * sizeof(float);
-#define DM_INV32(R_, CAP_)                                                                                         \
-  do {                                                                                                             \
-    static bool set = false;                                                                                       \
-    if (!set) {                                                                                                    \
-      cudaFuncSetAttribute(inv32::k_inv_f32<R_>, cudaFuncAttributeMaxDynamicSharedMemorySize,                      \
-                           CAP_ * (CAP_ | 1) * (int)sizeof(float));                                                \
-      set = true;                                                                                                  \
-    }                                                                                                              \
-    inv32::k_inv_f32<R_><<<nparts, inv32::kThreads, smem, st>>>(parts, t, B, G, status);                           \
-  } while (0)
-  if (max_m <= 128) DM_INV32(1, 128);
-  else DM_INV32(2, 224);
-#undef DM_INV32
+  auto go = [&](auto kernel) {
+    allow_smem(kernel, smem);
+    kernel<<<nparts, inv32::kThreads, smem, st>>>(parts, t, B, G, status);
+  };
+  if (max_m <= 128) go(inv32::k_inv_f32<1>);
+  else go(inv32::k_inv_f32<2>);
 }
 
 }  // namespace dm

@@ -1777,25 +1777,6 @@ __global__ void __launch_bounds__(256) k_axpy_norms(const SysDesc* __restrict__ 
   }
 }
 
-// Raise a kernel's dynamic shared memory limit once per kernel (to the
-// largest size asked for so far), so that launches inside a stream capture
-// make no attribute calls.
-std::mutex g_smem_mu;
-std::unordered_map<const void*, size_t> g_smem_granted;
-
-template <typename K>
-void allow_smem(K kernel, size_t bytes) {
-  // the default limit (48 KB) covers static + dynamic shared memory together
-  if (bytes + 4096 <= 48 * 1024) return;
-  const void* key = reinterpret_cast<const void*>(kernel);
-  std::lock_guard<std::mutex> lk(g_smem_mu);
-  size_t& g = g_smem_granted[key];
-  if (bytes > g) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    g = bytes;
-  }
-}
-
 template <typename T>
 int inv_smem_max_m() {
   // working matrix (m x (m+1)) + perm/idx/colk/rowk, within 227 KB
@@ -1841,12 +1822,14 @@ int inv_cluster_size(int max_m) {
 }
 
 // Whether a cluster of cs CTAs of `kernel` with `bytes` of shared memory each
-// can run (cached per kernel, size and bytes).
+// can run (cached per device, kernel, size and bytes).
 template <typename K>
 bool cluster_ok(K kernel, int cs, size_t bytes, int threads = 256) {
   static std::mutex mu;
-  static std::map<std::tuple<const void*, int, size_t>, bool> known;
-  const auto key = std::make_tuple(reinterpret_cast<const void*>(kernel), cs, bytes);
+  static std::map<std::tuple<int, const void*, int, size_t>, bool> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const auto key = std::make_tuple(dev, reinterpret_cast<const void*>(kernel), cs, bytes);
   std::lock_guard<std::mutex> lk(mu);
   auto it = known.find(key);
   if (it != known.end()) return it->second;

@@ -1135,12 +1135,8 @@ void launch_oz_step(int kind, const PartDesc* parts, int nparts, int step, int m
   const int grid = std::min(ntiles, nsm);
 #define DM_OZ(KIND_, S_)                                                                                          \
   do {                                                                                                            \
-    static bool set = false;                                                                                      \
     constexpr int smem = oz::smem_bytes<KIND_, S_>();                                                             \
-    if (!set) {                                                                                                   \
-      cudaFuncSetAttribute(oz::k_oz_step<KIND_, S_>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);          \
-      set = true;                                                                                                 \
-    }                                                                                                             \
+    allow_smem(oz::k_oz_step<KIND_, S_>, smem);                                                                   \
     oz::k_oz_step<KIND_, S_><<<grid, oz::threads_of(KIND_, S_), smem, st>>>(parts, step, aux, m, ntm, ntn, ntiles, out, lexp,  \
                                                                rexp0, rexp1, errflag, mp);                        \
   } while (0)
@@ -1188,12 +1184,7 @@ void launch_oz_assemble(const SepDesc* seps, int nseps, int m, const double* B, 
 void launch_band_gc(const PartDesc* parts, int nparts, int t, int m, const double* G, const double* C, double* Acal,
                     double* ZR, const int* band, cudaStream_t st) {
   if (nparts <= 0 || !band) return;
-  static bool set = false;
-  if (!set) {
-    cudaFuncSetAttribute(oz::k_band_gc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (2 * kBandMax + 1) * kMaxM * (int)sizeof(double));
-    set = true;
-  }
+  allow_smem(oz::k_band_gc, (2 * kBandMax + 1) * m * sizeof(double));
   oz::k_band_gc<<<nparts * ((m + 31) / 32), 256, (2 * kBandMax + 1) * m * sizeof(double), st>>>(parts, t, m, G, C, Acal, ZR, band);
 }
 

@@ -237,11 +237,7 @@ void launch_small_factor(const PartDesc* parts, int nparts, const double* A, con
                          double* Acal, double* ZL, double* ZR, int* status, const int* band, cudaStream_t st) {
   if (nparts <= 0) return;
   constexpr int smem = small::kBlocks * small::BLK * (int)sizeof(double);
-  static bool set = false;
-  if (!set) {
-    cudaFuncSetAttribute(small::k_small_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    set = true;
-  }
+  allow_smem(small::k_small_factor, smem);
   small::k_small_factor<<<nparts, small::kThreads, smem, st>>>(parts, A, B, C, G, Acal, ZL, ZR, status,
                                                                   band);
 }

@@ -705,19 +705,8 @@ __global__ void __launch_bounds__(kThreads) k_mma_probe(int iters, int* __restri
 
 // ---------------------------------------------------------------- launchers
 namespace {
-template <typename K>
-void raise_smem_once(K kernel, int bytes, bool* done) {
-  if (!*done) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    // the largest shared-memory carve-out, so that launches sized below the
-    // maximum fit several CTAs per SM
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    *done = true;
-  }
-}
-bool g_set_fwd[2], g_set_back[2];
-
-// Shared memory of one launch: the left buffers for its M-tiles and the right
+// Shared memory of one launch (the largest carve-out is preferred, so that
+// launches sized below the maximum fit several CTAs per SM): the left buffers for its M-tiles and the right
 // panel for its K-slabs (blocks up to max_m), so that blocks of m <= 128 fit
 // two CTAs per SM.
 template <int MODE>
@@ -742,12 +731,12 @@ void launch_fwd_factor_tc(int mode, const PartDesc* parts, int nparts, int t, in
   int cap = 0;
   if (mode == 0) {
     const int bytes = tc_launch_smem<0>(max_m, &cap);
-    raise_smem_once(tc::k_fwd_factor_tc<0>, tc::Smem<0>::total, &g_set_fwd[0]);
+    allow_smem(tc::k_fwd_factor_tc<0>, tc::Smem<0>::total, true);
     tc::k_fwd_factor_tc<0><<<grid, tc::kThreads, bytes, st>>>(parts, t, tiles_n, type_lo, A, B, C, G, Acal, ZL, ZR,
                                                               errflag, tm, use_tma, cap);
   } else {
     const int bytes = tc_launch_smem<1>(max_m, &cap);
-    raise_smem_once(tc::k_fwd_factor_tc<1>, tc::Smem<1>::total, &g_set_fwd[1]);
+    allow_smem(tc::k_fwd_factor_tc<1>, tc::Smem<1>::total, true);
     tc::k_fwd_factor_tc<1><<<grid, tc::kThreads, bytes, st>>>(parts, t, tiles_n, type_lo, A, B, C, G, Acal, ZL, ZR,
                                                               errflag, tm, 0, cap);
   }
@@ -765,12 +754,12 @@ void launch_back_factor_tc(int mode, const PartDesc* parts, int nparts, int s, i
   int cap = 0;
   if (mode == 0) {
     const int bytes = tc_launch_smem<0>(max_m, &cap);
-    raise_smem_once(tc::k_back_factor_tc<0>, tc::Smem<0>::total, &g_set_back[0]);
+    allow_smem(tc::k_back_factor_tc<0>, tc::Smem<0>::total, true);
     tc::k_back_factor_tc<0><<<grid, tc::kThreads, bytes, st>>>(parts, s, tiles_n, Acal, ZL, ZR, errflag, tm, use_tma,
                                                                cap);
   } else {
     const int bytes = tc_launch_smem<1>(max_m, &cap);
-    raise_smem_once(tc::k_back_factor_tc<1>, tc::Smem<1>::total, &g_set_back[1]);
+    allow_smem(tc::k_back_factor_tc<1>, tc::Smem<1>::total, true);
     tc::k_back_factor_tc<1><<<grid, tc::kThreads, bytes, st>>>(parts, s, tiles_n, Acal, ZL, ZR, errflag, tm, 0, cap);
   }
 }
@@ -840,10 +829,10 @@ double launch_mma_probe(int mode, int iters, int* errflag, cudaStream_t st) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int smem = 116 * 1024;
   if (mode == 0) {
-    cudaFuncSetAttribute(tc::k_mma_probe<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    allow_smem(tc::k_mma_probe<0>, smem);
     tc::k_mma_probe<0><<<sms, tc::kThreads, smem, st>>>(iters, errflag);
   } else {
-    cudaFuncSetAttribute(tc::k_mma_probe<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    allow_smem(tc::k_mma_probe<1>, smem);
     tc::k_mma_probe<1><<<sms, tc::kThreads, smem, st>>>(iters, errflag);
   }
   const double k_per_instr = mode == 0 ? 8.0 : 16.0;

@@ -434,11 +434,6 @@ EncodeFn encoder() {
   return enc;
 }
 
-template <typename K>
-void raise_smem(K kernel, int bytes) {
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-}
 }  // namespace
 
 bool tc2_eligible(int m) { return m >= 8 && m <= 256 && m % 8 == 0; }
@@ -501,11 +496,7 @@ void launch_tc2_step(int mode, int kind, const PartDesc* parts, int nparts, int 
   const int nt = tc2_ntile(m);
 #define DM_STEP(MODE_, KIND_)                                                                                     \
   do {                                                                                                            \
-    static bool set = false;                                                                                      \
-    if (!set) {                                                                                                   \
-      raise_smem(tc2::k_tc_step<MODE_, KIND_>, tc2::Cfg<MODE_>::smem);                                           \
-      set = true;                                                                                                 \
-    }                                                                                                             \
+    allow_smem(tc2::k_tc_step<MODE_, KIND_>, tc2::Cfg<MODE_>::smem, true);                                        \
     tc2::k_tc_step<MODE_, KIND_><<<grid, tc2::kThreads, tc2::Cfg<MODE_>::smem, st>>>(parts, step, m, nt, lo[0],   \
                                                                                     lo[1], lo[2], out, errflag, mp); \
   } while (0)
