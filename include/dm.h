@@ -133,7 +133,7 @@ int dm_plan(dm_plan_t* out, int N, int m, int nrhs, int P, int levels, int preci
  * equations and unknowns of less than 2^13 is not told from an ordinary
  * block and can cost 40 times the float64 products' error (7e-14).
  * DM_PLAN_FP64_FMA keeps the products on the float64 pipe; so does a plan with
- * m % 8 != 0 or m > 256 whose slices (about as much again as its factors) do
+ * m % 8 != 0 or m > 256 whose slices (about as much again as its float64 factors) do
  * not fit the device memory free at dm_plan (several times slower, and in
  * other roundings). */
 #define DM_PLAN_FP64_FMA 2

@@ -1231,9 +1231,10 @@ int Plan::init(const std::vector<SysSpec>& specs, int prec) {
     };
     size_t need = footprint();
     const size_t reserve = std::min<size_t>(total_b / 64, size_t(1) << 30);
-    if (need + reserve > free_b && !top.f32 && !top.fp64_fma && (top.max_m % 8 != 0 || top.max_m > kMaxMTensor)) {
-      // the digit slices about double a float64 plan's footprint: block sizes
-      // that have the float64 pipe's kernels as an equal in kind keep fitting
+    if (need + reserve > free_b && !top.fp64_fma && (top.max_m % 8 != 0 || top.max_m > kMaxMTensor)) {
+      // the digit slices about double the footprint of a float64 plan and of the
+      // supplementary levels of the others: block sizes that have the float64
+      // pipe's kernels as an equal in kind keep fitting
       top.fp64_fma = true;
       if ((rc = top.build(specs, prec != DM_FP64, tmode))) return rc;
       need = footprint();
