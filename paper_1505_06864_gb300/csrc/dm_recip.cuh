@@ -6,8 +6,9 @@
 
 namespace dm {
 
-// zero, below 2^-1022 (whose reciprocal overflows), at or above 2^1022
-// (whose reciprocal is not a normal number) or not finite
+// not for pivot_recip: zero, below 2^-1022 (whose reciprocal overflows or is
+// near it), at or above 2^1022 (whose reciprocal is not a normal number) or not
+// finite
 __device__ __forceinline__ bool pivot_unusable(double v) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
   return b < 0x0010000000000000ull || b >= 0x7fd0000000000000ull;
@@ -38,6 +39,12 @@ __device__ __forceinline__ double pivot_recip(double x) {
   const unsigned long long mant = (y + 64) >> 7;  // leading bit at 52, or 2^53
   return __longlong_as_double((long long)((bits & 0x8000000000000000ull) +
                                           ((unsigned long long)(2044 - ex) << 52) + mant));
+}
+
+// The same for every pivot that has a finite reciprocal, 0 for the others.
+static __device__ __noinline__ double pivot_recip_any(double x) {
+  const double r = 1.0 / x;
+  return fabs(x) > 0.0 && isfinite(x) && isfinite(r) ? r : 0.0;
 }
 
 __device__ __forceinline__ uint32_t abs_hi(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }

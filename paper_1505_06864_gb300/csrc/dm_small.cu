@@ -64,9 +64,11 @@ __device__ __forceinline__ void invert(const double* D, double* G, int m, Shared
     const uint32_t key = dead ? 0u : abs_hi(v) + 1u;
     const uint32_t kmax = __reduce_max_sync(0xffffffffu, key);
     const int src = (int)__reduce_min_sync(0xffffffffu, key == kmax ? (uint32_t)lane : 32u);
-    const double inv = pivot_unusable(v) ? 0.0 : pivot_recip(v);
+    double inv = pivot_unusable(v) ? 0.0 : pivot_recip(v);
     sh.f[j & 1][lane] = v;
     if (lane == src) {
+      // near the ends of the range the division (the blocks are not equilibrated here)
+      if (__double_as_longlong(inv) == 0) inv = pivot_recip_any(v);
       sh.pv[j & 1] = Pivot{inv, lane, 0};
       sh.order[j] = lane;
       if (__double_as_longlong(inv) == 0) bad = true;
