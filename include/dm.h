@@ -138,9 +138,10 @@ int dm_plan(dm_plan_t* out, int N, int m, int nrhs, int P, int levels, int preci
  * other roundings). */
 #define DM_PLAN_FP64_FMA 2
 /* The float64 block inverse of those levels is by default blocked
- * Gauss-Jordan (panels of 32 columns in float64, their rank-32 trailing
- * updates as digit-sliced tensor-core products); DM_PLAN_FP64_INV_COLUMN
- * takes the column-by-column Gauss-Jordan kernel instead (same pivoting). */
+ * Gauss-Jordan of the equilibrated block (panels of 32 columns, eight at a
+ * time in float64, all other updates as digit-sliced tensor-core products;
+ * pivot candidates that agree to 2^-20 count as equal); DM_PLAN_FP64_INV_COLUMN
+ * takes the column-by-column Gauss-Jordan kernel on the block as it is. */
 #define DM_PLAN_FP64_INV_COLUMN 4
 int dm_plan_ex(dm_plan_t* out, int N, int m, int nrhs, int P, int levels, int precision, int flags);
 

@@ -409,8 +409,8 @@ __device__ __noinline__ void gj_slice8(double v0, double v1, double v2, double v
 // One panel of every active subsystem's working matrix, a CTA per block: up to
 // eight chain warps (a row per lane; two rows above m = 256), the control
 // warp, and eight helpers.  Bound by the chain's float64 instructions and
-// barriers: about 1150 cycles per pivot to m = 128 (one warp per SM
-// sub-partition) and 1800 at m = 256 (two), half of the kernel's time; the updates that the
+// barriers: about 1150 cycles per pivot at m = 64, 1290 at 128 (one warp per SM
+// sub-partition) and 1880 at m = 256 (two), half of the kernel's time; the updates that the
 // chain waits for take a sixth, the slices at the end an eighth.  A cluster of CTAs with the rows
 // split and a cluster barrier per pivot took 83 / 90 / 98 us per panel at m =
 // 64 / 128 / 256, this one with every warp making its own digits of U and V 40 / 48 / 74 us, and
