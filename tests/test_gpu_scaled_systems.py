@@ -150,3 +150,30 @@ def test_refinement_of_scaled_unknowns(dm, m, r, N):  # noqa: F811
             dm.dm_destroy(plan)
         assert np.max(np.abs(x * q - ref)) <= 1e-10 * np.max(np.abs(ref)), mode
     assert abs(iters[0] - iters[1]) <= 1
+
+
+def test_neighbours_in_a_batch_do_not_share_scales(dm):  # noqa: F811
+    """Three systems of one block size in one level, each in units of its own, their outer blocks NaN: each comes out
+    as it does alone."""
+    m = 40
+    systems = [w.dominant_system(n, m, 1, 60 + n) for n in (12, 9, 15)]
+    parts = []
+    for k, s in enumerate(systems):
+        f = 2.0 ** (-300 * k)
+        A, C = s.A * f, s.C * f
+        A[0], C[-1] = np.nan, np.nan
+        parts.append((A, s.B * f, C, s.b * f))
+    plan = dm.dm_plan_batch([s.N for s in systems], [m] * 3, [1] * 3, "fp64")
+    try:
+        cat = [np.concatenate([p[i].ravel() for p in parts]) for i in range(4)]
+        dm.dm_factor(plan, *cat[:3])
+        assert panels(dm, plan, *cat[:3]) > 0
+        x = np.zeros_like(cat[3])
+        dm.dm_solve(plan, cat[3], x, count=3)
+    finally:
+        dm.dm_destroy(plan)
+    at = 0
+    for s in systems:
+        xs = x[at:at + s.b.size].reshape(s.b.shape)
+        at += s.b.size
+        assert o.rel_err(xs, o.thomas(s.A, s.B, s.C, s.b)) <= 1e-12
